@@ -129,15 +129,16 @@ def _spectrum(dtype, d, k):
     if d >= 1536:
         j1, j2 = np.arange(1, k + 1), np.arange(k + 1, 4 * k + 1)
         return np.concatenate([j1 ** -1.5, 0.5 * j2 ** -1.5]), math.sqrt(1e-3)
-    return 0.85 ** np.arange(1, d + 1), 0.0
+    # 0.85^j; what lies beyond 96 spikes (1e-7 of the first) is below the stored rows' rounding
+    return 0.85 ** np.arange(1, min(d, 96) + 1), 0.0
 
 
 def _rows(n, d, lam, sigma, seed):
     """n x d FP32 spiked-Gaussian rows on the GPU."""
     g = torch.Generator(device=DEV).manual_seed(int(seed))
     q = len(lam)
-    U = torch.linalg.qr(torch.randn(d, q, device=DEV, generator=g))[0]
-    basis = (U * torch.tensor(lam, device=DEV, dtype=torch.float32).sqrt()).T.contiguous()
+    U = torch.linalg.qr(_gauss((d, q), seed + 5).float())[0]
+    basis = (U.to(DEV) * torch.tensor(lam, device=DEV, dtype=torch.float32).sqrt()).T.contiguous()
     out = torch.empty(n, d, device=DEV)
     for r in range(0, n, 131_072):
         e = min(n, r + 131_072)
@@ -320,8 +321,8 @@ def _orth64(Y):
     """Orthonormal basis with positive diagonal of R, blocks d x k: two passes of Gram and Cholesky in FP64
     (the second removes what the conditioning of the first leaves), equal to a Householder QR with that sign."""
     for _ in range(2):
-        L = torch.linalg.cholesky(Y.mT @ Y)
-        Y = torch.linalg.solve_triangular(L.mT, Y, upper=True, left=False)
+        L = torch.linalg.cholesky((Y.mT @ Y).cpu())
+        Y = Y @ torch.linalg.inv(L).mT.to(DEV)
     return Y
 
 
@@ -355,17 +356,16 @@ def _solve64(parts, scales, dtype, k, schedule, refine, agg, y0, ritz):
             dots = (Zi * Zi[base]).sum(dim=1)
             Yi = Yi * torch.where(dots < 0, -1.0, 1.0).to(torch.float64)[:, None, :]
         elif p > 1 and agg == "opt":
-            C = Zi.mT @ Zi[base]
-            W1, _, W2 = torch.linalg.svd(C)
+            W1, _, W2 = torch.linalg.svd((Zi.mT @ Zi[base]).cpu())
             D = W1 @ W2
-            D[base] = torch.eye(k, dtype=torch.float64, device=DEV)
-            Yi = Yi @ D
+            D[base] = torch.eye(k, dtype=torch.float64)
+            Yi = Yi @ D.to(DEV)
         Z = _orth64((w * Yi).sum(dim=0))
     if not ritz:
         return Z.cpu().numpy(), None
     H = Z.T @ (w * op.step(Z.expand(m, -1, -1))).sum(dim=0)
-    lam, V = torch.linalg.eigh((H + H.T) / 2)
-    lam, V = lam.flip(0), V.flip(1)
+    lam, V = torch.linalg.eigh(((H + H.T) / 2).cpu())
+    lam, V = lam.flip(0).to(DEV), V.flip(1).to(DEV)
     # a Ritz vector's sign: along the column of Z_T that it has most of
     V = V * torch.sign(V.gather(0, V.abs().argmax(dim=0, keepdim=True)))
     return (Z @ V).cpu().numpy(), (n * lam.clamp(min=0)).sqrt().cpu().numpy()
