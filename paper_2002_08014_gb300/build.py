@@ -19,7 +19,7 @@ OUT_DIR = os.path.join(PKG, "_build")
 LIB_NAME = "liblocalpower.so"
 LIB_PATH = os.path.join(OUT_DIR, LIB_NAME)
 
-SOURCES = ["lp_capi.cu", "lp_server.cu", "step_simt.cu", "step_tc.cu", "step_tcs.cu", "small_kernels.cu",
+SOURCES = ["lp_capi.cu", "lp_server.cu", "step_simt.cu", "step_tc.cu", "step_tcs.cu", "small_kernels.cu", "cholqr2.cu",
            "step_static.cu", "eta.cu", "step_simt_tmem.cu",
            "step_pair.cu", "step_tcs8.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -1,18 +1,16 @@
 // The d x k and k x k kernels around the fused power step:
 //   reduce     Y_i = (1/s_i) sum of the step kernel's per-CTA partials (fixed order)
-//   cholqr2    Z = orth(Y) by two passes of Gram / Cholesky / triangular solve
 //   align      sign-fixing (eq. (4)) or orthogonal Procrustes (eq. (3)) matrices
 //   aggregate  Y = sum_i p_i Y_i D_i (Alg. 1 aggregation)
 //   ritz       Rayleigh-Ritz on span(Z): ordered basis and sigma_j = sqrt(n lambda_j)
 //   split      FP32 rows -> hi / lo BF16 planes (load time)
 //   rho        residual error of Def. 3 per partition (traced solves)
-// Precision, by default: the d-sized work (Gram, solves, averaging) and the k x k
-// Jacobi SVD / eigen-solves are FP32; the Cholesky factor is FP32 when its pivots
-// allow (else FP64); the Ritz matrix H and the sign-fix inner products that
+// (the orthonormalisation is in cholqr2.cu).
+// Precision, by default: the d-sized work (averaging) and the k x k Jacobi SVD /
+// eigen-solves are FP32; the Ritz matrix H and the sign-fix inner products that
 // decide D_i are accumulated in FP64.  GB300's FP64 pipe is a small fraction of
 // its FP32 pipe, and these k x k steps are serial latency on every round.  With
-// LP_FLAG_KXK_FP64 the k x k work is FP64 throughout: the CholQR2 Gram (summed in
-// FP64) and its Cholesky, the Procrustes SVD and the Ritz eigen-solve.
+// LP_FLAG_KXK_FP64 the Procrustes SVD and the Ritz eigen-solve are FP64 too.
 #include <algorithm>
 #include <cfloat>
 #include <mutex>
@@ -26,21 +24,6 @@ namespace lp {
 namespace {
 
 constexpr int kT = 256;
-
-// FP64 1/sqrt(x) by Newton-Raphson iteration from an FP32 seed
-// (y <- y (3 - x y^2) / 2); each step doubles the number of correct bits, so two
-// steps take the FP32 seed (about 2^-22) past FP64 precision.  An FP64 square
-// root is a long instruction sequence on this GPU; this is a few FMAs on the
-// FP64 Cholesky's critical path.  Arguments outside the FP32 normal range take
-// the plain sqrt.
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  if (!(x > 1e-30 && x < 1e30)) return 1.0 / sqrt(x);
-  double y = static_cast<double>(rsqrtf(static_cast<float>(x)));
-  const double hx = 0.5 * x;
-  y = y * (1.5 - hx * y * y);
-  y = y * (1.5 - hx * y * y);
-  return y;
-}
 
 // ---------------------------------------------------------------- pack / unpack
 // FP32 rows -> two BF16 planes: hi = RNE(a), lo = RNE(a - hi).  a - hi is exact
@@ -249,360 +232,6 @@ __device__ void procrustes_factor(T* C, const T* V, T* inv, int k, int K, float*
     Gi[e] = static_cast<float>(sum);
   }
 }
-
-// ---------------------------------------------------------------- CholQR2
-// One CTA per block, two passes of:
-//   G = Y^T Y        FP32 products and partial sums over row slices, combined in FP32
-//   G = L L^T        right-looking Cholesky on warp 0: FP32, or FP64 when an FP32
-//                    pivot is too small to trust
-//   Z = Y L^{-T}     per-row forward substitution in FP32, one thread per row
-// The column space is Y's whatever the precision of L; the second pass restores
-// orthonormality lost to the FP32 Gram.  A pivot that is not positive and finite
-// sets ST_CHOL (the pivot is then taken as 1 so the kernel can finish).
-// G = Y^T Y: thread (block (bi, bj) of 4 x 4 entries, row slice) accumulates
-// Y[r][4bi..4bi+3]^T Y[r][4bj..4bj+3] over its rows in FP32 registers (16 FMAs
-// per two 16-byte loads); the slices are added in FP32 through shared memory.
-template <int K>
-__device__ void gram_fp32(const float* Y, int d, float* red, double* G) {
-  constexpr int NB = K / 4, NBB = NB * NB, S = kT / NBB;
-  const int t = threadIdx.x;
-  const int blk = t % NBB, sl = t / NBB;
-  const int bi = blk / NB, bj = blk % NB;
-  float acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-  // eight rows per trip, all loads issued before the FMAs: one block reads the
-  // whole d x K block with ~16 loads in flight per thread instead of one
-  constexpr int U = 8;
-  for (int r0 = sl; r0 < d; r0 += S * U) {
-    float4 u[U], v[U];
-#pragma unroll
-    for (int q = 0; q < U; ++q) {
-      const int r = r0 + q * S;
-      u[q] = r < d ? *reinterpret_cast<const float4*>(Y + int64_t(r) * K + 4 * bi) : make_float4(0.f, 0.f, 0.f, 0.f);
-      v[q] = r < d ? *reinterpret_cast<const float4*>(Y + int64_t(r) * K + 4 * bj) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-#pragma unroll
-    for (int q = 0; q < U; ++q) {
-      const float uu[4] = {u[q].x, u[q].y, u[q].z, u[q].w}, vv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(uu[a], vv[b], acc[a][b]);
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) red[(sl * NBB + blk) * 16 + 4 * a + b] = acc[a][b];
-  __syncthreads();
-  for (int e = t; e < K * K; e += kT) {
-    const int i = e / K, j = e % K;
-    const int bb = (i / 4) * NB + j / 4, el = 4 * (i % 4) + j % 4;
-    // four interleaved FP32 partial sums in slice order, then pairwise: short
-    // dependency chains (the factorisation reads the Gram in FP32 first)
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    int q = 0;
-    for (; q + 4 <= S; q += 4) {
-      s0 += red[(q * NBB + bb) * 16 + el];
-      s1 += red[((q + 1) * NBB + bb) * 16 + el];
-      s2 += red[((q + 2) * NBB + bb) * 16 + el];
-      s3 += red[((q + 3) * NBB + bb) * 16 + el];
-    }
-    for (; q < S; ++q) s0 += red[(q * NBB + bb) * 16 + el];
-    G[e] = static_cast<double>((s0 + s1) + (s2 + s3));
-  }
-  __syncthreads();
-}
-
-// G = Y^T Y in FP64 (LP_FLAG_KXK_FP64): the upper triangle of 4 x 4 blocks, one
-// per thread of a row slice; each FP32 product is exact in FP64 (two 24-bit
-// significands need 48 of its 53 bits) and is summed in FP64 over the slice's
-// rows; the slices are added in slice order and the lower triangle mirrored.
-template <int K>
-__device__ void gram_fp64(const float* Y, int d, double* red, double* G) {
-  constexpr int NB = K / 4, NBU = NB * (NB + 1) / 2, S = kT / NBU;
-  const int t = threadIdx.x;
-  const int blk = t % NBU, sl = t / NBU;
-  int bi = 0, rem = blk;
-  while (rem >= NB - bi) {
-    rem -= NB - bi;
-    ++bi;
-  }
-  const int bj = bi + rem;
-  if (sl < S) {
-    double acc[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-    constexpr int U = 4;
-    for (int r0 = sl; r0 < d; r0 += S * U) {
-      float4 u[U], v[U];
-#pragma unroll
-      for (int q = 0; q < U; ++q) {
-        const int r = r0 + q * S;
-        u[q] = r < d ? *reinterpret_cast<const float4*>(Y + int64_t(r) * K + 4 * bi) : make_float4(0.f, 0.f, 0.f, 0.f);
-        v[q] = r < d ? *reinterpret_cast<const float4*>(Y + int64_t(r) * K + 4 * bj) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int q = 0; q < U; ++q) {
-        const double uu[4] = {u[q].x, u[q].y, u[q].z, u[q].w}, vv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) acc[a][b] = fma(uu[a], vv[b], acc[a][b]);
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) red[(sl * NBU + blk) * 16 + 4 * a + b] = acc[a][b];
-  }
-  __syncthreads();
-  for (int e = t; e < K * K; e += kT) {
-    const int i = e / K, j = e % K;
-    const int a = i < j ? i : j, b = i < j ? j : i;
-    const int ba = a / 4, bb = b / 4;
-    const int idx = ba * NB - ba * (ba - 1) / 2 + (bb - ba);
-    const int el = 4 * (a % 4) + b % 4;
-    double sum = 0.0;
-    for (int q = 0; q < S; ++q) sum += red[(q * NBU + idx) * 16 + el];
-    G[e] = sum;
-  }
-  __syncthreads();
-}
-
-// One-warp right-looking Cholesky with the matrix in registers: lane l holds
-// column l (rows 0..K-1) of the symmetric Gram; at pivot j lane j scales its
-// column into L[:, j], the other lanes receive L[i][j] from lane j by shuffles,
-// lane l keeps L[l][j] when i reaches l and updates its rows i >= l:
-// G[i][l] -= L[i][j] L[l][j].  Every entry of the lower triangle sees the same
-// operations in the same order as the textbook shared-memory form; the upper
-// rows of a column (i < l) are never read.  No index arithmetic by k in the
-// inner loops (the shared-memory form divided by the trailing size for every
-// entry, which dominated CholQR2 at K = 32).
-
-// FP64 factor of the FP64 Gram G (k x k, stride K; not modified).  Writes L in FP32
-// (lower, stride K) and 1 / L[j][j] in FP32; returns false on breakdown (a pivot
-// that is not positive and finite is then taken as 1 so the kernel can finish).
-template <int K>
-__device__ bool warp_cholesky_rl(const double* G, float* Lf, float* invd, int k) {
-  const int lane = threadIdx.x & 31;
-  double col[K];
-#pragma unroll
-  for (int i = 0; i < K; ++i) col[i] = (i < k && lane < k) ? G[i * K + lane] : 0.0;
-  bool ok = true;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    if (j >= k) continue;  // (not break: the loop stays unrolled, col[] in registers)
-    double piv = __shfl_sync(0xffffffffu, col[j], j);
-    if (!(piv > 0.0) || !isfinite(piv)) {
-      ok = false;
-      piv = 1.0;
-    }
-    const double inv = rsqrt_nr(piv);
-    const double ljj = piv * inv;
-    if (lane == j) {
-      col[j] = ljj;
-#pragma unroll
-      for (int i = j + 1; i < K; ++i) col[i] *= inv;
-      invd[j] = static_cast<float>(inv);
-    }
-    double my = 0.0;  // L[lane][j], known once i reaches lane
-#pragma unroll
-    for (int i = j + 1; i < K; ++i) {
-      const double lij = __shfl_sync(0xffffffffu, col[i], j);
-      if (i == lane) my = lij;
-      if (lane > j && i >= lane) col[i] -= lij * my;
-    }
-  }
-  if (lane < K) {
-#pragma unroll
-    for (int i = 0; i < K; ++i) Lf[i * K + lane] = (i < k && lane <= i) ? static_cast<float>(col[i]) : 0.f;
-  }
-  __syncwarp();
-  return ok;
-}
-
-// FP32 factor of the FP64 Gram (read in FP32) on one warp, written to Lf (lower,
-// stride K) and invd.  Returns false (G untouched, for warp_cholesky_rl) when a
-// pivot is not above 1e-6 of the largest diagonal entry or not finite: GB300's
-// FP64 pipe is a small fraction of its FP32 pipe, and the FP32 factor serves both
-// CholQR passes whenever the Gram allows it (the column space is that of Y for
-// any invertible factor; the second pass restores orthonormality).
-template <int K>
-__device__ bool warp_cholesky_f32(const double* G, float* Lf, float* invd, int k) {
-  const int lane = threadIdx.x & 31;
-  float col[K];
-#pragma unroll
-  for (int i = 0; i < K; ++i) col[i] = (i < k && lane < k) ? static_cast<float>(G[i * K + lane]) : 0.f;
-  float dmax = lane < k ? static_cast<float>(G[lane * K + lane]) : 0.f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-  if (!(dmax > 0.f) || !isfinite(dmax)) return false;
-  const float floor = 1e-6f * dmax;
-  bool good = true;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    if (j >= k || !good) continue;  // (not break / return: the loop stays unrolled, col[] in registers)
-    const float piv = __shfl_sync(0xffffffffu, col[j], j);
-    if (!(piv > floor) || !isfinite(piv)) {
-      good = false;
-      continue;
-    }
-    const float ljj = sqrtf(piv);
-    const float inv = 1.0f / ljj;
-    if (lane == j) {
-      col[j] = ljj;
-#pragma unroll
-      for (int i = j + 1; i < K; ++i) col[i] *= inv;
-      invd[j] = inv;
-    }
-    float my = 0.f;  // L[lane][j], known once i reaches lane
-#pragma unroll
-    for (int i = j + 1; i < K; ++i) {
-      const float lij = __shfl_sync(0xffffffffu, col[i], j);
-      if (i == lane) my = lij;
-      if (lane > j && i >= lane) col[i] -= lij * my;
-    }
-  }
-  if (!good) return false;
-  if (lane < K) {
-#pragma unroll
-    for (int i = 0; i < K; ++i) Lf[i * K + lane] = (i < k && lane <= i) ? col[i] : 0.f;
-  }
-  __syncwarp();
-  return true;
-}
-
-// Z[r][:] = Y[r][:] L^{-T}: z_j = (y_j - sum_{p<j} z_p L[j][p]) / L[j][j].  Each
-// thread solves four rows at once, column j outermost, so a row of L read from
-// shared memory serves four independent FMA chains.
-template <int K>
-__device__ void forward_rows(const float* Yin, float* Zout, const float* Lf, const float* invd, int d, int k) {
-  constexpr int RPT = 4;
-  for (int rb = 0; rb < d; rb += RPT * kT) {
-    asm volatile("" ::: "memory");  // keep the L reads inside this iteration
-    float y[RPT][K];
-#pragma unroll
-    for (int g = 0; g < RPT; ++g) {
-      const int r = rb + threadIdx.x + g * kT;
-#pragma unroll
-      for (int q = 0; q < K / 4; ++q) {
-        const float4 v = r < d ? reinterpret_cast<const float4*>(Yin + int64_t(r) * K)[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-        y[g][4 * q] = v.x; y[g][4 * q + 1] = v.y; y[g][4 * q + 2] = v.z; y[g][4 * q + 3] = v.w;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-      const float inv = j < k ? invd[j] : 0.f;
-#pragma unroll
-      for (int g = 0; g < RPT; ++g) {
-        float s = y[g][j];
-#pragma unroll
-        for (int p = 0; p < j; ++p) s = fmaf(-y[g][p], Lf[j * K + p], s);
-        y[g][j] = s * inv;
-      }
-    }
-#pragma unroll
-    for (int g = 0; g < RPT; ++g) {
-      const int r = rb + threadIdx.x + g * kT;
-      if (r < d) {
-        float4* dst = reinterpret_cast<float4*>(Zout + int64_t(r) * K);
-#pragma unroll
-        for (int q = 0; q < K / 4; ++q) dst[q] = make_float4(y[g][4 * q], y[g][4 * q + 1], y[g][4 * q + 2], y[g][4 * q + 3]);
-      }
-    }
-  }
-}
-
-// Z = orth(Y) of one d x K block by the CTA: the first pass writes Zmid from Y,
-// the second Zout from Zmid (Zmid may be Y itself: each thread solves its own
-// rows in place; or Zout).  Any of them may have been written earlier in the same
-// kernel.  F64: Gram and Cholesky in FP64 (LP_FLAG_KXK_FP64); else the FP32 Gram
-// and FP32 Cholesky with the FP64 factorisation as fallback.  The d x k forward
-// substitution is FP32 either way.
-template <int K, bool F64>
-__device__ void cholqr2_block(const float* Y, float* Zmid, float* Zout, int d, int k, int* status) {
-  __shared__ __align__(16) double G[K * K];
-  __shared__ __align__(16) float Lf[K * K];
-  __shared__ float invd[K];
-  __shared__ __align__(16) unsigned char red[(F64 ? 8 : 4) * kT * 16];
-  for (int pass = 0; pass < 2; ++pass) {
-    const float* src = pass == 0 ? Y : Zmid;
-    if (F64) {
-      gram_fp64<K>(src, d, reinterpret_cast<double*>(red), G);
-      if (threadIdx.x < 32) {
-        const bool ok = warp_cholesky_rl<K>(G, Lf, invd, k);
-        if (!ok && threadIdx.x == 0) atomicOr(status, ST_CHOL);
-      }
-    } else {
-      gram_fp32<K>(src, d, reinterpret_cast<float*>(red), G);
-      if (threadIdx.x < 32 && !warp_cholesky_f32<K>(G, Lf, invd, k)) {
-        const bool ok = warp_cholesky_rl<K>(G, Lf, invd, k);
-        if (!ok && threadIdx.x == 0) atomicOr(status, ST_CHOL);
-      }
-    }
-    __syncthreads();
-    forward_rows<K>(src, pass == 0 ? Zmid : Zout, Lf, invd, d, k);
-    __syncthreads();
-  }
-}
-
-// One CTA per block.  STAGED: the d x K block is copied into shared memory once
-// (eight 16-byte loads in flight per thread), both Grams and the first solve
-// work there (the first pass's Z overwrites Y in place) and only the second
-// pass writes global memory; otherwise each pass reads global memory (blocks
-// larger than kCholStageBytes).
-constexpr size_t kCholStageBytes = size_t(128) << 10;
-
-template <int K, bool F64, bool STAGED>
-__global__ void __launch_bounds__(kT) cholqr2_kernel(const float* __restrict__ Yall, float* __restrict__ Zall, int d,
-                                                     int k, int* status) {
-  const float* Y = Yall + int64_t(blockIdx.x) * d * K;
-  float* Z = Zall + int64_t(blockIdx.x) * d * K;
-  if constexpr (STAGED) {
-    extern __shared__ __align__(16) float4 stage4[];
-    const float4* Y4 = reinterpret_cast<const float4*>(Y);
-    const int n4 = d * (K / 4);
-    constexpr int UL = 8;
-    for (int e0 = threadIdx.x; e0 < n4; e0 += kT * UL) {
-      float4 v[UL];
-#pragma unroll
-      for (int q = 0; q < UL; ++q) {
-        const int e = e0 + q * kT;
-        v[q] = e < n4 ? Y4[e] : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int q = 0; q < UL; ++q) {
-        const int e = e0 + q * kT;
-        if (e < n4) stage4[e] = v[q];
-      }
-    }
-    __syncthreads();
-    float* stage = reinterpret_cast<float*>(stage4);
-    cholqr2_block<K, F64>(stage, stage, Z, d, k, status);
-  } else {
-    cholqr2_block<K, F64>(Y, Z, Z, d, k, status);
-  }
-}
-
-template <int K, bool F64>
-cudaError_t launch_cholqr2_t(const float* Y, float* Z, int batch, int d, int k, int* status, cudaStream_t s) {
-  const size_t bytes = size_t(d) * K * 4;
-  if (bytes <= kCholStageBytes) {
-    const cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void*>(cholqr2_kernel<K, F64, true>));
-    if (e != cudaSuccess) return e;
-    cholqr2_kernel<K, F64, true><<<batch, kT, bytes, s>>>(Y, Z, d, k, status);
-  } else {
-    cholqr2_kernel<K, F64, false><<<batch, kT, 0, s>>>(Y, Z, d, k, status);
-  }
-  return cudaGetLastError();
-}
-
 
 // ---------------------------------------------------------------- align
 // One CTA per partition.  G_i (K x K float, row-major) = D_i (sign) or O_i (OPT).
@@ -1060,19 +689,6 @@ cudaError_t launch_reduce(const float* P, const int* slot_begin, const float* sc
     default: reduce_kernel<32><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y); break;
   }
   return cudaGetLastError();
-}
-
-cudaError_t launch_cholqr2(const float* Y, float* Z, int batch, int d, int k, int K, int* status, cudaStream_t s,
-                           bool kxk_fp64) {
-  switch (K * 2 + (kxk_fp64 ? 1 : 0)) {
-    case 16: return launch_cholqr2_t<8, false>(Y, Z, batch, d, k, status, s);
-    case 17: return launch_cholqr2_t<8, true>(Y, Z, batch, d, k, status, s);
-    case 32: return launch_cholqr2_t<16, false>(Y, Z, batch, d, k, status, s);
-    case 33: return launch_cholqr2_t<16, true>(Y, Z, batch, d, k, status, s);
-    case 64: return launch_cholqr2_t<32, false>(Y, Z, batch, d, k, status, s);
-    case 65: return launch_cholqr2_t<32, true>(Y, Z, batch, d, k, status, s);
-    default: return cudaErrorInvalidValue;
-  }
 }
 
 cudaError_t launch_align(const float* Zl, int64_t z_stride, const float* Zb, int m, int d, int k, int K, int base,
