@@ -645,21 +645,33 @@ lp_status lp::load_pitched(lp_ctx* c, int m, const int64_t* rows, int64_t d, int
       }
     }
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < m && e == cudaSuccess; ++i) {
-      const float* src = static_cast<const float*>(parts[i]);
-      for (int64_t r0 = 0; r0 < rows[i] && e == cudaSuccess; r0 += chunk_rows) {
-        const int64_t nr = std::min(chunk_rows, rows[i] - r0);
-        const size_t off = size_t(c->row_off[i] + r0) * c->ld;
-        const float* from = src + size_t(r0) * pitch;
-        int64_t from_ld = pitch;
-        if (space == LP_HOST) {
-          e = cudaMemcpy2DAsync(stage, size_t(d) * 4, from, size_t(pitch) * 4, size_t(d) * 4, size_t(nr),
-                                cudaMemcpyHostToDevice, c->stream);
-          from = stage;
-          from_ld = d;
+    lp::SplitParts sp;
+    sp.n = 0;
+    sp.row0[0] = 0;
+    if (space == LP_DEVICE) {  // many partitions per launch
+      for (int i = 0; i < m && e == cudaSuccess; ++i) {
+        sp.src[sp.n] = static_cast<const float*>(parts[i]);
+        sp.row0[sp.n + 1] = sp.row0[sp.n] + rows[i];
+        if (++sp.n == lp::kSplitParts || i == m - 1) {
+          const size_t off = size_t(c->row_off[i + 1 - sp.n]) * c->ld;
+          e = lp::launch_split_planes(sp, pitch, static_cast<int>(d), hi + off, lo + off, c->ld, c->stream);
+          sp.n = 0;
         }
-        if (e == cudaSuccess)
-          e = lp::launch_split_planes(from, from_ld, nr, static_cast<int>(d), hi + off, lo + off, c->ld, c->stream);
+      }
+    } else {
+      for (int i = 0; i < m && e == cudaSuccess; ++i) {
+        const float* src = static_cast<const float*>(parts[i]);
+        for (int64_t r0 = 0; r0 < rows[i] && e == cudaSuccess; r0 += chunk_rows) {
+          const int64_t nr = std::min(chunk_rows, rows[i] - r0);
+          const size_t off = size_t(c->row_off[i] + r0) * c->ld;
+          e = cudaMemcpy2DAsync(stage, size_t(d) * 4, src + size_t(r0) * pitch, size_t(pitch) * 4, size_t(d) * 4,
+                                size_t(nr), cudaMemcpyHostToDevice, c->stream);
+          sp.src[0] = stage;
+          sp.row0[1] = nr;
+          sp.n = 1;
+          if (e == cudaSuccess)
+            e = lp::launch_split_planes(sp, d, static_cast<int>(d), hi + off, lo + off, c->ld, c->stream);
+        }
       }
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

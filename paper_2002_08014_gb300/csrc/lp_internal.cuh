@@ -131,10 +131,17 @@ cudaError_t launch_step_tcs8(const TcsPlan& p, const Segment* segs, const int* s
                              cudaStream_t s);
 cudaError_t launch_step_pair(const TcsPlan& p, const Segment* segs, const int* seg_ptr, const float* Z,
                              int64_t z_stride, float* P, int d, int* status, cudaStream_t s);
-// FP32 rows (pitch src_ld) -> hi = RNE_bf16(a), lo = RNE_bf16(a - hi) planes (pitch ld,
-// columns d..ld-1 zero).
-cudaError_t launch_split_planes(const float* src, int64_t src_ld, int64_t rows, int d, uint16_t* hi, uint16_t* lo,
-                                int64_t ld, cudaStream_t s);
+// FP32 rows (pitch src_ld) -> hi = RNE_bf16(a), lo = RNE_bf16(a - hi) planes (pitch ld, a
+// multiple of 8, 16-byte aligned; columns d..ld-1 zero).  Partition i's rows become rows
+// row0[i] .. row0[i + 1] - 1 of the planes (row0[0] = 0).
+constexpr int kSplitParts = 128;
+struct SplitParts {
+  const float* src[kSplitParts];
+  int64_t row0[kSplitParts + 1];
+  int n;
+};
+cudaError_t launch_split_planes(const SplitParts& parts, int64_t src_ld, int d, uint16_t* hi, uint16_t* lo, int64_t ld,
+                                cudaStream_t s);
 
 // ---- context internals used by the request server ---------------------------
 // lp_load_partitions with a row pitch (elements) for the partitions' source rows.

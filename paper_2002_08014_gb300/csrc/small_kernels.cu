@@ -28,17 +28,70 @@ constexpr int kT = 256;
 // ---------------------------------------------------------------- pack / unpack
 // FP32 rows -> two BF16 planes: hi = RNE(a), lo = RNE(a - hi).  a - hi is exact
 // in FP32, so hi + lo matches a to within half an ulp of lo (<= 2^-17 |a|).
-__global__ void split_planes_kernel(const float* __restrict__ src, int64_t src_ld, int64_t rows, int d,
-                                    uint16_t* __restrict__ hi, uint16_t* __restrict__ lo, int64_t ld) {
-  const int64_t total = rows * ld;
-  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t r = e / ld;
-    const int c = static_cast<int>(e - r * ld);
-    const float a = c < d ? src[r * src_ld + c] : 0.f;
-    const __nv_bfloat16 h = __float2bfloat16_rn(a);
-    const __nv_bfloat16 l = __float2bfloat16_rn(a - __bfloat162float(h));
-    hi[e] = __bfloat16_as_ushort(h);
-    lo[e] = __bfloat16_as_ushort(l);
+// Bound by HBM (4 bytes read, 4 written per element).  One launch takes up to
+// kSplitParts partitions, so that a load of many small ones has no launch tails;
+// a thread converts eight columns of a row (two 16-byte loads, one 16-byte store
+// per plane) and has two such groups in flight.  Rows that are not 16-byte
+// aligned, and a row's last columns, are read one by one.  Measured, 64 partitions
+// of 2,048 x 1,024: 732 us (64 launches, an element per thread) -> 158 us, 6.8 TB/s.
+__device__ __forceinline__ void split8(const float* __restrict__ src, int64_t src_ld, bool vec, int64_t row, int c, int d,
+                                       float (&v)[8]) {
+  const float* p = src + row * src_ld + c;
+  if (vec && c + 8 <= d) {
+    const float4 x = reinterpret_cast<const float4*>(p)[0], y = reinterpret_cast<const float4*>(p)[1];
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+  } else {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = c + q < d ? p[q] : 0.f;
+  }
+}
+
+__global__ void __launch_bounds__(kT) split_planes_kernel(const __grid_constant__ SplitParts parts, int64_t src_ld,
+                                                          int d, uint16_t* __restrict__ hi,
+                                                          uint16_t* __restrict__ lo, int ld8) {
+  const int64_t total = parts.row0[parts.n] * ld8;
+  const int64_t step = int64_t(gridDim.x) * kT;
+  int part = 0;
+  for (int64_t e0 = blockIdx.x * int64_t(kT) + threadIdx.x; e0 < total; e0 += 2 * step) {
+    float v[2][8];
+    int64_t at[2];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const int64_t e = e0 + x * step;
+      at[x] = -1;
+      if (e >= total) continue;
+      int64_t r;
+      int c;
+      if (total < (int64_t(1) << 31)) {
+        r = static_cast<uint32_t>(e) / static_cast<uint32_t>(ld8);
+        c = static_cast<int>(static_cast<uint32_t>(e) - static_cast<uint32_t>(r) * ld8);
+      } else {
+        r = e / ld8;
+        c = static_cast<int>(e - r * ld8);
+      }
+      while (r >= parts.row0[part + 1]) ++part;  // a thread's rows ascend
+      const float* src = parts.src[part];
+      const bool vec = ((reinterpret_cast<uintptr_t>(src) | static_cast<uintptr_t>(src_ld * 4)) & 15) == 0;
+      split8(src, src_ld, vec, r - parts.row0[part], 8 * c, d, v[x]);
+      at[x] = e;
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      if (at[x] < 0) continue;
+      uint32_t h[4], l[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float a0 = v[x][2 * q], a1 = v[x][2 * q + 1];
+        const __nv_bfloat16 h0 = __float2bfloat16_rn(a0), h1 = __float2bfloat16_rn(a1);
+        const __nv_bfloat16 l0 = __float2bfloat16_rn(a0 - __bfloat162float(h0));
+        const __nv_bfloat16 l1 = __float2bfloat16_rn(a1 - __bfloat162float(h1));
+        h[q] = __bfloat16_as_ushort(h0) | (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
+        l[q] = __bfloat16_as_ushort(l0) | (static_cast<uint32_t>(__bfloat16_as_ushort(l1)) << 16);
+      }
+      reinterpret_cast<uint4*>(hi)[at[x]] = make_uint4(h[0], h[1], h[2], h[3]);
+      reinterpret_cast<uint4*>(lo)[at[x]] = make_uint4(l[0], l[1], l[2], l[3]);
+    }
   }
 }
 
@@ -649,12 +702,12 @@ cudaError_t allow_max_dynamic_smem(const void* kern) {
   return e;
 }
 
-cudaError_t launch_split_planes(const float* src, int64_t src_ld, int64_t rows, int d, uint16_t* hi, uint16_t* lo,
-                                int64_t ld, cudaStream_t s) {
-  if (rows <= 0) return cudaSuccess;
-  const int64_t total = rows * ld;
-  const int64_t blocks = std::min<int64_t>((total + kT - 1) / kT, 4096);
-  split_planes_kernel<<<static_cast<unsigned>(blocks), kT, 0, s>>>(src, src_ld, rows, d, hi, lo, ld);
+cudaError_t launch_split_planes(const SplitParts& parts, int64_t src_ld, int d, uint16_t* hi, uint16_t* lo, int64_t ld,
+                                cudaStream_t s) {
+  const int64_t total = parts.n > 0 ? parts.row0[parts.n] * (ld / 8) : 0;
+  if (total <= 0) return cudaSuccess;
+  const int64_t blocks = std::min<int64_t>((total + 2 * kT - 1) / (2 * kT), 152 * 8);
+  split_planes_kernel<<<static_cast<unsigned>(blocks), kT, 0, s>>>(parts, src_ld, d, hi, lo, static_cast<int>(ld / 8));
   return cudaGetLastError();
 }
 
