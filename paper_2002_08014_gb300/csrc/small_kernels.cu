@@ -18,6 +18,7 @@
 
 #include <cuda_bf16.h>
 
+#include "inv_sqrt.cuh"
 #include "lp_internal.cuh"
 
 namespace lp {
@@ -170,6 +171,10 @@ __device__ __forceinline__ float warp_sumf(float v) {
 // error times k, so the last sweep only sees rounding noise below it); `tiny`
 // skips pairs whose product underflows; beyond `huge` t = 1 / (2 |zeta|) avoids
 // squaring zeta.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float inv_root(float x) { return inv_sqrt(x); }
+__device__ __forceinline__ double inv_root(double x) { return 1.0 / sqrt(x); }
 template <typename T> struct JacobiLimits;
 template <> struct JacobiLimits<float> {
   static constexpr float tol = 1e-6f, tiny = 1e-35f, huge = 1e15f;
@@ -178,7 +183,7 @@ template <> struct JacobiLimits<double> {
   static constexpr double tol = 1e-13, tiny = 1e-300, huge = 1e150;
 };
 
-// One-sided (Hestenes) Jacobi on the k x k matrix C (stride K, in shared memory),
+// One-sided (Hestenes) Jacobi on the k x k matrix C (stride ks, in shared memory),
 // accumulating the rotations in V, in precision T: on return C's columns are
 // mutually orthogonal, C_in V = C_out, so C_in = U Sigma V^T with
 // sigma_j = ||C_out[:, j]|| and U[:, j] = C_out[:, j] / sigma_j.  FP32 by
@@ -196,13 +201,20 @@ template <> struct JacobiLimits<double> {
 // of the two columns, sum the three inner products over the half-warp and
 // rotate their rows.  One barrier per step; the sweeps stop when a whole sweep
 // rotated nothing.  Returns false if the sweep limit was hit.
+// ks = jacobi_stride(K), one past K: a half-warp reads 16 rows of one column, which
+// at a stride of 32 words would all lie in one bank (OPT align, 20 blocks of 362 x 24:
+// 212 -> 90 us with it, the pair's rows read once and the rotation's root as inv_sqrt;
+// 64 of 1,024 x 16: 82 -> 50).  What is left is the chain of a step, ~750 cycles: the
+// four shuffles, two divisions and two roots, and the barrier.
+__host__ __device__ constexpr int jacobi_stride(int K) { return K + 1; }
 template <typename T>
 __device__ bool cta_jacobi(T* C, T* V, int k, int K) {
+  const int ks = jacobi_stride(K);
   using L = JacobiLimits<T>;
   const int t = threadIdx.x;
   const int slot = t >> 4, h = t & 15;
   const int np = k + (k & 1);
-  for (int e = t; e < K * K; e += kT) V[e] = (e / K == e % K) ? T(1) : T(0);
+  for (int e = t; e < K * K; e += kT) V[e / K * ks + e % K] = (e / K == e % K) ? T(1) : T(0);
   __syncthreads();
   for (int sweep = 0; sweep < 40; ++sweep) {
     int rotated = 0;
@@ -210,45 +222,58 @@ __device__ bool cta_jacobi(T* C, T* V, int k, int K) {
       int p = 0, q = 0;
       bool live = slot < np / 2;
       if (live) {
-        if (slot == 0) {
-          p = s;
-          q = np - 1;
-        } else {
-          p = (s + slot) % (np - 1);
-          q = (s - slot + np - 1) % (np - 1);
-        }
+        p = s + (slot == 0 ? 0 : slot);
+        if (p >= np - 1) p -= np - 1;
+        q = slot == 0 ? np - 1 : s - slot;
+        if (q < 0) q += np - 1;
         live = p < k && q < k;
       }
+      // rows h and h + 16 of the pair, read once for the products and the rotation
+      const bool r0 = live && h < k, r1 = live && h + 16 < k;
+      T *c0 = C + h * ks, *c1 = c0 + 16 * ks;
+      const T p0 = r0 ? c0[p] : T(0), q0 = r0 ? c0[q] : T(0);
+      const T p1 = r1 ? c1[p] : T(0), q1 = r1 ? c1[q] : T(0);
       T a = 0, b = 0, g = 0;
-      if (live)
-        for (int r = h; r < k; r += 16) {
-          const T cp = C[r * K + p], cq = C[r * K + q];
-          a += cp * cp;
-          b += cq * cq;
-          g += cp * cq;
+      if (__any_sync(0xffffffffu, live)) {  // a warp without a pair skips the sums (FP64: its pipe is the bound)
+        a = mul_rn(p0, p0);
+        b = mul_rn(q0, q0);
+        g = mul_rn(p0, q0);
+        if (k > 16) {
+          a = fma(p1, p1, a);
+          b = fma(q1, q1, b);
+          g = fma(p1, q1, g);
         }
-      // every lane takes part in the shuffles; offsets below 16 stay in the half-warp
+        // every lane takes part in the shuffles; offsets below 16 stay in the half-warp
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-        g += __shfl_xor_sync(0xffffffffu, g, o);
+        for (int o = 8; o > 0; o >>= 1) {
+          a += __shfl_xor_sync(0xffffffffu, a, o);
+          b += __shfl_xor_sync(0xffffffffu, b, o);
+          g += __shfl_xor_sync(0xffffffffu, g, o);
+        }
       }
       if (live && fabs(g) > L::tol * sqrt(a * b) && fabs(g) > L::tiny) {
         rotated = 1;
         // zeta = (b - a) / 2g, t = sgn(zeta) / (|zeta| + sqrt(1 + zeta^2)), c = 1 / sqrt(1 + t^2)
         const T zeta = (b - a) / (T(2) * g);
         const T az = fabs(zeta);
-        const T tn = (zeta >= T(0) ? T(1) : T(-1)) / (az > L::huge ? T(2) * az : az + sqrt(T(1) + zeta * zeta));
-        const T c = T(1) / sqrt(T(1) + tn * tn);
+        const T tn = (zeta >= T(0) ? T(1) : T(-1)) / (az > L::huge ? T(2) * az : az + sqrt(fma(zeta, zeta, T(1))));
+        const T c = inv_root(fma(tn, tn, T(1)));
         const T sn = c * tn;
-        for (int r = h; r < k; r += 16) {
-          const T cp = C[r * K + p], cq = C[r * K + q];
-          C[r * K + p] = c * cp - sn * cq;
-          C[r * K + q] = sn * cp + c * cq;
-          const T vp = V[r * K + p], vq = V[r * K + q];
-          V[r * K + p] = c * vp - sn * vq;
-          V[r * K + q] = sn * vp + c * vq;
+        // a rotated pair of values: (c x - s y, s x + c y), one product of each rounded first
+        auto rot = [&](T x, T y, T& lo, T& hi) {
+          lo = fma(c, x, -mul_rn(sn, y));
+          hi = fma(sn, x, mul_rn(c, y));
+        };
+        T *v0 = V + h * ks, *v1 = v0 + 16 * ks;
+        if (r0) {
+          const T vp = v0[p], vq = v0[q];
+          rot(p0, q0, c0[p], c0[q]);
+          rot(vp, vq, v0[p], v0[q]);
+        }
+        if (r1) {
+          const T vp = v1[p], vq = v1[q];
+          rot(p1, q1, c1[p], c1[q]);
+          rot(vp, vq, v1[p], v1[q]);
         }
       }
       __syncthreads();
@@ -265,23 +290,23 @@ __device__ bool cta_jacobi(T* C, T* V, int k, int K) {
 // threads call it; `inv` holds K values of scratch.
 template <typename T>
 __device__ void procrustes_factor(T* C, const T* V, T* inv, int k, int K, float* Gi, int* status) {
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, ks = jacobi_stride(K);
   const T small = sizeof(T) == 8 ? T(1e-300) : T(1e-37);
   if (t < k) {
     T nrm = 0;
-    for (int r = 0; r < k; ++r) nrm += C[r * K + t] * C[r * K + t];
+    for (int r = 0; r < k; ++r) nrm += C[r * ks + t] * C[r * ks + t];
     inv[t] = nrm > small ? T(1) / sqrt(nrm) : T(0);
     if (!(nrm > small)) atomicOr(status, ST_JACOBI);
   }
   __syncthreads();
   for (int e = t; e < k * K; e += kT)
-    if (e % K < k) C[e] *= inv[e % K];
+    if (e % K < k) C[e / K * ks + e % K] *= inv[e % K];
   __syncthreads();
   for (int e = t; e < K * K; e += kT) {
     const int a = e / K, b = e % K;
     T sum = 0;
     if (a < k && b < k)
-      for (int j = 0; j < k; ++j) sum = fma(C[a * K + j], V[b * K + j], sum);
+      for (int j = 0; j < k; ++j) sum = fma(C[a * ks + j], V[b * ks + j], sum);
     Gi[e] = static_cast<float>(sum);
   }
 }
@@ -293,9 +318,10 @@ __global__ void __launch_bounds__(kT) align_kernel(const float* __restrict__ Zl,
                                                    int base_one, const int* __restrict__ part_base, int opt, int f64,
                                                    float* __restrict__ Gout, int* status) {
   extern __shared__ __align__(16) unsigned char sm[];
-  double* C = reinterpret_cast<double*>(sm);   // K*K
-  double* V = C + K * K;                        // K*K
-  double* part = V + K * K;                     // kT x 16 floats
+  const int ks = jacobi_stride(K);
+  double* C = reinterpret_cast<double*>(sm);   // K rows of stride ks
+  double* V = C + K * ks;                       // the same
+  double* part = V + K * ks;                    // kT x 16 floats
   const int i = blockIdx.x;
   const int t = threadIdx.x;
   // the base of partition i's problem: one for the context, or per partition (batch groups)
@@ -308,22 +334,53 @@ __global__ void __launch_bounds__(kT) align_kernel(const float* __restrict__ Zl,
   }
   const float* Zi = Zl + z_stride * i;
   if (!opt) {
-    // sgn <Z_i[:, j], Z_b[:, j]> with FP64 accumulation; sgn(0) = +1.
+    // sgn <Z_i[:, j], Z_b[:, j]> as FP64 accumulation gives it; sgn(0) = +1.  The FP64
+    // pipe would take 12 us at d = 1,024, K = 16 (two conversions and a multiply-add per
+    // entry at 2 per clock), so an FP32 sum decides where it can: with D the sum of
+    // the products' magnitudes, any order of n FP32 multiply-adds is within n u D / (1 -
+    // n u) of the exact sum, u = 2^-24 (Higham, Accuracy and Stability of Numerical
+    // Algorithms, Sec. 3.1), and the FP64 sum within far less.  A column whose FP32
+    // sum is not above twice that bound (or is NaN) sends the block to the FP64 sums.
+    // Measured, 64 blocks of 1,024 x 16: 16.3 -> 5.6 us; 4 of 100 x 5: 3.6 -> 2.2.
     const int j = t % K, sl = t / K, RS = kT / K;
-    double s = 0.0;
-    for (int r = sl; r < d; r += RS) s += static_cast<double>(Zi[int64_t(r) * K + j]) * Zb[int64_t(r) * K + j];
-    part[t] = s;
-    __syncthreads();
-    if (t < K) {
-      double tot = 0.0;
-      for (int q = 0; q < RS; ++q) tot += part[q * K + t];
-      part[kT - K + t] = tot;  // scratch beyond the first RS*K entries is not re-read
+    float* dots = reinterpret_cast<float*>(part);
+    float f = 0.f, m = 0.f;
+#pragma unroll 4
+    for (int r = sl; r < d; r += RS) {
+      const float x = Zi[int64_t(r) * K + j], y = Zb[int64_t(r) * K + j];
+      f = fmaf(x, y, f);
+      m = fmaf(fabsf(x), fabsf(y), m);
     }
+    dots[t] = f;
+    dots[kT + t] = m;
     __syncthreads();
+    bool sure = true;
+    if (t < K) {
+      float tot = 0.f, mag = 0.f;
+      for (int q = 0; q < RS; ++q) {
+        tot += dots[q * K + t];
+        mag += dots[kT + q * K + t];
+      }
+      // columns beyond k hold zeros: nothing to decide
+      sure = t >= k || fabsf(tot) > 2.f * (static_cast<float>(d) + RS + 2) * 0x1.0p-24f * mag;
+      part[kT + t] = tot;  // beyond the sums of either precision
+    }
+    if (__syncthreads_or(!sure)) {
+      double s = 0.0;
+      for (int r = sl; r < d; r += RS) s += static_cast<double>(Zi[int64_t(r) * K + j]) * Zb[int64_t(r) * K + j];
+      part[t] = s;
+      __syncthreads();
+      if (t < K) {
+        double tot = 0.0;
+        for (int q = 0; q < RS; ++q) tot += part[q * K + t];
+        part[kT + t] = tot;
+      }
+      __syncthreads();
+    }
     for (int e = t; e < K * K; e += kT) {
       const int a = e / K, b = e % K;
       float v = 0.f;
-      if (a == b && a < k) v = part[kT - K + a] < 0.0 ? -1.f : 1.f;
+      if (a == b && a < k) v = part[kT + a] < 0.0 ? -1.f : 1.f;
       Gi[e] = v;
     }
     return;
@@ -362,14 +419,14 @@ __global__ void __launch_bounds__(kT) align_kernel(const float* __restrict__ Zl,
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) red[t * 16 + 4 * a + b] = acc[a][b];
+      for (int b = 0; b < 4; ++b) red[(4 * a + b) * kT + t] = acc[a][b];
     __syncthreads();
     for (int e = t; e < K * K; e += kT) {
       const int a = e / K, b = e % K;
       const int bb = (a / 4) * NB + b / 4, el = 4 * (a % 4) + b % 4;
       double sum = 0.0;
-      for (int q = 0; q < S; ++q) sum += red[(q * NBB + bb) * 16 + el];
-      C[e] = sum;
+      for (int q = 0; q < S; ++q) sum += red[el * kT + q * NBB + bb];
+      C[a * ks + b] = sum;
     }
     __syncthreads();
   }
@@ -379,10 +436,10 @@ __global__ void __launch_bounds__(kT) align_kernel(const float* __restrict__ Zl,
     if (!ok && t == 0) atomicOr(status, ST_JACOBI);
     procrustes_factor<double>(C, V, part, k, K, Gi, status);
   } else {
-    // FP32 copies in the V area (2 K*K floats fit in K*K doubles)
+    // FP32 copies in the V area (two float blocks fit in one of doubles)
     float* Cf = reinterpret_cast<float*>(V);
-    float* Vf = Cf + K * K;
-    for (int e = t; e < K * K; e += kT) Cf[e] = static_cast<float>(C[e]);
+    float* Vf = Cf + K * ks;
+    for (int e = t; e < K * ks; e += kT) Cf[e] = static_cast<float>(C[e]);
     __syncthreads();
     const bool ok = cta_jacobi<float>(Cf, Vf, k, K);
     if (!ok && t == 0) atomicOr(status, ST_JACOBI);
@@ -390,10 +447,10 @@ __global__ void __launch_bounds__(kT) align_kernel(const float* __restrict__ Zl,
   }
 }
 
-// C and V (K x K doubles each), then the partial-block area (kT x 16 floats; it
+// C and V (K rows of stride K + 1, doubles), then the partial-block area (kT x 16 floats; it
 // also holds the column scales of the Procrustes factor, and the sign path's
 // kT doubles)
-size_t align_smem(int K) { return size_t(2) * K * K * 8 + size_t(kT) * 16 * 4 + 16; }
+size_t align_smem(int K) { return size_t(2) * K * jacobi_stride(K) * 8 + size_t(kT) * 16 * 4 + 16; }
 
 // ---------------------------------------------------------------- residual error
 // rho_i = ||Z_i G_i - Z_b||_2 (Def. 3) for one partition per CTA: E = Z_i G_i - Z_b
@@ -407,9 +464,10 @@ __global__ void __launch_bounds__(kT) rho_kernel(const float* __restrict__ Zl, i
                                                  int diag_only, int base, int d, int k, int K,
                                                  double* __restrict__ out, int* status) {
   extern __shared__ __align__(16) unsigned char sm[];
-  double* C = reinterpret_cast<double*>(sm);  // K*K Gram, then Jacobi workspace
-  double* V = C + K * K;                       // K*K
-  float* E = reinterpret_cast<float*>(V + K * K);  // kRhoRows x K
+  const int ks = jacobi_stride(K);
+  double* C = reinterpret_cast<double*>(sm);  // K*K Gram
+  double* V = C + K * K;                       // Jacobi workspace, K rows of stride ks
+  float* E = reinterpret_cast<float*>(V + K * ks);  // kRhoRows x K
   const int i = blockIdx.x, t = threadIdx.x;
   if (i == base) {
     if (t == 0) out[i] = 0.0;
@@ -453,8 +511,8 @@ __global__ void __launch_bounds__(kT) rho_kernel(const float* __restrict__ Zl, i
   __syncthreads();
   // E^T E is symmetric positive semidefinite: the one-sided Jacobi's column norms are its eigenvalues
   float* Cf = reinterpret_cast<float*>(V);
-  float* Vf = Cf + K * K;
-  for (int e = t; e < K * K; e += kT) Cf[e] = static_cast<float>(C[e]);
+  float* Vf = Cf + K * ks;
+  for (int e = t; e < K * K; e += kT) Cf[e / K * ks + e % K] = static_cast<float>(C[e]);
   __syncthreads();
   const bool ok = cta_jacobi<float>(Cf, Vf, k, K);
   if (!ok && t == 0) atomicOr(status, ST_JACOBI);
@@ -462,7 +520,7 @@ __global__ void __launch_bounds__(kT) rho_kernel(const float* __restrict__ Zl, i
     float top = 0.f;
     for (int j = 0; j < k; ++j) {
       float v = 0.f;
-      if (t < k) v = Cf[t * K + j] * Cf[t * K + j];
+      if (t < k) v = Cf[t * ks + j] * Cf[t * ks + j];
       v = warp_sumf(v);
       top = fmaxf(top, v);
     }
@@ -602,24 +660,25 @@ __global__ void __launch_bounds__(kT) ritz_solve_kernel(const double* __restrict
   Vo += int64_t(qp) * K * K;
   sigma += int64_t(qp) * LP_MAX_K;
   const double n = n_of ? n_of[qp] : n_one;
-  double* H = reinterpret_cast<double*>(sm);  // K*K
-  double* V = H + K * K;                       // K*K
-  double* lam = V + K * K;                     // K
+  const int ks = jacobi_stride(K);
+  double* H = reinterpret_cast<double*>(sm);  // K rows of stride ks
+  double* V = H + K * ks;                      // the same
+  double* lam = V + K * ks;                    // K
   int* order = reinterpret_cast<int*>(lam + K);
   const int t = threadIdx.x;
   for (int e = t; e < K * K; e += kT) {
     double sum = 0.0;
     for (int g = 0; g < slices; ++g) sum += Hpart[int64_t(g) * K * K + e];
-    H[e] = sum;
+    H[e / K * ks + e % K] = sum;
   }
   __syncthreads();
   // symmetrise: the thread of entry (a, b), a < b, writes both halves
   for (int e = t; e < K * K; e += kT) {
     const int a = e / K, b = e % K;
     if (a < b) {
-      const double v = 0.5 * (H[a * K + b] + H[b * K + a]);
-      H[a * K + b] = v;
-      H[b * K + a] = v;
+      const double v = 0.5 * (H[a * ks + b] + H[b * ks + a]);
+      H[a * ks + b] = v;
+      H[b * ks + a] = v;
     }
   }
   __syncthreads();
@@ -631,19 +690,19 @@ __global__ void __launch_bounds__(kT) ritz_solve_kernel(const double* __restrict
     if (!ok && t == 0) atomicOr(status, ST_JACOBI);
     if (t < k) {
       double v = 0.0;
-      for (int r = 0; r < k; ++r) v += H[r * K + t] * H[r * K + t];
+      for (int r = 0; r < k; ++r) v += H[r * ks + t] * H[r * ks + t];
       lam[t] = v > 0.0 ? sqrt(v) : 0.0;
     }
   } else {
     float* Hf = reinterpret_cast<float*>(V);
-    float* Vf = Hf + K * K;
-    for (int e = t; e < K * K; e += kT) Hf[e] = static_cast<float>(H[e]);
+    float* Vf = Hf + K * ks;
+    for (int e = t; e < K * K; e += kT) Hf[e / K * ks + e % K] = static_cast<float>(H[e / K * ks + e % K]);
     __syncthreads();
     const bool ok = cta_jacobi<float>(Hf, Vf, k, K);
     if (!ok && t == 0) atomicOr(status, ST_JACOBI);
     if (t < k) {
       float v = 0.f;
-      for (int r = 0; r < k; ++r) v += Hf[r * K + t] * Hf[r * K + t];
+      for (int r = 0; r < k; ++r) v += Hf[r * ks + t] * Hf[r * ks + t];
       lam[t] = v > 0.f ? sqrt(static_cast<double>(v)) : 0.0;
     }
   }
@@ -663,8 +722,8 @@ __global__ void __launch_bounds__(kT) ritz_solve_kernel(const double* __restrict
   for (int e = t; e < K * K; e += kT) {
     const int l = e / K, j = e % K;
     Vo[e] = j >= k ? 0.0
-                   : f64 ? V[l * K + order[j]]
-                         : static_cast<double>(reinterpret_cast<const float*>(V)[K * K + l * K + order[j]]);
+                   : f64 ? V[l * ks + order[j]]
+                         : static_cast<double>(reinterpret_cast<const float*>(V)[K * ks + l * ks + order[j]]);
   }
 }
 
@@ -787,7 +846,7 @@ cudaError_t launch_ritz(const float* Z, const float* MZ, int d, int k, int K, do
   ritz_partial_kernel<<<dim3(slices, nprob), kT, 0, s>>>(Z, MZ, d, k, K, Hpart);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const size_t sm = size_t(2) * K * K * 8 + size_t(K) * 8 + size_t(K) * 4 + 16;
+  const size_t sm = size_t(2) * K * jacobi_stride(K) * 8 + size_t(K) * 8 + size_t(K) * 4 + 16;
   ritz_solve_kernel<<<nprob, kT, sm, s>>>(Hpart, slices, k, K, n, n_of, kxk_fp64 ? 1 : 0, Vo, sigma, status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int64_t total = int64_t(nprob) * d * k;
@@ -797,7 +856,7 @@ cudaError_t launch_ritz(const float* Z, const float* MZ, int d, int k, int K, do
 
 cudaError_t launch_rho(const float* Zl, int64_t z_stride, const float* Zb, const float* G, int diag_only, int base,
                        int m, int d, int k, int K, double* out, int* status, cudaStream_t s) {
-  const size_t sm = size_t(2) * K * K * 8 + size_t(kRhoRows) * K * 4;
+  const size_t sm = (size_t(K) * K + size_t(K) * jacobi_stride(K)) * 8 + size_t(kRhoRows) * K * 4;
   rho_kernel<<<m, kT, sm, s>>>(Zl, z_stride, Zb, G, diag_only, base, d, k, K, out, status);
   return cudaGetLastError();
 }
