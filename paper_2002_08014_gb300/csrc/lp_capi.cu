@@ -107,6 +107,7 @@ struct lp_ctx {
   double *dZout = nullptr, *dSigma = nullptr, *dStage = nullptr;
   size_t stage_bytes = 0;
   int* dStatus = nullptr;
+  int* hStatus = nullptr;  // pinned, written by the device: the single power step's status (allocated at its first call)
 
   // last solve
   bool solved = false;
@@ -473,6 +474,7 @@ void lp_destroy(lp_ctx* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   free_partitions(c);
   dfree(c, c->dStatus, 16);
+  if (c->hStatus) cudaFreeHost(c->hStatus);
   drop_graph(c);
   for (cudaEvent_t e : c->step_ev) cudaEventDestroy(e);
   if (c->ev0) cudaEventDestroy(c->ev0);
@@ -1386,24 +1388,30 @@ lp_status lp_power_step(lp_ctx* c, int k, const double* z, int z_shared, double*
   const int K = kcap_of(k);
   if ((st = select_path(c, k, 0))) return st;
   if ((st = ensure_state(c, K))) return st;
-  LP_CUDA(cudaMemsetAsync(c->dStatus, 0, 4, c->stream));
+  // the status word reaches the host by the last kernel's store: a copy to pageable memory
+  // would stage and wait, a third of the smallest call's time
+  if (!c->hStatus && cudaHostAlloc(reinterpret_cast<void**>(&c->hStatus), 4, cudaHostAllocMapped) != cudaSuccess) {
+    (void)cudaGetLastError();
+    c->hStatus = nullptr;
+  }
   const int d = static_cast<int>(c->d);
   const int nb = z_shared ? 1 : c->m;
   const double* dz;
   if ((st = stage_in(c, z, size_t(nb) * d * k, space, &dz))) return st;
   float* Zt = z_shared ? c->dZ : c->dZl;
-  if ((st = check_launch(c, lp::launch_pack(dz, Zt, nb, d, k, K, c->stream), "pack"))) return st;
+  if ((st = check_launch(c, lp::launch_pack(dz, Zt, nb, d, k, K, c->stream, c->dStatus), "pack"))) return st;
   if ((st = launch_step(c, K, Zt, z_shared ? 0 : int64_t(d) * K, false))) return st;
-  if ((st = check_launch(c, lp::launch_reduce(c->dP, slot_begin_of(c), c->dInvS, c->m, d, K, c->dYl, c->stream, c->max_slots[c->path]),
+  double* dst = space == LP_DEVICE ? y_out : c->dStage;
+  if ((st = check_launch(c, lp::launch_reduce_f64(c->dP, slot_begin_of(c), c->dInvS, c->m, d, k, K, dst, c->dStatus,
+                                                  c->hStatus, c->stream, c->max_slots[c->path]),
                          "reduce")))
     return st;
-  double* dst = space == LP_DEVICE ? y_out : c->dStage;
-  if ((st = check_launch(c, lp::launch_unpack(c->dYl, dst, c->m, d, k, K, c->stream), "unpack"))) return st;
   if (space == LP_HOST)
     LP_CUDA(cudaMemcpyAsync(y_out, dst, size_t(c->m) * d * k * 8, cudaMemcpyDeviceToHost, c->stream));
   int status = 0;
-  LP_CUDA(cudaMemcpyAsync(&status, c->dStatus, 4, cudaMemcpyDeviceToHost, c->stream));
+  if (!c->hStatus) LP_CUDA(cudaMemcpyAsync(&status, c->dStatus, 4, cudaMemcpyDeviceToHost, c->stream));
   LP_CUDA(cudaStreamSynchronize(c->stream));
+  if (c->hStatus) status = *static_cast<volatile int*>(c->hStatus);
   if (status & lp::ST_TIMEOUT) return fail(c, LP_ERR_TIMEOUT, "device wait timed out in the power step");
   return LP_OK;
 }
@@ -1587,7 +1595,7 @@ lp_status lp_align_aggregate(lp_ctx* c, int m, int64_t d, int k, lp_aggregator a
   LP_CUDA(cudaMemsetAsync(c->dStatus, 0, 4, c->stream));
   if ((st = check_launch(c, lp::launch_pack(dys, Yl, m, di, k, K, c->stream), "pack")) ||
       (st = check_launch(c, lp::launch_pack(dzs, Zl, m, di, k, K, c->stream), "pack")) ||
-      (st = check_launch(c, lp::launch_pack(dw, W, 1, m, 1, 1, c->stream), "pack")))
+      (st = check_launch(c, lp::launch_to_float(dw, W, m, c->stream), "pack")))
     return st;
   const bool align = agg != LP_AGG_IDENTITY;
   if (align && (st = check_launch(c, lp::launch_align(Zl, int64_t(d) * K, Zl + int64_t(d) * K * base, m, di, k, K, base,

@@ -182,6 +182,10 @@ inline void set_no_context_error(const std::string& msg) { set_no_context_error(
 // slots any partition has) picks how many threads share one output.
 cudaError_t launch_reduce(const float* P, const int* slot_begin, const float* scale, int m, int d, int K,
                           float* Y, cudaStream_t s, int max_slots);
+// The same sums as m blocks of d rows of k in FP64; *status_host (host memory the device can
+// write, may be nullptr) receives *status.
+cudaError_t launch_reduce_f64(const float* P, const int* slot_begin, const float* scale, int m, int d, int k, int K,
+                              double* Y, const int* status, int* status_host, cudaStream_t s, int max_slots);
 // Z_b = orth(Y_b) (CholQR2 on FP32 data), batch blocks of d x K.  kxk_fp64: the k x k
 // Gram and Cholesky in FP64; else FP32 with an FP64 Cholesky when a pivot is too small.
 cudaError_t launch_cholqr2(const float* Y, float* Z, int batch, int d, int k, int K, int* status, cudaStream_t s,
@@ -226,8 +230,11 @@ cudaError_t launch_lanczos_norms(const float* Mall, int nmat, int d, float* V, d
 int lanczos_steps(int d);
 size_t lanczos_smem(int d);
 
-// FP64 d x k (row-major) <-> FP32 d x K padded blocks
-cudaError_t launch_pack(const double* src, float* dst, int batch, int d, int k, int K, cudaStream_t s);
+// FP64 d x k (row-major) <-> FP32 d x K padded blocks (K a multiple of 4); pack also zeroes
+// *clear (may be nullptr)
+cudaError_t launch_pack(const double* src, float* dst, int batch, int d, int k, int K, cudaStream_t s,
+                        int* clear = nullptr);
+cudaError_t launch_to_float(const double* src, float* dst, int n, cudaStream_t s);
 cudaError_t launch_unpack(const float* src, double* dst, int batch, int d, int k, int K, cudaStream_t s);
 
 }  // namespace lp

@@ -96,20 +96,57 @@ __global__ void __launch_bounds__(kT) split_planes_kernel(const __grid_constant_
   }
 }
 
-__global__ void pack_kernel(const double* __restrict__ src, float* __restrict__ dst, int batch, int d, int k, int K) {
-  const int64_t total = int64_t(batch) * d * K;
-  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
-    const int j = static_cast<int>(e % K);
-    const int64_t row = e / K;  // b * d + c
-    dst[e] = j < k ? static_cast<float>(src[row * k + j]) : 0.f;
+// FP64 rows of k -> FP32 rows of K, zero beyond k; a thread converts four columns
+// of a row (K is a multiple of four).  `clear` (may be nullptr): a status word to
+// zero, for kernels later on the stream.
+__global__ void __launch_bounds__(kT) pack_kernel(const double* __restrict__ src, float* __restrict__ dst, int64_t rows,
+                                                  int k, int K, int* clear) {
+  if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0;
+  const int KQ = K / 4;
+  const bool vec = k % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+  const int64_t total = rows * KQ;
+  for (int64_t e = blockIdx.x * int64_t(kT) + threadIdx.x; e < total; e += int64_t(gridDim.x) * kT) {
+    const int64_t row = e / KQ;
+    const int j = 4 * static_cast<int>(e - row * KQ);
+    const double* p = src + row * k + j;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (vec && j + 4 <= k) {
+      const double2 x = reinterpret_cast<const double2*>(p)[0], y = reinterpret_cast<const double2*>(p)[1];
+      v = make_float4(static_cast<float>(x.x), static_cast<float>(x.y), static_cast<float>(y.x), static_cast<float>(y.y));
+    } else {
+      if (j < k) v.x = static_cast<float>(p[0]);
+      if (j + 1 < k) v.y = static_cast<float>(p[1]);
+      if (j + 2 < k) v.z = static_cast<float>(p[2]);
+      if (j + 3 < k) v.w = static_cast<float>(p[3]);
+    }
+    reinterpret_cast<float4*>(dst)[e] = v;
   }
 }
-__global__ void unpack_kernel(const float* __restrict__ src, double* __restrict__ dst, int batch, int d, int k, int K) {
-  const int64_t total = int64_t(batch) * d * k;
-  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
-    const int j = static_cast<int>(e % k);
-    const int64_t row = e / k;
-    dst[e] = static_cast<double>(src[row * K + j]);
+__global__ void to_float_kernel(const double* __restrict__ src, float* __restrict__ dst, int n) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < n) dst[e] = static_cast<float>(src[e]);
+}
+// The inverse: FP32 rows of K -> FP64 rows of k.
+__device__ __forceinline__ void store_f64(double* __restrict__ row, int j, int k, bool vec, float4 v) {
+  if (vec && j + 4 <= k) {
+    reinterpret_cast<double2*>(row + j)[0] = make_double2(v.x, v.y);
+    reinterpret_cast<double2*>(row + j)[1] = make_double2(v.z, v.w);
+  } else {
+    if (j < k) row[j] = v.x;
+    if (j + 1 < k) row[j + 1] = v.y;
+    if (j + 2 < k) row[j + 2] = v.z;
+    if (j + 3 < k) row[j + 3] = v.w;
+  }
+}
+__global__ void __launch_bounds__(kT) unpack_kernel(const float* __restrict__ src, double* __restrict__ dst,
+                                                    int64_t rows, int k, int K) {
+  const int KQ = K / 4;
+  const bool vec = k % 4 == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
+  const int64_t total = rows * KQ;
+  for (int64_t e = blockIdx.x * int64_t(kT) + threadIdx.x; e < total; e += int64_t(gridDim.x) * kT) {
+    const int64_t row = e / KQ;
+    const int j = 4 * static_cast<int>(e - row * KQ);
+    if (j < k) store_f64(dst + row * k, j, k, vec, reinterpret_cast<const float4*>(src)[e]);
   }
 }
 
@@ -119,10 +156,15 @@ __global__ void unpack_kernel(const float* __restrict__ src, double* __restrict_
 // its G partials by an xor butterfly.  The order is fixed for a given G, so
 // results are reproducible; G > 1 only when partitions have many slots (small
 // problems spread over many CTAs), where it cuts the chain of dependent loads.
-template <int G>
+// OUT64: the sums go to the caller's FP64 rows of k (the single power step, which
+// needs no FP32 copy: 128 blocks of 2,048 x 32, 18 + 25 us as two kernels), and the
+// first thread hands the status word to host memory.
+template <int G, bool OUT64>
 __global__ void reduce_kernel(const float* __restrict__ P, const int* __restrict__ slot_begin,
-                              const float* __restrict__ scale, int d, int K, float* __restrict__ Y) {
+                              const float* __restrict__ scale, int d, int K, float* __restrict__ Y,
+                              double* __restrict__ Yd, int k, const int* status, int* status_host) {
   const int i = blockIdx.y;
+  if (OUT64 && status_host && blockIdx.x == 0 && i == 0 && threadIdx.x == 0) *status_host = *status;
   const int64_t n4 = int64_t(d) * K / 4;
   const int g = threadIdx.x % G;
   const int64_t e = blockIdx.x * int64_t(blockDim.x / G) + threadIdx.x / G;
@@ -156,7 +198,13 @@ __global__ void reduce_kernel(const float* __restrict__ P, const int* __restrict
   if (!live || g != 0) return;
   const float sc = scale[i];
   acc.x *= sc; acc.y *= sc; acc.z *= sc; acc.w *= sc;
-  reinterpret_cast<float4*>(Y + int64_t(i) * d * K)[e] = acc;
+  if constexpr (OUT64) {
+    const int KQ = K / 4, row = static_cast<int>(e / KQ), j = 4 * static_cast<int>(e - int64_t(row) * KQ);
+    const bool vec = k % 4 == 0 && (reinterpret_cast<uintptr_t>(Yd) & 15) == 0;
+    if (j < k) store_f64(Yd + (int64_t(i) * d + row) * k, j, k, vec, acc);
+  } else {
+    reinterpret_cast<float4*>(Y + int64_t(i) * d * K)[e] = acc;
+  }
 }
 
 // ---------------------------------------------------------------- k x k helpers
@@ -770,37 +818,63 @@ cudaError_t launch_split_planes(const SplitParts& parts, int64_t src_ld, int d, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack(const double* src, float* dst, int batch, int d, int k, int K, cudaStream_t s) {
-  const int64_t total = int64_t(batch) * d * K;
-  const int64_t nb = (total + kT - 1) / kT;
-  const int blocks = static_cast<int>(nb < 4096 ? (nb > 0 ? nb : 1) : 4096);
-  pack_kernel<<<blocks, kT, 0, s>>>(src, dst, batch, d, k, K);
+namespace {
+unsigned rows_grid(int64_t total) {
+  return static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>((total + kT - 1) / kT, 152 * 16)));
+}
+}  // namespace
+
+cudaError_t launch_pack(const double* src, float* dst, int batch, int d, int k, int K, cudaStream_t s, int* clear) {
+  const int64_t rows = int64_t(batch) * d;
+  pack_kernel<<<rows_grid(rows * (K / 4)), kT, 0, s>>>(src, dst, rows, k, K, clear);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_to_float(const double* src, float* dst, int n, cudaStream_t s) {
+  to_float_kernel<<<(n + kT - 1) / kT, kT, 0, s>>>(src, dst, n);
   return cudaGetLastError();
 }
 
 cudaError_t launch_unpack(const float* src, double* dst, int batch, int d, int k, int K, cudaStream_t s) {
-  const int64_t total = int64_t(batch) * d * k;
-  const int64_t nb = (total + kT - 1) / kT;
-  const int blocks = static_cast<int>(nb < 4096 ? (nb > 0 ? nb : 1) : 4096);
-  unpack_kernel<<<blocks, kT, 0, s>>>(src, dst, batch, d, k, K);
+  const int64_t rows = int64_t(batch) * d;
+  unpack_kernel<<<rows_grid(rows * (K / 4)), kT, 0, s>>>(src, dst, rows, k, K);
   return cudaGetLastError();
 }
 
-cudaError_t launch_reduce(const float* P, const int* slot_begin, const float* scale, int m, int d, int K, float* Y,
-                          cudaStream_t s, int max_slots) {
+namespace {
+template <int G>
+cudaError_t launch_reduce_g(const float* P, const int* slot_begin, const float* scale, int m, int d, int K, float* Y,
+                            double* Yd, int k, const int* status, int* status_host, cudaStream_t s) {
   const int64_t n4 = int64_t(d) * K / 4;
+  const dim3 grid(static_cast<unsigned>((n4 + kT / G - 1) / (kT / G)), static_cast<unsigned>(m));
+  if (Yd) reduce_kernel<G, true><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y, Yd, k, status, status_host);
+  else reduce_kernel<G, false><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y, Yd, k, status, status_host);
+  return cudaGetLastError();
+}
+
+cudaError_t reduce_any(const float* P, const int* slot_begin, const float* scale, int m, int d, int K, float* Y,
+                       double* Yd, int k, const int* status, int* status_host, cudaStream_t s, int max_slots) {
   int G = 1;
   while (G < 32 && max_slots > 4 * G) G <<= 1;
-  dim3 grid(static_cast<unsigned>((n4 + kT / G - 1) / (kT / G)), static_cast<unsigned>(m));
   switch (G) {
-    case 1: reduce_kernel<1><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y); break;
-    case 2: reduce_kernel<2><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y); break;
-    case 4: reduce_kernel<4><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y); break;
-    case 8: reduce_kernel<8><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y); break;
-    case 16: reduce_kernel<16><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y); break;
-    default: reduce_kernel<32><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y); break;
+    case 1: return launch_reduce_g<1>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
+    case 2: return launch_reduce_g<2>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
+    case 4: return launch_reduce_g<4>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
+    case 8: return launch_reduce_g<8>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
+    case 16: return launch_reduce_g<16>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
+    default: return launch_reduce_g<32>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
   }
-  return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_reduce(const float* P, const int* slot_begin, const float* scale, int m, int d, int K, float* Y,
+                          cudaStream_t s, int max_slots) {
+  return reduce_any(P, slot_begin, scale, m, d, K, Y, nullptr, 0, nullptr, nullptr, s, max_slots);
+}
+
+cudaError_t launch_reduce_f64(const float* P, const int* slot_begin, const float* scale, int m, int d, int k, int K,
+                              double* Y, const int* status, int* status_host, cudaStream_t s, int max_slots) {
+  return reduce_any(P, slot_begin, scale, m, d, K, nullptr, Y, k, status, status_host, s, max_slots);
 }
 
 cudaError_t launch_align(const float* Zl, int64_t z_stride, const float* Zb, int m, int d, int k, int K, int base,
