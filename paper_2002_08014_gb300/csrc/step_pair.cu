@@ -38,8 +38,8 @@
 // round-robin, each into its own partial D1 that the epilogue sums in issuer
 // order, rank 1's take 128-column blocks round-robin, each block its own D2);
 // warps 8-11 (one per TMEM lane quadrant) run the epilogue; on rank 1, warp 5
-// lane 0 recycles W buffers; on rank 0 all warps stage Z when the partition
-// changes.  Every wait is bounded: on expiry the CTA records
+// lane 0 recycles W buffers; on rank 0 all warps but the producer's stage Z when the
+// partition changes, while the producer fills the ring for it.  Every wait is bounded: on expiry the CTA records
 // ST_TIMEOUT, stops issuing, waits (bounded) for its own copies in flight and
 // for W copies addressed to it, retires its MMAs, frees tensor memory and
 // returns; the partner's own bounded waits then expire the same way.
@@ -276,33 +276,28 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     constexpr uint32_t idesc1 = idesc_bf16(128, N, false, false);
     const int DC = 64 * a.ncd;
     uint32_t c_mma = 0, T_epi = 0, T_mma = 0, epi_phase = 0, sent = 0, run = 0;
-    bool prod_ok = true;
     int si = sb;
-    const uint64_t pol = a.hints ? l2_policy_evict_last() : 0;
-    while (si < se) {
+    // The producer runs through all segments on its own: the ring is full again by the
+    // time the other warps have restaged Z for the next partition.
+    if (warp == 0 && lane == 0) {
+      produce(sb, se, a.hints ? l2_policy_evict_last() : 0, a.prefetch);
+      drain_ring();
+    }
+    constexpr int kOthers = kPairThreads - 32;
+    while (warp != 0 && si < se) {
       // a run: consecutive segments of one partition share Z_i
       const int part = a.segs[si].part;
       int sj = si + 1;
       while (sj < se && a.segs[sj].part == part) ++sj;
-      __syncthreads();  // every role finished the previous run (its MMAs retired: ZDRAIN)
-      if (*abort_flag) break;
-      if (run == 0 || a.z_stride != 0) {
-        const float* Zg = a.Z + a.z_stride * part;
-        for (int e = tid; e < DC * K; e += kPairThreads) {
-          const int c = e / K, j = e % K;
-          const float z = c < a.d ? Zg[static_cast<int64_t>(c) * K + j] : 0.f;
-          const uint16_t hi = bf16_bits(z);
-          const uint16_t lo = bf16_bits(z - bf16_val(hi));
-          *reinterpret_cast<uint16_t*>(sZ + sw128_off(j, c, N)) = hi;
-          *reinterpret_cast<uint16_t*>(sZ + sw128_off(K + j, c, N)) = lo;
-        }
-      }
+      __syncwarp();
+      // every role finished the previous run (its MMAs retired: ZDRAIN); all leave together after an abort
+      if (bar_or(1, kOthers, *abort_flag != 0)) break;
+      if (run == 0 || a.z_stride != 0)
+        stage_z<K, Bf16Op>(sZ, a.Z + a.z_stride * part, 0, DC, a.d, tid - 32, kOthers);
       fence_async_smem();
-      __syncthreads();
+      bar_sync(1, kOthers);
 
-      if (warp == 0 && lane == 0) {
-        if (prod_ok) prod_ok = produce(si, sj, pol, a.prefetch);
-      } else if (issuer && h < HE) {
+      if (issuer && h < HE) {
         // ------------------------------------------------ MMA issuers, pass 1: issuer h takes units
         // u = h, h + HE, ... of every tile into its partial D1[buf][h]
         const int u_last = h + ((U - 1 - h) / HE) * HE;
@@ -399,7 +394,6 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       ++run;
       si = sj;
     }
-    if (warp == 0 && lane == 0) drain_ring();
     if (warp == kEpiWarp0 && lane == 0) st_cluster_u32(mapa(su32(const_cast<uint32_t*>(sent_slot)), 1), sent);
   } else {
     // ===================================================================== rank 1: Y += A_t^T W

@@ -200,5 +200,53 @@ __device__ __forceinline__ uint32_t sw128_off(int n, int kk, int rows) {
 __device__ __forceinline__ uint16_t bf16_bits(float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); }
 __device__ __forceinline__ float bf16_val(uint16_t b) { return __uint_as_float(static_cast<uint32_t>(b) << 16); }
 
+// The 16-bit operand types of the step kernels: the bits of rn(x) and its value.
+struct Bf16Op {
+  static __device__ __forceinline__ uint16_t bits(float x) { return bf16_bits(x); }
+  static __device__ __forceinline__ float val(uint16_t b) { return bf16_val(b); }
+};
+
+// [Z_hi | Z_lo]^T of columns c0 .. c0 + dc - 1 of Z (d x K, FP32; zero beyond d) as a
+// K-major SWIZZLE_128B operand of 2 K rows, hi = rn(z), lo = rn(z - hi), by threads
+// t = 0 .. n - 1.  A thread takes eight consecutive columns at one j: eight loads in
+// flight, contiguous over the lanes' j, and one 16-byte store per half (a row's
+// eight columns are one swizzle atom, so eight rows hit eight bank groups).
+// Element by element, the same staging of 1,024 x 16 took about 6 us of 2-byte
+// stores behind dependent loads, at every partition a CTA works on.
+template <int K, typename Op>
+__device__ __forceinline__ void stage_z(unsigned char* s, const float* __restrict__ Z, int c0, int dc, int d, int t, int n) {
+  constexpr int N = 2 * K;
+#pragma unroll 2
+  for (int e = t; e < dc / 8 * K; e += n) {
+    const int j = e % K, c = e / K * 8;
+    float z[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) z[q] = c0 + c + q < d ? Z[static_cast<int64_t>(c0 + c + q) * K + j] : 0.f;
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint16_t h0 = Op::bits(z[2 * q]), h1 = Op::bits(z[2 * q + 1]);
+      hi[q] = h0 | (static_cast<uint32_t>(h1) << 16);
+      lo[q] = Op::bits(z[2 * q] - Op::val(h0)) | (static_cast<uint32_t>(Op::bits(z[2 * q + 1] - Op::val(h1))) << 16);
+    }
+    *reinterpret_cast<uint4*>(s + sw128_off(j, c, N)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(s + sw128_off(K + j, c, N)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+  }
+}
+
+// Barrier `id` over n threads (whole warps); and the same with the OR of a flag over them.
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ bool bar_or(int id, int n, bool flag) {
+  uint32_t r;
+  asm volatile(
+      "{ .reg .pred p, q; setp.ne.u32 q, %3, 0;\n\t"
+      "bar.red.or.pred p, %1, %2, q;\n\t"
+      "selp.u32 %0, 1, 0, p; }"
+      : "=r"(r)
+      : "r"(id), "r"(n), "r"(flag ? 1u : 0u)
+      : "memory");
+  return r != 0;
+}
+
 }  // namespace tc
 }  // namespace lp
