@@ -121,6 +121,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_rank();
   const int cluster_id = blockIdx.x >> 1;
+  // the segment range, loaded while the barriers and tensor memory are set up
+  const int sb = a.seg_ptr[cluster_id], se = a.seg_ptr[cluster_id + 1];
   const int NB = a.ncd / 2;
   const int U = NB * PL;
   const int R = rank == 0 ? a.ring0 : a.ring1;
@@ -197,11 +199,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     }
   };
 
-  const int sb = a.seg_ptr[cluster_id], se = a.seg_ptr[cluster_id + 1];
   auto tiles_of = [&](int s) { return static_cast<int>((a.segs[s].row1 - a.segs[s].row0 + kBM - 1) / kBM); };
-  uint32_t total_tiles = 0;
-  for (int s = sb; s < se; ++s) total_tiles += static_cast<uint32_t>(tiles_of(s));
-
   // TMA producer over the segments [s0, s1): every unit of every tile, in order,
   // each into the next slot of the issuer that consumes it, optionally bringing
   // the unit PF places ahead into L2 first.  pcnt[h] counts the units dealt to
@@ -444,6 +442,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       consumed_slot[h] = consumed;
     } else if (warp == kRecycler && lane == 0) {
       // ------------------------------------------------ W buffer recycler
+      uint32_t total_tiles = 0;
+      for (int s = sb; s < se; ++s) total_tiles += static_cast<uint32_t>(tiles_of(s));
       for (uint32_t b = 0; b < 2 && b < total_tiles; ++b) {
         mbar_expect_tx(&bar[R1_B2FULL + b], B2BUF);
         mbar_arrive_remote(mapa(su32(&bar[R0_B2FREE + b]), 0));

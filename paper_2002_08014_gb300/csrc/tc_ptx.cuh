@@ -208,30 +208,50 @@ struct Bf16Op {
 
 // [Z_hi | Z_lo]^T of columns c0 .. c0 + dc - 1 of Z (d x K, FP32; zero beyond d) as a
 // K-major SWIZZLE_128B operand of 2 K rows, hi = rn(z), lo = rn(z - hi), by threads
-// t = 0 .. n - 1.  A thread takes eight consecutive columns at one j: eight loads in
-// flight, contiguous over the lanes' j, and one 16-byte store per half (a row's
-// eight columns are one swizzle atom, so eight rows hit eight bank groups).
-// Element by element, the same staging of 1,024 x 16 took about 6 us of 2-byte
-// stores behind dependent loads, at every partition a CTA works on.
+// t = 0 .. n - 1.  A thread takes eight consecutive columns at J values of j: eight
+// loads in flight, contiguous over the lanes' j, and one 16-byte store per j and half
+// (a row's eight columns are one swizzle atom).  Element by element, the same staging
+// of 1,024 x 16 took about 16 us of 2-byte stores behind dependent loads, at every
+// partition a CTA works on; with J = 1 4.5 us, with J = 4 (16-byte loads) 3.4.  J = 1
+// spreads a small block over more threads (128 x 16: 11.9 us a launch against 12.3).
+template <int K, int J, typename Op>
+__device__ __forceinline__ void stage_z_items(unsigned char* s, const float* __restrict__ Z, int c0, int dc, int d, int t,
+                                              int n) {
+  constexpr int N = 2 * K, KJ = K / J;
+#pragma unroll(J == 1 ? 2 : 1)
+  for (int e = t; e < dc / 8 * KJ; e += n) {
+    const int j = e % KJ * J, c = e / KJ * 8;
+    float z[8][J];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float* p = Z + static_cast<int64_t>(c0 + c + q) * K + j;
+      const bool in = c0 + c + q < d;
+      if constexpr (J == 4) {
+        const float4 v = in ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+        z[q][0] = v.x; z[q][1] = v.y; z[q][2] = v.z; z[q][3] = v.w;
+      } else {
+        z[q][0] = in ? *p : 0.f;
+      }
+    }
+#pragma unroll
+    for (int jj = 0; jj < J; ++jj) {
+      uint32_t hi[4], lo[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float z0 = z[2 * q][jj], z1 = z[2 * q + 1][jj];
+        const uint16_t h0 = Op::bits(z0), h1 = Op::bits(z1);
+        hi[q] = h0 | (static_cast<uint32_t>(h1) << 16);
+        lo[q] = Op::bits(z0 - Op::val(h0)) | (static_cast<uint32_t>(Op::bits(z1 - Op::val(h1))) << 16);
+      }
+      *reinterpret_cast<uint4*>(s + sw128_off(j + jj, c, N)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+      *reinterpret_cast<uint4*>(s + sw128_off(K + j + jj, c, N)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    }
+  }
+}
 template <int K, typename Op>
 __device__ __forceinline__ void stage_z(unsigned char* s, const float* __restrict__ Z, int c0, int dc, int d, int t, int n) {
-  constexpr int N = 2 * K;
-#pragma unroll 2
-  for (int e = t; e < dc / 8 * K; e += n) {
-    const int j = e % K, c = e / K * 8;
-    float z[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) z[q] = c0 + c + q < d ? Z[static_cast<int64_t>(c0 + c + q) * K + j] : 0.f;
-    uint32_t hi[4], lo[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint16_t h0 = Op::bits(z[2 * q]), h1 = Op::bits(z[2 * q + 1]);
-      hi[q] = h0 | (static_cast<uint32_t>(h1) << 16);
-      lo[q] = Op::bits(z[2 * q] - Op::val(h0)) | (static_cast<uint32_t>(Op::bits(z[2 * q + 1] - Op::val(h1))) << 16);
-    }
-    *reinterpret_cast<uint4*>(s + sw128_off(j, c, N)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-    *reinterpret_cast<uint4*>(s + sw128_off(K + j, c, N)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-  }
+  if (dc / 8 * K <= 2 * n) stage_z_items<K, 1, Op>(s, Z, c0, dc, d, t, n);
+  else stage_z_items<K, 4, Op>(s, Z, c0, dc, d, t, n);
 }
 
 // Barrier `id` over n threads (whole warps); and the same with the OR of a flag over them.
