@@ -176,16 +176,9 @@ constexpr int kDefaultTcKernel = LP_KERNEL_PAIR;
 // lp_stats::path code of the pass-split pair kernel (it shares PATH_TCS's tables).
 constexpr int kReportedPathPair = 3;
 
-// Tensor-core step kernels accumulate a segment's A^T W in TMEM, and the tensor
-// cores round that FP32 accumulator toward zero on every MMA, so a long chain
-// shrinks the result a little (about half an ulp per MMA).  Their segments are
-// cut into pieces of at most this many rows (32 tiles, 256 accumulating MMAs
-// per entry); the reduction adds the pieces with round-to-nearest.
-constexpr int64_t kTcChainRows = 4096;
-
 // Most segments any step kernel's table can have for `workers` workers: each
 // worker's row range is cut at partition ends and into kTcChainRows pieces.
-int64_t max_segments(int64_t workers, int64_t m, int64_t n) { return workers + m + n / kTcChainRows + 1; }
+int64_t max_segments(int64_t workers, int64_t m, int64_t n) { return workers + m + n / lp::kTcChainRows + 1; }
 
 // Launches of the SIMT step per local step (0: no SIMT kernel for the shape).
 int simt_launches(int d, int64_t ld, lp_dtype dtype, int K) {
@@ -551,7 +544,7 @@ static lp_status setup_partitions(lp_ctx* c, int m, const int64_t* rows, int64_t
   if (dtype == LP_BF16 && lp::tc_plan(static_cast<int>(d), LP_MAX_K, c->sms, &c->tc)) {
     const int G = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(c->tc.nclusters, (n + 127) / 128)));
     c->tc.nclusters = G;
-    build_segments(c, G, segs_tc, seg_ptr_tc, slot_begin_tc, kTcChainRows);
+    build_segments(c, G, segs_tc, seg_ptr_tc, slot_begin_tc, lp::kTcChainRows);
     c->nslots_tc = static_cast<int>(segs_tc.size());
     c->max_slots[PATH_TC] = max_slots_in(slot_begin_tc);
     c->tc_ready = true;
@@ -892,7 +885,7 @@ static lp_status ensure_tcs(lp_ctx* c, int k) {
   if (G != c->tcs_G) {
     std::vector<Segment> segs;
     std::vector<int> seg_ptr, slot_begin;
-    build_segments(c, G, segs, seg_ptr, slot_begin, kTcChainRows);
+    build_segments(c, G, segs, seg_ptr, slot_begin, lp::kTcChainRows);
     lp_status st;
     if (!c->dSegsTcs &&
         ((st = dalloc(c, &c->dSegsTcs, size_t(max_segments(c->sms, c->m, c->n)) * sizeof(Segment))) ||

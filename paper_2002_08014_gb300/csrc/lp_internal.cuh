@@ -25,6 +25,15 @@ struct Segment {
   int slot;            // output slot of the CTA's partial A_i^T A_i Z_i
 };
 
+// Tensor-core step kernels accumulate a segment's A^T W in TMEM, and the tensor
+// cores round that FP32 accumulator toward zero on every MMA, so a long chain
+// shrinks the result a little (about half an ulp per MMA).  Their segments are
+// cut into pieces of at most this many rows (32 tiles, 256 accumulating MMAs
+// per entry); the reduction adds the pieces with round-to-nearest.  A whole number
+// of 128-row tiles: the pieces of a partition that one worker owns follow each
+// other tile by tile.
+constexpr int64_t kTcChainRows = 4096;
+
 // Lets every launch of `kern` request up to the device's opt-in shared memory per
 // block, less the kernel's static shared memory (once per kernel).  The limit is
 // a property of the function, not of a launch: set to each plan's own size, a

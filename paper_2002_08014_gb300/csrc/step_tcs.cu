@@ -26,7 +26,8 @@
 // 128-column blocks (both planes of a block) with its own partial D1 (the
 // epilogue sums the two in issuer order) and its own part of the ring, so that
 // it consumes its slots strictly in order; warps 4-7 (one per TMEM lane
-// quadrant) run the epilogue; all warps stage Z at segment starts.  Every wait is bounded: on expiry the kernel records
+// quadrant) run the epilogue; all warps but the producer's stage Z when the partition
+// changes.  Every wait is bounded: on expiry the kernel records
 // ST_TIMEOUT, stops issuing, waits (bounded) for its own copies in flight,
 // frees tensor memory and returns.
 #include "lp_internal.cuh"
@@ -42,7 +43,7 @@ constexpr int kMaxRing = 8;
 constexpr int kSmemLimit = 232448;
 
 enum TcsBar { S_D1FULL0 = 0, S_D1EMPTY0 = 2, S_B2FULL0 = 4, S_B2FREE0 = 6, S_D2FULL = 8, S_REDFULL = 9,
-              S_WFULL = 10, S_DONE = 11, S_EPI = 12, S_RING0 = 13 };  // ring: FULL[s] = S_RING0 + s, EMPTY[s] = S_RING0 + ring + s
+              S_WFULL = 10, S_DONE = 11, S_EPI = 12, S_D2EMPTY = 13, S_RING0 = 14 };  // ring: FULL[s] = S_RING0 + s, EMPTY[s] = S_RING0 + ring + s
 
 struct TcsArgs {
   const Segment* segs;
@@ -118,6 +119,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&bar[S_B2FREE0 + s], HE);
     }
     mbar_init(&bar[S_D2FULL], HE);
+    mbar_init(&bar[S_D2EMPTY], 4);
     mbar_init(&bar[S_REDFULL], 1);
     mbar_init(&bar[S_WFULL], 1);
     mbar_init(&bar[S_DONE], 2);  // both issuer threads commit (an idle one at once)
@@ -161,33 +163,42 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr uint32_t idesc1 = idesc_bf16(128, N, false, false);
   constexpr uint32_t idesc2 = idesc_bf16(128, N, true, false);
 
+  // A run: the consecutive pieces of one partition that this cluster owns.  They share
+  // Z_i and their rows follow each other, every piece but the last a whole number of
+  // tiles (TP), so a run is one stream of tiles; the accumulation of A^T W starts anew
+  // at each piece.  The producer goes through all runs without stopping; the other
+  // warps meet between runs, when Z is restaged.
+  constexpr int TP = static_cast<int>(kTcChainRows / kBM);
+  static_assert(kTcChainRows % kBM == 0, "pieces are whole tiles");
+  constexpr int kOthers = kThreads - 32;
   const int sb = a.seg_ptr[cluster_id], se = a.seg_ptr[cluster_id + 1];
-  uint32_t T = 0;  // tiles before this segment (same in every CTA of the cluster)
+  uint32_t T = 0;  // tiles before this run (same in every CTA of the cluster)
+  uint32_t pieces = 0;     // pieces before this run
   uint32_t epi_phase = 0;  // uses of the epilogue barrier so far (epilogue threads)
   uint32_t pcnt[2] = {0u, 0u};  // producer: units dealt to each issuer so far
   uint32_t fills[kMaxRing] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};  // producer: fills of each slot
   uint32_t c_own = 0;           // issuer: own units consumed so far
-  for (int si = sb; si < se; ++si) {
+  bool prod_ok = true;
+  for (int si = sb, sj; si < se; si = sj) {
     const Segment sg = a.segs[si];
-    const int ntiles = static_cast<int>((sg.row1 - sg.row0 + kBM - 1) / kBM);
+    sj = si + 1;
+    while (sj < se && a.segs[sj].part == sg.part) ++sj;
+    const int64_t run_end = a.segs[sj - 1].row1;
+    const int ntiles = static_cast<int>((run_end - sg.row0 + kBM - 1) / kBM);
 
-    // ---- stage this slice of Z as [Z_hi | Z_lo]^T (N rows x DC, K-major, SWIZZLE_128B)
-    __syncthreads();
-    if (si == sb || sg.part != a.segs[si - 1].part) {  // consecutive pieces of a partition share Z_i
-      const float* Zg = a.Z + a.z_stride * sg.part;
-      for (int e = tid; e < DC * K; e += kThreads) {
-        const int c = e / K, j = e % K;
-        const float z = (c0 + c < a.d) ? Zg[static_cast<int64_t>(c0 + c) * K + j] : 0.f;
-        const uint16_t hi = bf16_bits(z);
-        const uint16_t lo = bf16_bits(z - bf16_val(hi));
-        *reinterpret_cast<uint16_t*>(sB1 + sw128_off(j, c, N)) = hi;
-        *reinterpret_cast<uint16_t*>(sB1 + sw128_off(K + j, c, N)) = lo;
-      }
+    if (warp != 0) {
+      __syncwarp();
+      // every role finished the previous run; all leave together after an abort
+      if (bar_or(1, kOthers, *abort_flag != 0)) break;
+      // this slice of Z as [Z_hi | Z_lo]^T (N rows x DC, K-major, SWIZZLE_128B)
+      if (si == sb || a.z_stride != 0)
+        stage_z<K, Bf16Op>(sB1, a.Z + a.z_stride * sg.part, c0, DC, a.d, tid - 32, kOthers);
+      fence_async_smem();
+      bar_sync(1, kOthers);
     }
-    fence_async_smem();
-    __syncthreads();
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
+      if (lane == 0 && prod_ok) {
       // ------------------------------------------------------------ TMA producer
       uint64_t pol_keep = 0, pol_drop = 0;
       if (a.hints) {
@@ -201,7 +212,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int j = 0; j < 2; ++j)
           tma_prefetch_2d(pl2 ? &map1 : &map0, c0 + 64 * (2 * b2 + j), static_cast<int>(sg.row0) + t2 * kBM);
       }
-      for_each_unit(ntiles, U, LAG, [&](bool second, int t, int u) -> bool {
+      prod_ok = for_each_unit(ntiles, U, LAG, [&](bool second, int t, int u) -> bool {
         // the next slot of the issuer that consumes this unit
         const int hh = (u / PL) % HE;
         const uint32_t k = pcnt[hh], RH = static_cast<uint32_t>(ring_len(hh));
@@ -230,14 +241,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         return true;
       });
-      // Copies still in flight (only after an abort) land before the CTA exits:
-      // the last fill of every slot (earlier fills were waited for by then).
-      for (int q = 0; q < R; ++q) {
-        if (fills[q] == 0) continue;
-        const uint32_t addr = su32(&bar[S_RING0 + q]);
-        const long long t0 = clock64();
-        while (!mbar_try(addr, (fills[q] - 1) & 1) && clock64() - t0 < kTimeoutCycles) {
-        }
       }
     } else if (issuer && h < HE) {
       // ------------------------------------------------------------ MMA issuers
@@ -253,6 +256,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (u == u_first) {
           if (!second && !wait(S_D1EMPTY0 + buf, ((Tg >> 1) + 1) & 1, false)) return false;
           if (second && !wait(S_B2FULL0 + buf, (Tg >> 1) & 1, false)) return false;
+          // a new piece accumulates from zero: the previous one's sums have been read out
+          if (second && t % TP == 0 && !wait(S_D2EMPTY, (pieces + t / TP + 1) & 1, false)) return false;
         }
         tc_fence_after();
         const int b = u / PL, pl = u % PL;
@@ -276,14 +281,16 @@ __global__ void __launch_bounds__(kThreads, 1)
             // A^T: M = 128 columns (two 64-column chunks, LBO apart), K = 16 rows (two 8-row groups, SBO apart)
             const uint64_t ad = sdesc(aS + kk * 2048, kChunkBytes, 1024);
             const uint64_t bd = sdesc(bS + (kk >> 2) * N * 128 + (kk & 3) * 32, 16, 1024);
-            mma_bf16(tmem + 2 * HE * N + b * N, ad, bd, idesc2, (t == 0 && pl == 0 && kk == 0) ? 0u : 1u);
+            mma_bf16(tmem + 2 * HE * N + b * N, ad, bd, idesc2, (t % TP == 0 && pl == 0 && kk == 0) ? 0u : 1u);
           }
           mma_commit(&bar[S_RING0 + R + s]);
-          if (u == u_last) mma_commit(&bar[S_B2FREE0 + buf]);
+          if (u == u_last) {
+            mma_commit(&bar[S_B2FREE0 + buf]);
+            if (t % TP == TP - 1 || t == ntiles - 1) mma_commit(&bar[S_D2FULL]);
+          }
         }
         return true;
       });
-      mma_commit(&bar[S_D2FULL]);
     } else if (warp >= 4) {
       // ------------------------------------------------------------ epilogue
       const int r = (warp - 4) * 32 + lane;
@@ -318,7 +325,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar[S_D1EMPTY0 + buf]);
-        const bool valid = sg.row0 + static_cast<int64_t>(t) * kBM + r < sg.row1;
+        const bool valid = sg.row0 + static_cast<int64_t>(t) * kBM + r < run_end;
         if (!valid) {
 #pragma unroll
           for (int j = 0; j < K; ++j) w[j] = 0.f;
@@ -390,11 +397,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         fence_async_smem();
         mbar_arrive(&bar[S_B2FULL0 + buf]);
-      }
-      // segment end: Y slice = D2[:, :K] + D2[:, K:] -> P[slot]
-      if (ok && wait(S_D2FULL, (si - sb) & 1, false)) {
+        if (t % TP != TP - 1 && t != ntiles - 1) continue;
+        // piece end: Y slice = D2[:, :K] + D2[:, K:] -> P[slot]
+        const int piece = t / TP;
+        if (!(ok = wait(S_D2FULL, (pieces + piece) & 1, false))) break;
         tc_fence_after();
-        float* Pd = a.P + static_cast<int64_t>(sg.slot) * a.d * K;
+        float* Pd = a.P + static_cast<int64_t>(a.segs[si + piece].slot) * a.d * K;
         for (int b = 0; b < NB; ++b) {
           float y[K];
 #pragma unroll
@@ -416,11 +424,25 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
         tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar[S_D2EMPTY]);
       }
     }
     T += ntiles;
+    pieces += (ntiles + TP - 1) / TP;
   }
 
+  // Copies still in flight (only after an abort) land before the CTA exits: the last
+  // fill of every slot (earlier fills were waited for by then).
+  if (warp == 0 && lane == 0) {
+    for (int q = 0; q < R; ++q) {
+      if (fills[q] == 0) continue;
+      const uint32_t addr = su32(&bar[S_RING0 + q]);
+      const long long t0 = clock64();
+      while (!mbar_try(addr, (fills[q] - 1) & 1) && clock64() - t0 < kTimeoutCycles) {
+      }
+    }
+  }
   // ---- teardown: all MMAs retired, no remote traffic in flight, then free TMEM
   if (issuer) mma_commit(&bar[S_DONE]);
   __syncthreads();
