@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar + kNumBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
   volatile uint32_t* sent_slot = tmem_holder + 2;      // rank 1: W copies rank 0 issued (written by rank 0)
+  volatile uint32_t* issued = tmem_holder + 3;         // units the producer has issued
   volatile uint32_t* consumed_slot = tmem_holder + 4;  // rank 1, per issuer: W buffers whose arrival it waited for
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -127,16 +128,15 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   const int U = NB * PL;
   const int R = rank == 0 ? a.ring0 : a.ring1;
   const uint32_t tmem_cols = rank == 0 ? a.tmem0 : a.tmem1;
-  // Active issuers: rank 0 deals units round-robin, rank 1 deals 128-column blocks.
-  // The ring's slots are dealt to the issuers as well: issuer h owns slots
-  // [h * RH, (h + 1) * RH) and consumes its units strictly in order, so no thread
-  // ever waits on a slot phase more than one past the slot's last completed
-  // phase (an mbarrier parity wait further ahead would succeed at once).
+  // Active issuers: rank 0 deals units round-robin, rank 1 deals 128-column blocks; the
+  // units go through the ring's slots in order, whoever consumes them.  An issuer that
+  // skips the others' units could meet a slot one fill early, where an mbarrier parity
+  // wait succeeds at once on the fill before; so it first waits until the producer has
+  // issued its unit, which it does only after the slot's previous fill was consumed.
+  // (Slots dealt to the issuers left one of five or two of six unused at d = 512.)
   const int HE = rank == 0 ? min(min(U, kIssuers), R) : min(min(NB, kIssuers1), R);
-  const int RH = R / HE;
   const int h = warp - 1;  // issuer index on warps 1 .. kIssuers
   const bool issuer = lane == 0 && warp >= 1 && warp <= kIssuers;
-  auto issuer_of = [&](int u) { return rank == 0 ? u % HE : (u / PL) % HE; };
 
   if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
@@ -158,6 +158,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     }
     *abort_flag = 0;
     *sent_slot = 0;
+    *issued = 0;
     for (int i = 0; i < kIssuers; ++i) consumed_slot[i] = 0;
     fence_mbar_init();
   }
@@ -192,6 +193,29 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       }
     }
   };
+  auto wait_issued = [&](uint32_t g) -> bool {
+    const long long t0 = clock64();
+    while (*issued <= g) {
+      if (*abort_flag) return false;
+      if (clock64() - t0 > kTimeoutCycles) {
+        give_up();
+        return false;
+      }
+    }
+    return true;
+  };
+  // An issuer's place in the unit order: unit g sits in slot (g mod R), its fill's parity
+  // is that of g / R.
+  uint32_t at_g = 0, at_slot = 0, at_phase = 0;
+  auto unit_ready = [&](uint32_t g) -> bool {
+    at_slot += g - at_g;
+    at_g = g;
+    while (at_slot >= static_cast<uint32_t>(R)) {
+      at_slot -= R;
+      at_phase ^= 1;
+    }
+    return (HE == 1 || wait_issued(g)) && wait(B_RING0 + at_slot, at_phase, false);
+  };
   auto bounded_drain = [&](int id, uint32_t parity) {
     const uint32_t addr = su32(&bar[id]);
     const long long t0 = clock64();
@@ -200,13 +224,10 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   };
 
   auto tiles_of = [&](int s) { return static_cast<int>((a.segs[s].row1 - a.segs[s].row0 + kBM - 1) / kBM); };
-  // TMA producer over the segments [s0, s1): every unit of every tile, in order,
-  // each into the next slot of the issuer that consumes it, optionally bringing
-  // the unit PF places ahead into L2 first.  pcnt[h] counts the units dealt to
-  // issuer h, fills[s] the fills of slot s.  Returns false after an abort.
-  uint32_t pcnt[kIssuers] = {0u, 0u, 0u, 0u};
-  uint32_t issued_total = 0;
-  uint32_t fills[kMaxRing] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+  // TMA producer over the segments [s0, s1): every unit of every tile, in order, each
+  // into the next slot, optionally bringing the unit PF places ahead into L2 first.
+  // Returns false after an abort.
+  uint32_t issued_total = 0, p_slot = 0, p_phase = 0;
   auto produce = [&](int s0, int s1, uint64_t policy, int PF) -> bool {
     for (int s = s0; s < s1; ++s) {
       const Segment sg = a.segs[s];
@@ -224,12 +245,12 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       for (int t = 0; t < nt; ++t)
         for (int u = 0; u < U; ++u) {
           if (PF > 0 && t * U + u + PF < nt * U) prefetch_unit(t * U + u + PF);
-          const int hh = issuer_of(u);
-          const uint32_t k = pcnt[hh];
-          const uint32_t slot = static_cast<uint32_t>(hh * RH) + k % RH;
-          if (!wait(B_RING0 + kMaxRing + slot, ((k / RH) + 1) & 1, false)) return false;
-          pcnt[hh] = k + 1;
-          ++fills[slot];
+          const uint32_t slot = p_slot;
+          if (!wait(B_RING0 + kMaxRing + slot, p_phase ^ 1, false)) return false;
+          if (++p_slot == static_cast<uint32_t>(R)) {
+            p_slot = 0;
+            p_phase ^= 1;
+          }
           mbar_expect_tx(&bar[B_RING0 + slot], kUnitBytes);
           issued_total += 1;
           const int b = u / PL, pl = u % PL;
@@ -247,6 +268,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
               else tma_load_2d(dst, map, 64 * (2 * b + j), row, &bar[B_RING0 + slot]);
             }
           }
+          *issued = issued_total;
           // Test hook: after rank 0's first ring fill (copies in flight, MMAs started),
           // a wait that nothing can complete runs out its short limit and aborts.
           if (a.stall > 0 && rank == 0 && issued_total == static_cast<uint32_t>(R)) {
@@ -265,15 +287,15 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   // After an abort: copies still in flight land before the CTA's shared memory
   // goes (the last fill of every slot; earlier fills were waited for by then).
   auto drain_ring = [&]() {
-    for (int q = 0; q < HE * RH; ++q)
-      if (fills[q] > 0) bounded_drain(B_RING0 + q, (fills[q] - 1) & 1);
+    for (uint32_t g = issued_total > static_cast<uint32_t>(R) ? issued_total - R : 0; g < issued_total; ++g)
+      bounded_drain(B_RING0 + g % R, (g / R) & 1);
   };
 
   if (rank == 0) {
     // ===================================================================== rank 0: W = A_t Z
     constexpr uint32_t idesc1 = idesc_bf16(128, N, false, false);
     const int DC = 64 * a.ncd;
-    uint32_t c_mma = 0, T_epi = 0, T_mma = 0, epi_phase = 0, sent = 0, run = 0;
+    uint32_t T_epi = 0, T_mma = 0, epi_phase = 0, sent = 0, run = 0;
     int si = sb;
     // The producer runs through all segments on its own: the ring is full again by the
     // time the other warps have restaged Z for the next partition.
@@ -305,9 +327,9 @@ __global__ void __launch_bounds__(kPairThreads, 1)
           for (int t = 0; ok && t < nt; ++t, ++T_mma) {
             const uint32_t buf = T_mma & 1;
             if (!(ok = wait(R0_D1EMPTY + buf, ((T_mma >> 1) + 1) & 1, false))) break;
-            for (int u = h; u < U; u += HE, ++c_mma) {
-              const uint32_t slot = static_cast<uint32_t>(h * RH) + c_mma % RH;
-              if (!(ok = wait(B_RING0 + slot, (c_mma / RH) & 1, false))) break;
+            for (int u = h; u < U; u += HE) {
+              if (!(ok = unit_ready(T_mma * U + u))) break;
+              const uint32_t slot = at_slot;
               tc_fence_after();
               const int b = u / PL;
               const uint32_t aS = su32(sRing + slot * kUnitBytes);
@@ -405,16 +427,16 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       const int b_last = h + ((NB - 1 - h) / HE) * HE;
       const int u_first = h * PL, u_last = b_last * PL + PL - 1;
       bool ok = true;
-      uint32_t c = 0, T = 0, consumed = 0;
+      uint32_t T = 0, consumed = 0;
       for (int s = sb, pi = 0; ok && s < se; ++s, ++pi) {
         const int pb = pi % a.nd2;
         const uint32_t use = static_cast<uint32_t>(pi / a.nd2);
         const int nt = tiles_of(s);
         for (int t = 0; ok && t < nt; ++t, ++T) {
           const uint32_t buf = T & 1;
-          for (int u = u_first; u <= u_last; u = ((u % PL) == PL - 1) ? u + (HE - 1) * PL + 1 : u + 1, ++c) {
-            const uint32_t slot = static_cast<uint32_t>(h * RH) + c % RH;
-            if (!(ok = wait(B_RING0 + slot, (c / RH) & 1, false))) break;
+          for (int u = u_first; u <= u_last; u = ((u % PL) == PL - 1) ? u + (HE - 1) * PL + 1 : u + 1) {
+            if (!(ok = unit_ready(T * U + u))) break;
+            const uint32_t slot = at_slot;
             if (u == u_first) {
               if (!(ok = wait(R1_B2FULL + buf, (T >> 1) & 1, true))) break;
               consumed = T + 1;

@@ -24,8 +24,9 @@
 // MMAs (two issuers: one thread issues a small-N MMA only every ~55 cycles, and
 // every ~100 when it polls barriers between MMAs), each owning alternate
 // 128-column blocks (both planes of a block) with its own partial D1 (the
-// epilogue sums the two in issuer order) and its own part of the ring, so that
-// it consumes its slots strictly in order; warps 4-7 (one per TMEM lane
+// epilogue sums the two in issuer order); both take their units from one ring in
+// unit order (dealing a ring of three slots 2 + 1 left one issuer a single slot,
+// load after MMA after load, and held up the other); warps 4-7 (one per TMEM lane
 // quadrant) run the epilogue; all warps but the producer's stage Z when the partition
 // changes.  Every wait is bounded: on expiry the kernel records
 // ST_TIMEOUT, stops issuing, waits (bounded) for its own copies in flight,
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int R = a.ring;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar + S_RING0 + 2 * R);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  volatile uint32_t* issued = tmem_holder + 2;  // units the producer has issued
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t crank = cluster_rank();
@@ -103,11 +105,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int NB = a.ncd / 2;
   const int U = NB * PL;
   const int LAG = a.lag;
-  // Issuer h owns blocks b = h, h + HE, ... and ring slots [ring_base(h),
-  // ring_base(h) + ring_len(h)) (R dealt as evenly as it goes: 3 = 2 + 1).
+  // Issuer h owns blocks b = h, h + HE, ...; the units go through the ring's slots in
+  // order, whoever consumes them.  An issuer that skips the other's units could meet a
+  // slot one fill early, where an mbarrier parity wait succeeds at once on the fill
+  // before; so it first waits until the producer has issued its unit, which it does
+  // only after the slot's previous fill was consumed.
   const int HE = a.issuers < NB ? a.issuers : NB;
-  auto ring_len = [&](int hh) { return R / HE + (hh < R % HE ? 1 : 0); };
-  auto ring_base = [&](int hh) { return hh * (R / HE) + (hh < R % HE ? hh : R % HE); };
   const int h = warp - 1;
   const bool issuer = lane == 0 && (warp == 1 || warp == 2);
 
@@ -129,6 +132,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&bar[S_RING0 + R + s], 1);
     }
     *abort_flag = 0;
+    *issued = 0;
     fence_mbar_init();
   }
   if (warp == 0) {
@@ -160,6 +164,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   };
 
+  auto wait_issued = [&](uint32_t g) -> bool {
+    const long long t0 = clock64();
+    while (*issued <= g) {
+      if (*abort_flag) return false;
+      if (clock64() - t0 > kTimeoutCycles) {
+        give_up();
+        return false;
+      }
+    }
+    return true;
+  };
+
   constexpr uint32_t idesc1 = idesc_bf16(128, N, false, false);
   constexpr uint32_t idesc2 = idesc_bf16(128, N, true, false);
 
@@ -175,9 +191,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t T = 0;  // tiles before this run (same in every CTA of the cluster)
   uint32_t pieces = 0;     // pieces before this run
   uint32_t epi_phase = 0;  // uses of the epilogue barrier so far (epilogue threads)
-  uint32_t pcnt[2] = {0u, 0u};  // producer: units dealt to each issuer so far
-  uint32_t fills[kMaxRing] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};  // producer: fills of each slot
-  uint32_t c_own = 0;           // issuer: own units consumed so far
+  // units so far and the next one's slot and parity (producer and issuers)
+  uint32_t unit = 0, slot = 0, phase = 0;
+  auto next_unit = [&]() {
+    ++unit;
+    if (++slot == static_cast<uint32_t>(R)) {
+      slot = 0;
+      phase ^= 1;
+    }
+  };
   bool prod_ok = true;
   for (int si = sb, sj; si < se; si = sj) {
     const Segment sg = a.segs[si];
@@ -213,13 +235,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           tma_prefetch_2d(pl2 ? &map1 : &map0, c0 + 64 * (2 * b2 + j), static_cast<int>(sg.row0) + t2 * kBM);
       }
       prod_ok = for_each_unit(ntiles, U, LAG, [&](bool second, int t, int u) -> bool {
-        // the next slot of the issuer that consumes this unit
-        const int hh = (u / PL) % HE;
-        const uint32_t k = pcnt[hh], RH = static_cast<uint32_t>(ring_len(hh));
-        const uint32_t s = static_cast<uint32_t>(ring_base(hh)) + k % RH;
-        if (!wait(S_RING0 + R + s, ((k / RH) + 1) & 1, false)) return false;
-        pcnt[hh] = k + 1;
-        ++fills[s];
+        const uint32_t s = slot;
+        if (!wait(S_RING0 + R + s, phase ^ 1, false)) return false;
         mbar_expect_tx(&bar[S_RING0 + s], kUnitBytes);
         const int b = u / PL, pl = u % PL;
         const int row = static_cast<int>(sg.row0) + t * kBM;
@@ -231,6 +248,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           else
             tma_load_2d(dst, map, c0 + 64 * (2 * b + j), row, &bar[S_RING0 + s]);
         }
+        next_unit();
+        *issued = unit;
         if (!second && PF > 0) {
           const int q = t * U + u + PF;
           if (q < ntiles * U) {
@@ -247,12 +266,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       // issuer h: units of blocks b = h, h + HE, ... in the shared unit order
       const int b_last = h + ((NB - 1 - h) / HE) * HE;
       const int u_first = h * PL, u_last = b_last * PL + PL - 1;
-      const uint32_t RH = static_cast<uint32_t>(ring_len(h)), rb = static_cast<uint32_t>(ring_base(h));
       for_each_unit(ntiles, U, LAG, [&](bool second, int t, int u) -> bool {
+        const uint32_t s = slot, Tg = T + t, buf = Tg & 1;
+        const uint32_t g = unit, ph = phase;
+        next_unit();
         if ((u / PL) % HE != h) return true;
-        const uint32_t s = rb + c_own % RH, Tg = T + t, buf = Tg & 1;
-        if (!wait(S_RING0 + s, (c_own / RH) & 1, false)) return false;
-        ++c_own;
+        if ((HE > 1 && !wait_issued(g)) || !wait(S_RING0 + s, ph, false)) return false;
         if (u == u_first) {
           if (!second && !wait(S_D1EMPTY0 + buf, ((Tg >> 1) + 1) & 1, false)) return false;
           if (second && !wait(S_B2FULL0 + buf, (Tg >> 1) & 1, false)) return false;
@@ -435,11 +454,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   // Copies still in flight (only after an abort) land before the CTA exits: the last
   // fill of every slot (earlier fills were waited for by then).
   if (warp == 0 && lane == 0) {
-    for (int q = 0; q < R; ++q) {
-      if (fills[q] == 0) continue;
-      const uint32_t addr = su32(&bar[S_RING0 + q]);
+    for (uint32_t g = unit > static_cast<uint32_t>(R) ? unit - R : 0; g < unit; ++g) {
+      const uint32_t addr = su32(&bar[S_RING0 + g % R]);
       const long long t0 = clock64();
-      while (!mbar_try(addr, (fills[q] - 1) & 1) && clock64() - t0 < kTimeoutCycles) {
+      while (!mbar_try(addr, (g / R) & 1) && clock64() - t0 < kTimeoutCycles) {
       }
     }
   }
