@@ -390,8 +390,8 @@ lp_status launch_step(lp_ctx* c, int K, const float* Z, int64_t z_stride, bool t
     e = lp::launch_step_pair(*c->tcs_cur, c->dSegsTcs, c->dSegPtrTcs, Z, z_stride, c->dP, static_cast<int>(c->d),
                              c->dStatus, c->stream);
   else if (c->path == PATH_TCS && c->tcs_cur->fp8)
-    e = lp::launch_step_tcs8(*c->tcs_cur, c->dSegsTcs, c->dSegPtrTcs, Z, z_stride, c->dP, static_cast<int>(c->d),
-                             c->dScales, c->smax2, c->dStatus, c->stream);
+    e = lp::launch_step_tcs8(*c->tcs_cur, c->dA, c->n, c->ld, c->dSegsTcs, c->dSegPtrTcs, Z, z_stride, c->dP,
+                             static_cast<int>(c->d), c->dScales, c->smax2, c->dStatus, c->stream);
   else if (c->path == PATH_TCS)
     e = lp::launch_step_tcs(*c->tcs_cur, c->dSegsTcs, c->dSegPtrTcs, Z, z_stride, c->dP, static_cast<int>(c->d),
                             c->dStatus, c->stream);
@@ -859,7 +859,6 @@ static lp_status ensure_tcs(lp_ctx* c, int k) {
       planned = lp::tcs8_plan(static_cast<int>(c->d), K, c->sms, c->tuning, &p);
       if (!planned)
         return fail(c, LP_ERR_UNSUPPORTED, "no FP8 tensor-core plan for d=" + std::to_string(c->d));
-      LP_CUDA(lp::tcs8_encode_map(c->dA, c->n, static_cast<int>(c->d), c->ld, &p));
     } else {
       const int want = c->tuning.kernel == LP_KERNEL_DEFAULT ? kDefaultTcKernel : c->tuning.kernel;
       if (want == LP_KERNEL_PAIR)

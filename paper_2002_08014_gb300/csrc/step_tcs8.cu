@@ -1,16 +1,17 @@
 // Fused local power step on the 5th-generation tensor cores for A stored as
 // FP8-E4M3 codes with one FP32 scale per row (a_r = s_r q_r):
 //   P[slot] = A_seg^T (A_seg Z_i) = Q^T diag(s^2) Q Z_i      (eq. (2), unscaled),
-// streaming form (the geometry, ring, interleave and cluster exchange of the
-// streaming BF16 kernel in step_tcs.cu).
+// streaming form (the geometry, unit ring and cluster exchange of the streaming
+// BF16 kernel in step_tcs.cu).
 //
 // The scales factor out of both contractions, so the tensor cores only ever see
 // the codes.  Every E4M3 value is exactly an FP16 value (3 significand bits,
 // exponents 2^-9 .. 2^8), and one cvt.rn.f16x2.e4m3x2 turns two codes into two
 // FP16, so:
-//   * TMA lands each 128-row x 128-column box of codes (16 KB) in a staging ring;
-//   * four converter warps widen it into the FP16 operand layout the MMAs read
-//     (SWIZZLE_128B, K-major, 32 KB per unit) in the operand ring;
+//   * eight converter warps read each 128-row x 128-column unit of codes (16 KB)
+//     straight into registers, kDepth units ahead, widen it and write the FP16
+//     operand layout the MMAs read (SWIZZLE_128B, K-major, 32 KB per unit) into the
+//     operand ring;
 //   * first pass  D1 += Q_u [Z_hi | Z_lo]  (kind::f16 with FP16 operands; Z
 //     split into FP16 hi + lo, 22 significand bits between them);
 //   * epilogue    W = D1[:, :K] + D1[:, K:] (cluster-summed), then row r scaled
@@ -21,11 +22,21 @@
 // A row whose s_r^2 / S is below the FP16 range contributes nothing: its
 // contribution is below 2^-24 of the largest row's, under FP32 rounding of P.
 //
-// Roles (384 threads): warp 0 lane 0 issues TMA; warp 1 lane 0 issues MMAs;
-// warps 4-7 run the epilogue; warps 8-11 convert; all warps stage Z at segment
-// starts.  Every wait is bounded: on expiry the kernel records ST_TIMEOUT, stops
-// issuing, waits (bounded) for its own copies in flight, retires its MMAs,
-// frees tensor memory and returns.
+// What bounds it.  Z, the W operands and the exchange buffers leave about 96 KB of
+// shared memory at d = 2,048, k = 32.  With the codes staged there by TMA (two 16 KB
+// slots beside two operand slots) both passes together had 32 KB in flight and every
+// unit crossed shared memory twice; the launch took 2,150 us at n = 1M.  In registers
+// the codes in flight cost no shared memory (48 KB at kDepth = 3) and the operand ring
+// has three slots.  The second pass of a tile runs two tiles behind the first where
+// tensor memory holds a third D1, so that the cluster exchange of W (about 3 us, as
+// long as the first pass of a whole tile) is off the chain.
+//
+// Roles (448 threads): warps 0-3 and 8-11 convert; warps 4-7 run the epilogue; lane 0
+// of warps 12 and 13 issue the first and the second pass's MMAs (one thread issues a
+// small-N MMA only every ~55 cycles, ~100 when it polls barriers in between); warps
+// 4-7, 12 and 13 stage Z when the partition changes, while the converters go on.
+// Every wait is bounded: on expiry the kernel records ST_TIMEOUT, stops issuing,
+// retires its MMAs, frees tensor memory and returns.
 #include <cuda_fp16.h>
 
 #include "lp_internal.cuh"
@@ -36,22 +47,24 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreads8 = 384;
-constexpr int kConvWarp0 = 8;                // warps 8-11
-constexpr int kConvThreads = 128;
+constexpr int kThreads8 = 448;
+constexpr int kConvThreads = 256;            // warps 0-3 and 8-11
+constexpr int kIssue1 = 12, kIssue2 = 13;    // warps whose lane 0 issues the first / second pass
+constexpr int kOthers8 = kThreads8 - kConvThreads;
+constexpr int kDepth = 3;                    // units of codes in flight per converter thread
 constexpr int kUnitBytes = 2 * kChunkBytes;  // 128 rows x 128 columns of FP16 (two 64-column chunks)
-constexpr int kStageBytes = kBM * 128;       // 128 rows x 128 E4M3 codes
 constexpr int kMaxRing = 8;
+constexpr int kMaxD1 = 3;                    // D1 buffers
 constexpr int kSmemLimit = 232448;
 
-enum Tcs8Bar { S_D1FULL0 = 0, S_D1EMPTY0 = 2, S_B2FULL0 = 4, S_B2FREE0 = 6, S_D2FULL = 8, S_REDFULL = 9,
-               S_WFULL = 10, S_DONE = 11, S_EPI = 12, S_RING0 = 13 };
-// operand ring: FULL[s] = S_RING0 + s, EMPTY[s] = S_RING0 + kMaxRing + s;
-// staging ring: FULL[q] = S_RING0 + 2 kMaxRing + q, EMPTY[q] = S_RING0 + 3 kMaxRing + q
-constexpr int S_STG0 = S_RING0 + 2 * kMaxRing;
-constexpr int kNumBars8 = S_RING0 + 4 * kMaxRing;
+enum Tcs8Bar { S_D1FULL0 = 0, S_D1EMPTY0 = 3, S_B2FULL0 = 6, S_B2FREE0 = 8, S_D2FULL = 10, S_D2EMPTY = 11,
+               S_REDFULL = 12, S_WFULL = 13, S_DONE = 14, S_EPI = 15, S_RING0 = 16 };
+// operand ring: FULL[s] = S_RING0 + s, EMPTY[s] = S_RING0 + kMaxRing + s
+constexpr int kNumBars8 = S_RING0 + 2 * kMaxRing;
 
 struct Tcs8Args {
+  const unsigned char* codes;  // n x ld, columns d .. ld - 1 zero
+  int64_t n, ld;
   const Segment* segs;
   const int* seg_ptr;  // per cluster
   const float* Z;
@@ -63,21 +76,89 @@ struct Tcs8Args {
   float smax2;          // S = max_r s_r^2
   int ncd;              // 64-column chunks in this CTA's slice (even)
   int ring;             // operand ring units
-  int stage;            // staging ring units
-  int lag;
+  int lag;              // units of a tile's first pass ahead of the second pass of the tile `behind` before it
+  int behind;           // tiles the second pass runs behind the first (D1 buffers less one)
   int hints;
-  uint32_t off_stage, off_B1, off_B2, off_W, off_Wrecv, off_bar, tmem_cols;
+  uint32_t off_B1, off_B2, off_W, off_Wrecv, off_bar, tmem_cols;
 };
 
-template <typename F>
-__device__ __forceinline__ bool for_each_unit8(int ntiles, int U, int lag, F&& fn) {
-  for (int t = 0; t <= ntiles; ++t)
-    for (int u = 0; u < U + lag; ++u) {
-      if (t < ntiles && u < U && !fn(false, t, u)) return false;
-      if (t >= 1 && u >= lag && u - lag < U && !fn(true, t - 1, u - lag)) return false;
-    }
-  return true;
+// A run: the consecutive pieces of one partition that a cluster owns, one stream of
+// tiles (every piece but the last is a whole number of tiles).
+struct Run8 {
+  int si, sj;      // segments
+  int64_t row0, row1;
+  int ntiles;
+};
+__device__ __forceinline__ Run8 run_at(const Segment* segs, int si, int se) {
+  Run8 r;
+  r.si = si;
+  r.row0 = segs[si].row0;
+  const int part = segs[si].part;
+  r.sj = si + 1;
+  while (r.sj < se && segs[r.sj].part == part) ++r.sj;
+  r.row1 = segs[r.sj - 1].row1;
+  r.ntiles = static_cast<int>((r.row1 - r.row0 + kBM - 1) / kBM);
+  return r;
 }
+
+// The unit order of a cluster, walked by every role: within a run, the first pass of
+// tile t (units 0 .. U-1) interleaved with the second pass of tile t - behind, `lag`
+// units later.
+struct Walk8 {
+  const Segment* segs;
+  int se, U, lag, behind;
+  Run8 run;
+  uint32_t T = 0;       // tiles before the run
+  uint32_t pieces = 0;  // pieces before the run
+  int t = 0, u = -1, half = 1;
+  // the unit
+  bool second = false;
+  int tile = 0, blk = 0;
+  bool new_run = true;
+  __device__ Walk8(const Segment* s, int sb, int se_, int U_, int lag_, int behind_)
+      : segs(s), se(se_), U(U_), lag(lag_), behind(behind_) {
+    run = run_at(segs, sb, se);
+  }
+  __device__ static int pieces_of(int ntiles) {
+    constexpr int TP = static_cast<int>(kTcChainRows / kBM);
+    return (ntiles + TP - 1) / TP;
+  }
+  // moves to the next unit; false after the last
+  __device__ bool next() {
+    new_run = false;
+    while (true) {
+      if (half == 0) {
+        half = 1;
+      } else {
+        half = 0;
+        if (++u == U + lag) {
+          u = 0;
+          if (++t == run.ntiles + behind) {
+            T += run.ntiles;
+            pieces += pieces_of(run.ntiles);
+            if (run.sj >= se) return false;
+            run = run_at(segs, run.sj, se);
+            t = 0;
+            new_run = true;
+          }
+        }
+      }
+      if (half == 0) {
+        if (t < run.ntiles && u < U) {
+          second = false;
+          tile = t;
+          blk = u;
+          return true;
+        }
+      } else if (t >= behind && u >= lag && u - lag < U) {
+        second = true;
+        tile = t - behind;
+        blk = u - lag;
+        return true;
+      }
+    }
+  }
+};
 
 // Instruction descriptor: kind::f16 with FP16 A and B, FP32 accumulate, dense.
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, bool a_mn_major, bool b_mn_major) {
@@ -93,24 +174,36 @@ __device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t two_codes) {
 
 __device__ __forceinline__ uint16_t f16_bits(float x) { return __half_as_ushort(__float2half_rn(x)); }
 __device__ __forceinline__ float f16_val(uint16_t b) { return __half2float(__ushort_as_half(b)); }
+struct F16Op {
+  static __device__ __forceinline__ uint16_t bits(float x) { return f16_bits(x); }
+  static __device__ __forceinline__ float val(uint16_t b) { return f16_val(b); }
+};
+
+__device__ __forceinline__ uint4 ld_codes(const unsigned char* p, uint64_t policy) {
+  uint4 v;
+  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p), "l"(policy));
+  return v;
+}
 
 template <int K>
-__global__ void __launch_bounds__(kThreads8, 1)
-    step_tcs8_kernel(const __grid_constant__ CUtensorMap map, Tcs8Args a) {
+__global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
   constexpr int N = 2 * K;
   constexpr uint32_t B2BUF = 2 * N * 128;
+  constexpr int TP = static_cast<int>(kTcChainRows / kBM);
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char* sRing = base;
-  unsigned char* sStage = base + a.off_stage;
   unsigned char* sB1 = base + a.off_B1;
   unsigned char* sB2 = base + a.off_B2;
   float* sW = reinterpret_cast<float*>(base + a.off_W);
   float* sWrecv = reinterpret_cast<float*>(base + a.off_Wrecv);
   uint64_t* bar = reinterpret_cast<uint64_t*>(base + a.off_bar);
-  const int R = a.ring, R8 = a.stage;
+  const int R = a.ring;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar + kNumBars8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  volatile uint32_t* filled = tmem_holder + 2;  // units the converters have begun to fill
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t crank = cluster_rank();
@@ -120,27 +213,29 @@ __global__ void __launch_bounds__(kThreads8, 1)
   const int DC = 64 * a.ncd;
   const int c0 = static_cast<int>(crank) * DC;
   const int U = a.ncd / 2;  // one unit per 128-column block
-  const int LAG = a.lag;
+  const int ND1 = a.behind + 1;
 
   if (tid == 0) {
-    for (int s = 0; s < 2; ++s) {
+    for (int s = 0; s < kMaxD1; ++s) {
       mbar_init(&bar[S_D1FULL0 + s], 1);
       mbar_init(&bar[S_D1EMPTY0 + s], 4);
+    }
+    for (int s = 0; s < 2; ++s) {
       mbar_init(&bar[S_B2FULL0 + s], kBM);
       mbar_init(&bar[S_B2FREE0 + s], 1);
     }
     mbar_init(&bar[S_D2FULL], 1);
+    mbar_init(&bar[S_D2EMPTY], 4);
     mbar_init(&bar[S_REDFULL], 1);
     mbar_init(&bar[S_WFULL], 1);
-    mbar_init(&bar[S_DONE], 1);
+    mbar_init(&bar[S_DONE], 2);
     mbar_init(&bar[S_EPI], 128);
     for (int s = 0; s < kMaxRing; ++s) {
       mbar_init(&bar[S_RING0 + s], kConvThreads / 32);  // one arrival per converter warp
       mbar_init(&bar[S_RING0 + kMaxRing + s], 1);        // MMA commit
-      mbar_init(&bar[S_STG0 + s], 1);                    // TMA bytes
-      mbar_init(&bar[S_STG0 + kMaxRing + s], kConvThreads / 32);
     }
     *abort_flag = 0;
+    *filled = 0;
     fence_mbar_init();
   }
   if (warp == 0) {
@@ -154,6 +249,7 @@ __global__ void __launch_bounds__(kThreads8, 1)
   cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem = *tmem_holder;
+  const uint32_t tD2 = tmem + static_cast<uint32_t>(ND1 * N);
 
   auto give_up = [&]() {
     *abort_flag = 1;
@@ -171,265 +267,316 @@ __global__ void __launch_bounds__(kThreads8, 1)
       }
     }
   };
+  // Both issuers take units from one ring; before a parity wait on a slot an issuer sees
+  // that its unit's fill has begun, i.e. that the fill before was consumed (a wait a fill
+  // early would succeed at once).
+  auto wait_filled = [&](uint32_t g) -> bool {
+    const long long t0 = clock64();
+    while (*filled <= g) {
+      if (*abort_flag) return false;
+      if (clock64() - t0 > kTimeoutCycles) {
+        give_up();
+        return false;
+      }
+    }
+    return true;
+  };
 
   constexpr uint32_t idesc1 = idesc_f16(128, N, false, false);
   constexpr uint32_t idesc2 = idesc_f16(128, N, true, false);
 
   const int sb = a.seg_ptr[cluster_id], se = a.seg_ptr[cluster_id + 1];
-  uint32_t T = 0;          // tiles before this segment (same in every CTA of the cluster)
-  uint32_t epi_phase = 0;  // uses of the epilogue barrier so far
-  uint32_t G = 0;          // units before this segment
-  uint32_t g_prod_end = 0;
-  for (int si = sb; si < se; ++si) {
-    const Segment sg = a.segs[si];
-    const int ntiles = static_cast<int>((sg.row1 - sg.row0 + kBM - 1) / kBM);
-
-    // ---- stage this slice of Z as [Z_hi | Z_lo]^T in FP16 (N rows x DC, K-major, SWIZZLE_128B)
-    __syncthreads();
-    if (si == sb || sg.part != a.segs[si - 1].part) {
-      const float* Zg = a.Z + a.z_stride * sg.part;
-      for (int e = tid; e < DC * K; e += kThreads8) {
-        const int c = e / K, j = e % K;
-        const float z = (c0 + c < a.d) ? Zg[static_cast<int64_t>(c0 + c) * K + j] : 0.f;
-        const uint16_t hi = f16_bits(z);
-        const uint16_t lo = f16_bits(z - f16_val(hi));
-        *reinterpret_cast<uint16_t*>(sB1 + sw128_off(j, c, N)) = hi;
-        *reinterpret_cast<uint16_t*>(sB1 + sw128_off(K + j, c, N)) = lo;
-      }
+  const bool converter = warp < 4 || (warp >= 8 && warp < 12);
+  if (sb >= se) {
+    // no rows: straight to the teardown
+  } else if (converter) {
+    // -------------------------------------------------------------- converters: codes -> FP16 operand
+    const int ct = warp < 4 ? tid : tid - 128;  // 0 .. 255
+    const int col16 = ct & 7, row8 = ct >> 3;   // 16 codes of row row8 + 32 i
+    uint64_t pol_keep = l2_policy_evict_last(), pol_drop = l2_policy_evict_first();
+    if (!a.hints) pol_drop = pol_keep;
+    uint4 buf[kDepth][4];
+    Walk8 ahead(a.segs, sb, se, U, a.lag, a.behind);
+    bool more = true;
+    auto fetch = [&](uint4 (&v)[4]) {
+      if (more) more = ahead.next();
+      const int64_t r0 = ahead.run.row0 + static_cast<int64_t>(ahead.tile) * kBM + row8;
+      const int c = c0 + 128 * ahead.blk + 16 * col16;
+      const unsigned char* p = a.codes + r0 * a.ld + c;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        v[i] = more && c < a.ld && r0 + 32 * i < a.n ? ld_codes(p + static_cast<int64_t>(32 * i) * a.ld,
+                                                                 ahead.second ? pol_drop : pol_keep)
+                                                     : make_uint4(0u, 0u, 0u, 0u);
+    };
+    // units in all: two passes over every tile's U units
+    uint32_t total = 0;
+    for (int si = sb; si < se;) {
+      const Run8 r = run_at(a.segs, si, se);
+      total += 2u * static_cast<uint32_t>(r.ntiles) * static_cast<uint32_t>(U);
+      si = r.sj;
     }
-    fence_async_smem();
-    __syncthreads();
-
-    if (warp == 0 && lane == 0) {
-      // ------------------------------------------------------------ TMA producer (codes into staging)
-      uint64_t pol_keep = 0, pol_drop = 0;
-      if (a.hints) {
-        pol_keep = l2_policy_evict_last();
-        pol_drop = l2_policy_evict_first();
-      }
-      uint32_t g = G;
-      for_each_unit8(ntiles, U, LAG, [&](bool second, int t, int u) -> bool {
-        const uint32_t q = g % R8;
-        if (!wait(S_STG0 + kMaxRing + q, ((g / R8) + 1) & 1, false)) return false;
-        mbar_expect_tx(&bar[S_STG0 + q], kStageBytes);
-        const int row = static_cast<int>(sg.row0) + t * kBM;
-        const uint32_t dst = su32(sStage + q * kStageBytes);
-        if (a.hints) tma_load_2d_hint(dst, &map, c0 + 128 * u, row, &bar[S_STG0 + q], second ? pol_drop : pol_keep);
-        else tma_load_2d(dst, &map, c0 + 128 * u, row, &bar[S_STG0 + q]);
-        ++g;
-        return true;
-      });
-      g_prod_end = g;
-    } else if (warp >= kConvWarp0 && warp < kConvWarp0 + kConvThreads / 32) {
-      // ------------------------------------------------------------ converters: codes -> FP16 operand
-      const int ct = tid - kConvWarp0 * 32;
-      uint32_t g = G;
-      for_each_unit8(ntiles, U, LAG, [&](bool, int, int) -> bool {
-        const uint32_t q = g % R8, s = g % R;
-        if (!wait(S_STG0 + q, (g / R8) & 1, false)) return false;
-        if (!wait(S_RING0 + kMaxRing + s, ((g / R) + 1) & 1, false)) return false;
-        const unsigned char* stg = sStage + q * kStageBytes;
-        unsigned char* dst = sRing + s * kUnitBytes;
-#pragma unroll 4
-        for (int gi = ct; gi < kBM * 16; gi += kConvThreads) {
-          const int r = gi >> 4, c8 = gi & 15;  // row, group of 8 columns
-          const uint2 codes = *reinterpret_cast<const uint2*>(stg + r * 128 + c8 * 8);
-          uint4 out;
-          out.x = e4m3x2_to_f16x2(codes.x & 0xFFFFu);
-          out.y = e4m3x2_to_f16x2(codes.x >> 16);
-          out.z = e4m3x2_to_f16x2(codes.y & 0xFFFFu);
-          out.w = e4m3x2_to_f16x2(codes.y >> 16);
-          *reinterpret_cast<uint4*>(dst + (c8 >> 3) * kChunkBytes + r * 128 + ((((c8 & 7) ^ (r & 7))) << 4)) = out;
+#pragma unroll
+    for (int x = 0; x < kDepth; ++x) fetch(buf[x]);
+    uint32_t slot = 0, phase = 0;
+    bool ok = true;
+    for (uint32_t g0 = 0; ok && g0 < total; g0 += kDepth) {
+#pragma unroll
+      for (int x = 0; x < kDepth; ++x) {
+        if (!ok || g0 + x >= total) continue;
+        if (!(ok = wait(S_RING0 + kMaxRing + static_cast<int>(slot), phase ^ 1, false))) continue;
+        if (ct == 0) *filled = g0 + x + 1;
+        unsigned char* dst = sRing + slot * kUnitBytes + (col16 >> 2) * kChunkBytes;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = row8 + 32 * i;
+          const uint4 v = buf[x][i];
+          uint4 h[2];
+          h[0].x = e4m3x2_to_f16x2(v.x & 0xFFFFu);
+          h[0].y = e4m3x2_to_f16x2(v.x >> 16);
+          h[0].z = e4m3x2_to_f16x2(v.y & 0xFFFFu);
+          h[0].w = e4m3x2_to_f16x2(v.y >> 16);
+          h[1].x = e4m3x2_to_f16x2(v.z & 0xFFFFu);
+          h[1].y = e4m3x2_to_f16x2(v.z >> 16);
+          h[1].z = e4m3x2_to_f16x2(v.w & 0xFFFFu);
+          h[1].w = e4m3x2_to_f16x2(v.w >> 16);
+          // the two chunks' halves in opposite order: the eight lanes of a row hit eight bank groups
+          const int flip = col16 >> 2;
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int hf = q ^ flip, c8 = 2 * (col16 & 3) + hf;
+            *reinterpret_cast<uint4*>(dst + r * 128 + ((c8 ^ (r & 7)) << 4)) = hf ? h[1] : h[0];
+          }
         }
+        fetch(buf[x]);
         fence_async_smem();  // the MMAs read these tiles through the async proxy
         __syncwarp();
-        if (lane == 0) {
-          mbar_arrive(&bar[S_RING0 + s]);
-          mbar_arrive(&bar[S_STG0 + kMaxRing + q]);
+        if (lane == 0) mbar_arrive(&bar[S_RING0 + slot]);
+        if (++slot == static_cast<uint32_t>(R)) {
+          slot = 0;
+          phase ^= 1;
         }
-        ++g;
-        return true;
-      });
-    } else if (warp == 1 && lane == 0) {
-      // ------------------------------------------------------------ MMA issuer
-      uint32_t g = G;
-      for_each_unit8(ntiles, U, LAG, [&](bool second, int t, int u) -> bool {
-        const uint32_t s = g % R, Tg = T + t, buf = Tg & 1;
-        if (!wait(S_RING0 + s, (g / R) & 1, false)) return false;
-        if (u == 0) {
-          if (!second && !wait(S_D1EMPTY0 + buf, ((Tg >> 1) + 1) & 1, false)) return false;
-          if (second && !wait(S_B2FULL0 + buf, (Tg >> 1) & 1, false)) return false;
-        }
-        tc_fence_after();
-        const uint32_t aS = su32(sRing + s * kUnitBytes);
-        if (!second) {
-          const uint32_t bS = su32(sB1);
-#pragma unroll
-          for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              const uint64_t ad = sdesc(aS + j * kChunkBytes + kk * 32, 16, 1024);
-              const uint64_t bd = sdesc(bS + (2 * u + j) * N * 128 + kk * 32, 16, 1024);
-              mma_bf16(tmem + buf * N, ad, bd, idesc1, (u | j | kk) != 0);
-            }
-          mma_commit(&bar[S_RING0 + kMaxRing + s]);
-          if (u == U - 1) mma_commit(&bar[S_D1FULL0 + buf]);
-        } else {
-          const uint32_t bS = su32(sB2 + buf * B2BUF);
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint64_t ad = sdesc(aS + kk * 2048, kChunkBytes, 1024);
-            const uint64_t bd = sdesc(bS + (kk >> 2) * N * 128 + (kk & 3) * 32, 16, 1024);
-            mma_bf16(tmem + 2 * N + u * N, ad, bd, idesc2, (t == 0 && kk == 0) ? 0u : 1u);
-          }
-          mma_commit(&bar[S_RING0 + kMaxRing + s]);
-          if (u == U - 1) mma_commit(&bar[S_B2FREE0 + buf]);
-        }
-        ++g;
-        return true;
-      });
-      mma_commit(&bar[S_D2FULL]);
-    } else if (warp >= 4 && warp < 8) {
-      // ------------------------------------------------------------ epilogue
-      const int r = (warp - 4) * 32 + lane;
-      const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
-      bool ok = true;
-      auto epi_sync = [&]() -> bool {
-        mbar_arrive(&bar[S_EPI]);
-        return wait(S_EPI, (epi_phase++) & 1, false);
-      };
-      for (int t = 0; ok && t < ntiles; ++t) {
-        const uint32_t Tg = T + t, buf = Tg & 1;
-        if (!(ok = wait(S_D1FULL0 + buf, (Tg >> 1) & 1, false))) break;
-        tc_fence_after();
-        float w[K];
-#pragma unroll
-        for (int q = 0; q < N / 16; ++q) {
-          float v[16];
-          tmem_ld16(tmem + lane_base + buf * N + q * 16, v);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int col = q * 16 + i;
-            if (col < K) w[col] = v[i];
-            else w[col - K] += v[i];
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bar[S_D1EMPTY0 + buf]);
-        const int64_t grow = sg.row0 + static_cast<int64_t>(t) * kBM + r;
-        const bool valid = grow < sg.row1;
-        if (!valid) {
-#pragma unroll
-          for (int j = 0; j < K; ++j) w[j] = 0.f;
-        }
-        if (CL > 1) {
-          const uint32_t rows_bytes = static_cast<uint32_t>(RPC * K * 4);
-          if (!(ok = epi_sync())) break;
-#pragma unroll
-          for (int j = 0; j < K; j += 4)
-            *reinterpret_cast<float4*>(sW + wpos<K>(r, j)) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
-          fence_async_smem();
-          if (!(ok = epi_sync())) break;
-          if (r == 0) {
-            mbar_expect_tx(&bar[S_REDFULL], (CL - 1) * rows_bytes);
-            for (uint32_t o = 0; o < CL; ++o)
-              if (o != crank)
-                bulk_s2s_cluster(mapa(su32(sWrecv + crank * RPC * K), o), su32(sW + o * RPC * K), rows_bytes,
-                                 mapa(su32(&bar[S_REDFULL]), o));
-            bulk_commit();
-            bulk_wait_read0();
-          }
-          if (!(ok = wait(S_REDFULL, Tg & 1, true))) break;
-          const int per = RPC * K / kBM;
-          for (int e = 0; e < per; ++e) {
-            const int idx = r * per + e, rl = idx / K, col = idx % K;
-            const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
-            const int rel = own - static_cast<int>(crank) * RPC * K;
-            float sum = 0.f;
-            for (uint32_t src = 0; src < CL; ++src) sum += src == crank ? sW[own] : sWrecv[src * RPC * K + rel];
-            sW[own] = sum;
-          }
-          fence_async_smem();
-          if (!(ok = epi_sync())) break;
-          if (r == 0) {
-            mbar_expect_tx(&bar[S_WFULL], (CL - 1) * rows_bytes);
-            for (uint32_t dst = 0; dst < CL; ++dst)
-              if (dst != crank)
-                bulk_s2s_cluster(mapa(su32(sW + crank * RPC * K), dst), su32(sW + crank * RPC * K), rows_bytes,
-                                 mapa(su32(&bar[S_WFULL]), dst));
-            bulk_commit();
-            bulk_wait_read0();
-          }
-          if (!(ok = wait(S_WFULL, Tg & 1, true))) break;
-#pragma unroll
-          for (int j = 0; j < K; j += 4) {
-            const float4 v = *reinterpret_cast<const float4*>(sW + wpos<K>(r, j));
-            w[j] = v.x;
-            w[j + 1] = v.y;
-            w[j + 2] = v.z;
-            w[j + 3] = v.w;
-          }
-        }
-        // row scale: W_r <- W_r s_r^2 / S (so the FP16 operand cannot overflow)
-        const float sc = valid ? a.scales[grow] : 0.f;
-        const float f = sc * sc / a.smax2;
-#pragma unroll
-        for (int j = 0; j < K; ++j) w[j] *= f;
-        if (!(ok = wait(S_B2FREE0 + buf, ((Tg >> 1) + 1) & 1, false))) break;
-        unsigned char* B2 = sB2 + buf * B2BUF;
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-          const uint16_t hi = f16_bits(w[j]);
-          const uint16_t lo = f16_bits(w[j] - f16_val(hi));
-          *reinterpret_cast<uint16_t*>(B2 + sw128_off(j, r, N)) = hi;
-          *reinterpret_cast<uint16_t*>(B2 + sw128_off(K + j, r, N)) = lo;
-        }
-        fence_async_smem();
-        mbar_arrive(&bar[S_B2FULL0 + buf]);
       }
-      // segment end: Y slice = S (D2[:, :K] + D2[:, K:]) -> P[slot]
-      if (ok && wait(S_D2FULL, (si - sb) & 1, false)) {
-        tc_fence_after();
-        float* Pd = a.P + static_cast<int64_t>(sg.slot) * a.d * K;
-        for (int b = 0; b < U; ++b) {
-          float y[K];
+    }
+  } else {
+    // -------------------------------------------------------------- issuers and epilogue, run by run
+    const int ot = warp < 8 ? tid - 128 : tid - 384 + 128;  // 0 .. kOthers8 - 1
+    uint32_t T = 0, pieces = 0, epi_phase = 0;
+    uint32_t unit = 0, slot = 0, phase = 0;
+    Walk8 walk(a.segs, sb, se, U, a.lag, a.behind);
+    bool more = walk.next();
+    for (int si = sb; si < se;) {
+      const Run8 run = run_at(a.segs, si, se);
+      __syncwarp();
+      // every role finished the previous run; all leave together after an abort
+      if (bar_or(1, kOthers8, *abort_flag != 0)) break;
+      // this slice of Z as [Z_hi | Z_lo]^T in FP16 (N rows x DC, K-major, SWIZZLE_128B)
+      if (si == sb || a.z_stride != 0)
+        stage_z<K, F16Op>(sB1, a.Z + a.z_stride * a.segs[si].part, c0, DC, a.d, ot, kOthers8);
+      fence_async_smem();
+      bar_sync(1, kOthers8);
+
+      if (warp >= kIssue1) {
+        if (lane == 0) {
+          // ---------------------------------------------------------- MMA issuers (one per pass)
+          const bool mine2 = warp == kIssue2;
+          bool ok = true;
+          bool first_of_run = true;
+          while (more && (first_of_run || !walk.new_run)) {
+            first_of_run = false;
+            const uint32_t g = unit, s = slot, ph = phase;
+            const int t = walk.tile, u = walk.blk;
+            const bool second = walk.second;
+            ++unit;
+            if (++slot == static_cast<uint32_t>(R)) {
+              slot = 0;
+              phase ^= 1;
+            }
+            more = walk.next();
+            if (second != mine2 || !ok) continue;
+            const uint32_t Tg = T + t;
+            if (!(ok = wait_filled(g) && wait(S_RING0 + static_cast<int>(s), ph, false))) continue;
+            const uint32_t aS = su32(sRing + s * kUnitBytes);
+            if (!second) {
+              const uint32_t buf = Tg % ND1;
+              if (u == 0 && !(ok = wait(S_D1EMPTY0 + static_cast<int>(buf), ((Tg / ND1) + 1) & 1, false))) continue;
+              tc_fence_after();
+              const uint32_t bS = su32(sB1);
+#pragma unroll
+              for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                  const uint64_t ad = sdesc(aS + j * kChunkBytes + kk * 32, 16, 1024);
+                  const uint64_t bd = sdesc(bS + (2 * u + j) * N * 128 + kk * 32, 16, 1024);
+                  mma_bf16(tmem + buf * N, ad, bd, idesc1, (u | j | kk) != 0);
+                }
+              mma_commit(&bar[S_RING0 + kMaxRing + s]);
+              if (u == U - 1) mma_commit(&bar[S_D1FULL0 + buf]);
+            } else {
+              const uint32_t buf = Tg & 1;
+              if (u == 0) {
+                if (!(ok = wait(S_B2FULL0 + static_cast<int>(buf), (Tg >> 1) & 1, false))) continue;
+                // a new piece accumulates from zero: the previous one's sums have been read out
+                if (t % TP == 0 && !(ok = wait(S_D2EMPTY, (pieces + t / TP + 1) & 1, false))) continue;
+              }
+              tc_fence_after();
+              const uint32_t bS = su32(sB2 + buf * B2BUF);
+#pragma unroll
+              for (int kk = 0; kk < 8; ++kk) {
+                const uint64_t ad = sdesc(aS + kk * 2048, kChunkBytes, 1024);
+                const uint64_t bd = sdesc(bS + (kk >> 2) * N * 128 + (kk & 3) * 32, 16, 1024);
+                mma_bf16(tD2 + u * N, ad, bd, idesc2, (t % TP == 0 && kk == 0) ? 0u : 1u);
+              }
+              mma_commit(&bar[S_RING0 + kMaxRing + s]);
+              if (u == U - 1) {
+                mma_commit(&bar[S_B2FREE0 + buf]);
+                if (t % TP == TP - 1 || t == run.ntiles - 1) mma_commit(&bar[S_D2FULL]);
+              }
+            }
+          }
+          // the first pass's last D1 is full before the second pass ends, and the epilogue
+          // waits for that, so Z is free when the run is over
+        }
+      } else {
+        // ------------------------------------------------------------ epilogue
+        const int r = (warp - 4) * 32 + lane;
+        const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
+        bool ok = true;
+        auto epi_sync = [&]() -> bool {
+          mbar_arrive(&bar[S_EPI]);
+          return wait(S_EPI, (epi_phase++) & 1, false);
+        };
+        // Y slice = S (D2[:, :K] + D2[:, K:]) of piece `piece` -> P[slot]
+        auto drain = [&](int piece) -> bool {
+          if (!wait(S_D2FULL, (pieces + piece) & 1, false)) return false;
+          tc_fence_after();
+          float* Pd = a.P + static_cast<int64_t>(a.segs[si + piece].slot) * a.d * K;
+          for (int b = 0; b < U; ++b) {
+            float y[K];
+#pragma unroll
+            for (int q = 0; q < N / 16; ++q) {
+              float v[16];
+              tmem_ld16(tD2 + lane_base + b * N + q * 16, v);
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                const int col = q * 16 + i;
+                if (col < K) y[col] = v[i];
+                else y[col - K] += v[i];
+              }
+            }
+            const int dcol = c0 + b * 128 + (warp & 3) * 32 + lane;
+            if (dcol < a.d) {
+              float4* dst = reinterpret_cast<float4*>(Pd + static_cast<int64_t>(dcol) * K);
+#pragma unroll
+              for (int j = 0; j < K; j += 4)
+                dst[j / 4] = make_float4(a.smax2 * y[j], a.smax2 * y[j + 1], a.smax2 * y[j + 2], a.smax2 * y[j + 3]);
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bar[S_D2EMPTY]);
+          return true;
+        };
+        for (int t = 0; ok && t < run.ntiles; ++t) {
+          const uint32_t Tg = T + t, buf = Tg % ND1, wb = Tg & 1;
+          if (!(ok = wait(S_D1FULL0 + static_cast<int>(buf), (Tg / ND1) & 1, false))) break;
+          tc_fence_after();
+          float w[K];
 #pragma unroll
           for (int q = 0; q < N / 16; ++q) {
             float v[16];
-            tmem_ld16(tmem + lane_base + 2 * N + b * N + q * 16, v);
+            tmem_ld16(tmem + lane_base + buf * N + q * 16, v);
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
               const int col = q * 16 + i;
-              if (col < K) y[col] = v[i];
-              else y[col - K] += v[i];
+              if (col < K) w[col] = v[i];
+              else w[col - K] += v[i];
             }
           }
-          const int dcol = c0 + b * 128 + (warp & 3) * 32 + lane;
-          if (dcol < a.d) {
-            float4* dst = reinterpret_cast<float4*>(Pd + static_cast<int64_t>(dcol) * K);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bar[S_D1EMPTY0 + buf]);
+          const int64_t grow = run.row0 + static_cast<int64_t>(t) * kBM + r;
+          const bool valid = grow < run.row1;
+          const float sc = valid ? a.scales[grow] : 0.f;
+          if (!valid) {
+#pragma unroll
+            for (int j = 0; j < K; ++j) w[j] = 0.f;
+          }
+          if (CL > 1) {
+            const uint32_t rows_bytes = static_cast<uint32_t>(RPC * K * 4);
+            if (!(ok = epi_sync())) break;
 #pragma unroll
             for (int j = 0; j < K; j += 4)
-              dst[j / 4] = make_float4(a.smax2 * y[j], a.smax2 * y[j + 1], a.smax2 * y[j + 2], a.smax2 * y[j + 3]);
+              *reinterpret_cast<float4*>(sW + wpos<K>(r, j)) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
+            fence_async_smem();
+            if (!(ok = epi_sync())) break;
+            if (r == 0) {
+              mbar_expect_tx(&bar[S_REDFULL], (CL - 1) * rows_bytes);
+              for (uint32_t o = 0; o < CL; ++o)
+                if (o != crank)
+                  bulk_s2s_cluster(mapa(su32(sWrecv + crank * RPC * K), o), su32(sW + o * RPC * K), rows_bytes,
+                                   mapa(su32(&bar[S_REDFULL]), o));
+              bulk_commit();
+              bulk_wait_read0();
+            }
+            if (!(ok = wait(S_REDFULL, Tg & 1, true))) break;
+            const int per = RPC * K / kBM;
+            for (int e = 0; e < per; ++e) {
+              const int idx = r * per + e, rl = idx / K, col = idx % K;
+              const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
+              const int rel = own - static_cast<int>(crank) * RPC * K;
+              float sum = 0.f;
+              for (uint32_t src = 0; src < CL; ++src) sum += src == crank ? sW[own] : sWrecv[src * RPC * K + rel];
+              sW[own] = sum;
+            }
+            fence_async_smem();
+            if (!(ok = epi_sync())) break;
+            if (r == 0) {
+              mbar_expect_tx(&bar[S_WFULL], (CL - 1) * rows_bytes);
+              for (uint32_t dst = 0; dst < CL; ++dst)
+                if (dst != crank)
+                  bulk_s2s_cluster(mapa(su32(sW + crank * RPC * K), dst), su32(sW + crank * RPC * K), rows_bytes,
+                                   mapa(su32(&bar[S_WFULL]), dst));
+              bulk_commit();
+              bulk_wait_read0();
+            }
+            if (!(ok = wait(S_WFULL, Tg & 1, true))) break;
+#pragma unroll
+            for (int j = 0; j < K; j += 4) {
+              const float4 v = *reinterpret_cast<const float4*>(sW + wpos<K>(r, j));
+              w[j] = v.x;
+              w[j + 1] = v.y;
+              w[j + 2] = v.z;
+              w[j + 3] = v.w;
+            }
           }
+          // row scale: W_r <- W_r s_r^2 / S (so the FP16 operand cannot overflow)
+          const float f = sc * sc / a.smax2;
+#pragma unroll
+          for (int j = 0; j < K; ++j) w[j] *= f;
+          if (!(ok = wait(S_B2FREE0 + static_cast<int>(wb), ((Tg >> 1) + 1) & 1, false))) break;
+          unsigned char* B2 = sB2 + wb * B2BUF;
+#pragma unroll
+          for (int j = 0; j < K; ++j) {
+            const uint16_t hi = f16_bits(w[j]);
+            const uint16_t lo = f16_bits(w[j] - f16_val(hi));
+            *reinterpret_cast<uint16_t*>(B2 + sw128_off(j, r, N)) = hi;
+            *reinterpret_cast<uint16_t*>(B2 + sw128_off(K + j, r, N)) = lo;
+          }
+          fence_async_smem();
+          mbar_arrive(&bar[S_B2FULL0 + wb]);
+          if (t % TP == TP - 1 || t == run.ntiles - 1) ok = drain(t / TP);
         }
-        tc_fence_before();
       }
+      T += run.ntiles;
+      pieces += Walk8::pieces_of(run.ntiles);
+      si = run.sj;
     }
-    T += ntiles;
-    G += 2u * static_cast<uint32_t>(ntiles) * static_cast<uint32_t>(U);
   }
 
-  // ---- teardown: copies landed (after an abort), MMAs retired, no remote traffic, then free TMEM
-  if (warp == 0 && lane == 0) {
-    for (uint32_t q = g_prod_end > static_cast<uint32_t>(R8) ? g_prod_end - R8 : 0; q < g_prod_end; ++q) {
-      const uint32_t addr = su32(&bar[S_STG0 + q % R8]);
-      const long long t0 = clock64();
-      while (!mbar_try(addr, (q / R8) & 1) && clock64() - t0 < kTimeoutCycles) {
-      }
-    }
-  }
-  if (warp == 1 && lane == 0) mma_commit(&bar[S_DONE]);
+  // ---- teardown: MMAs retired, no remote traffic, then free TMEM
+  if (warp >= kIssue1 && lane == 0) mma_commit(&bar[S_DONE]);
   __syncthreads();
   if (warp == 0) {
     const uint32_t addr = su32(&bar[S_DONE]);
@@ -483,8 +630,7 @@ cudaError_t launch_tcs8_t(const TcsPlan& p, const Tcs8Args& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = tcs8_config<K>(static_cast<unsigned>(p.nclusters * p.cluster), p.cluster, p.smem, s, attr);
-  const CUtensorMap* m0 = reinterpret_cast<const CUtensorMap*>(p.tmap[0]);
-  return cudaLaunchKernelEx(&cfg, step_tcs8_kernel<K>, *m0, a);
+  return cudaLaunchKernelEx(&cfg, step_tcs8_kernel<K>, a);
 }
 
 }  // namespace
@@ -494,8 +640,7 @@ bool tcs8_plan_slice(int d, int k, int sms, const TcsTuning& tune, int ncd_max, 
 }  // namespace
 
 // Without a slice width from the tuning, the widest slice that has a plan (fewest
-// CTAs per cluster, least W exchange; measured at d = 2,048, k = 32: 512-column
-// slices with two staging units beat 256-column slices with four).
+// CTAs per cluster, least W exchange).
 bool tcs8_plan(int d, int k, int sms, const TcsTuning& tune, TcsPlan* p) {
   const int K = k <= 8 ? 8 : (k <= 16 ? 16 : 32);
   if (tune.slice_cols >= 128) return tcs8_plan_slice(d, k, sms, tune, (tune.slice_cols / 128) * 2, p);
@@ -520,32 +665,33 @@ bool tcs8_plan_slice(int d, int k, int sms, const TcsTuning& tune, int ncd_max, 
   const uint32_t W = cl > 1 ? 128u * K * 4 : 0u;
   const uint32_t bars = kNumBars8 * 8 + 16;
   const int avail = kSmemLimit - 1024 - static_cast<int>(B1 + B2 + 2 * W + bars);
-  // operand ring of 32 KB units (two suffice: the converters fill it as fast as the
-  // MMAs drain it), the rest to the staging ring that covers load latency
-  int ring = 2;
-  if (tune.ring_units > 0 && tune.ring_units < ring) ring = tune.ring_units;
-  int stage = (avail - ring * kUnitBytes) / kStageBytes;
-  if (stage > kMaxRing) stage = kMaxRing;
-  if (stage < 2 || ring < 2) return false;
+  // operand ring of 32 KB units: three at least (the narrower slices' plans start there), up
+  // to four (the converters' registers hold the units in flight, the ring only what
+  // the MMAs read)
+  int ring = avail / kUnitBytes;
+  if (ring < 3 || tune.ring_units == 1) return false;
+  if (ring > 4) ring = 4;
+  if (tune.ring_units > 0 && ring > tune.ring_units) ring = tune.ring_units;
   p->K = K;
   p->planes = 1;
   p->ncd = ncd;
   p->cluster = cl;
   p->ring = ring;
-  p->stage = stage;
   int lag = tune.lag_units > 0 ? tune.lag_units : (cl > 1 ? 4 : 2);
   const int U = ncd / 2;
   p->lag = lag < U ? lag : U;
   p->prefetch = 0;
   p->hints = 1;  // first pass evict_last, second pass evict_first
-  p->off_stage = static_cast<uint32_t>(ring) * kUnitBytes;
-  p->off_B1 = p->off_stage + static_cast<uint32_t>(stage) * kStageBytes;
+  p->off_B1 = static_cast<uint32_t>(ring) * kUnitBytes;
   p->off_B2 = p->off_B1 + B1;
   p->off_W = p->off_B2 + B2;
   p->off_Wrecv = p->off_W + W;
   p->off_bar = p->off_Wrecv + W;
   p->smem = p->off_bar + bars + 1024;
-  const uint32_t used = static_cast<uint32_t>(2 * N + U * N);
+  // a second tile between the passes where W crosses a cluster and tensor memory holds
+  // three D1
+  p->behind = cl > 1 && 3 * N + U * N <= 512 ? 2 : 1;
+  const uint32_t used = static_cast<uint32_t>((p->behind + 1) * N + U * N);
   uint32_t cols = 32;
   while (cols < used) cols *= 2;
   if (cols > 512) return false;
@@ -560,29 +706,13 @@ bool tcs8_plan_slice(int d, int k, int sms, const TcsTuning& tune, int ncd_max, 
 }
 }  // namespace
 
-cudaError_t tcs8_encode_map(const void* codes, int64_t n, int d, int64_t ld, TcsPlan* p) {
-  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-  if (!encode) {
-    cudaDriverEntryPointQueryResult q;
-    void* fn = nullptr;
-    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
-    if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-  }
-  cuuint64_t dims[2] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(n)};
-  cuuint64_t strides[1] = {static_cast<cuuint64_t>(ld)};
-  cuuint32_t box[2] = {128, static_cast<cuuint32_t>(kBM)};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = encode(reinterpret_cast<CUtensorMap*>(p->tmap[0]), CU_TENSOR_MAP_DATA_TYPE_UINT8, 2,
-                      const_cast<void*>(codes), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
-cudaError_t launch_step_tcs8(const TcsPlan& p, const Segment* segs, const int* seg_ptr, const float* Z,
-                             int64_t z_stride, float* P, int d, const float* scales, float smax2, int* status,
-                             cudaStream_t s) {
+cudaError_t launch_step_tcs8(const TcsPlan& p, const void* codes, int64_t n, int64_t ld, const Segment* segs,
+                             const int* seg_ptr, const float* Z, int64_t z_stride, float* P, int d, const float* scales,
+                             float smax2, int* status, cudaStream_t s) {
   Tcs8Args a;
+  a.codes = static_cast<const unsigned char*>(codes);
+  a.n = n;
+  a.ld = ld;
   a.segs = segs;
   a.seg_ptr = seg_ptr;
   a.Z = Z;
@@ -594,10 +724,9 @@ cudaError_t launch_step_tcs8(const TcsPlan& p, const Segment* segs, const int* s
   a.smax2 = smax2;
   a.ncd = p.ncd;
   a.ring = p.ring;
-  a.stage = p.stage;
   a.lag = p.lag;
+  a.behind = p.behind;
   a.hints = p.hints;
-  a.off_stage = p.off_stage;
   a.off_B1 = p.off_B1;
   a.off_B2 = p.off_B2;
   a.off_W = p.off_W;
