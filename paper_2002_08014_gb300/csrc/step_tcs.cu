@@ -357,7 +357,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           // back the same way.  A buffer is rewritten only after the waits show
           // its previous contents were consumed.
           const uint32_t rows_bytes = static_cast<uint32_t>(RPC * K * 4);
-          if (!(ok = epi_sync())) break;  // the previous tile's bulk copies have read sW (r == 0 waited)
+          if (r == 0) bulk_wait_read0();  // the previous tile's copies have read sW
+          if (!(ok = epi_sync())) break;
 #pragma unroll
           for (int j = 0; j < K; j += 4)
             *reinterpret_cast<float4*>(sW + wpos<K>(r, j)) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
@@ -370,18 +371,38 @@ __global__ void __launch_bounds__(kThreads, 1)
                 bulk_s2s_cluster(mapa(su32(sWrecv + crank * RPC * K), o), su32(sW + o * RPC * K), rows_bytes,
                                  mapa(su32(&bar[S_REDFULL]), o));
             bulk_commit();
-            bulk_wait_read0();
           }
           if (!(ok = wait(S_REDFULL, Tg & 1, true))) break;
-          const int per = RPC * K / kBM;  // values per epilogue thread (K / CL)
-          for (int e = 0; e < per; ++e) {
-            const int idx = r * per + e, rl = idx / K, col = idx % K;
-            const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
-            const int rel = own - static_cast<int>(crank) * RPC * K;  // offset inside one owner's row block
-            float sum = 0.f;
-            for (uint32_t src = 0; src < CL; ++src)
-              sum += src == crank ? sW[own] : sWrecv[src * RPC * K + rel];
-            sW[own] = sum;
+          const int per = RPC * K / kBM;  // values per epilogue thread (K / CL), neighbours in a row
+          // partials in source-rank order; four columns at a time where a thread has them
+          if (per % 4 == 0) {
+            for (int e = 0; e < per; e += 4) {
+              const int idx = r * per + e, rl = idx / K, col = idx % K;
+              const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
+              const int rel = own - static_cast<int>(crank) * RPC * K;  // offset inside one owner's row block
+              float4 v[8], sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+              for (uint32_t src = 0; src < 8; ++src)
+                if (src < CL) v[src] = *reinterpret_cast<const float4*>(src == crank ? sW + own : sWrecv + src * RPC * K + rel);
+#pragma unroll
+              for (uint32_t src = 0; src < 8; ++src)
+                if (src < CL) {
+                  sum.x += v[src].x;
+                  sum.y += v[src].y;
+                  sum.z += v[src].z;
+                  sum.w += v[src].w;
+                }
+              *reinterpret_cast<float4*>(sW + own) = sum;
+            }
+          } else {
+            for (int e = 0; e < per; ++e) {
+              const int idx = r * per + e, rl = idx / K, col = idx % K;
+              const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
+              const int rel = own - static_cast<int>(crank) * RPC * K;
+              float sum = 0.f;
+              for (uint32_t src = 0; src < CL; ++src) sum += src == crank ? sW[own] : sWrecv[src * RPC * K + rel];
+              sW[own] = sum;
+            }
           }
           fence_async_smem();
           if (!(ok = epi_sync())) break;
@@ -392,7 +413,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 bulk_s2s_cluster(mapa(su32(sW + crank * RPC * K), dst), su32(sW + crank * RPC * K), rows_bytes,
                                  mapa(su32(&bar[S_WFULL]), dst));
             bulk_commit();
-            bulk_wait_read0();
           }
           if (!(ok = wait(S_WFULL, Tg & 1, true))) break;
 #pragma unroll
@@ -461,6 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   }
+  if (tid == 4 * 32) bulk_wait_read0();  // the epilogue's last copies have read shared memory
   // ---- teardown: all MMAs retired, no remote traffic in flight, then free TMEM
   if (issuer) mma_commit(&bar[S_DONE]);
   __syncthreads();

@@ -8,10 +8,10 @@
 // the codes.  Every E4M3 value is exactly an FP16 value (3 significand bits,
 // exponents 2^-9 .. 2^8), and one cvt.rn.f16x2.e4m3x2 turns two codes into two
 // FP16, so:
-//   * eight converter warps read each 128-row x 128-column unit of codes (16 KB)
-//     straight into registers, kDepth units ahead, widen it and write the FP16
-//     operand layout the MMAs read (SWIZZLE_128B, K-major, 32 KB per unit) into the
-//     operand ring;
+//   * two groups of four converter warps, one for each pass, take 128-row x 128-column
+//     units of codes (16 KB): straight into registers, kDepth units ahead, widened and
+//     written in the FP16 operand layout the MMAs read (SWIZZLE_128B, K-major, 32 KB per
+//     unit) into the operand ring;
 //   * first pass  D1 += Q_u [Z_hi | Z_lo]  (kind::f16 with FP16 operands; Z
 //     split into FP16 hi + lo, 22 significand bits between them);
 //   * epilogue    W = D1[:, :K] + D1[:, K:] (cluster-summed), then row r scaled
@@ -25,13 +25,20 @@
 // What bounds it.  Z, the W operands and the exchange buffers leave about 96 KB of
 // shared memory at d = 2,048, k = 32.  With the codes staged there by TMA (two 16 KB
 // slots beside two operand slots) both passes together had 32 KB in flight and every
-// unit crossed shared memory twice; the launch took 2,150 us at n = 1M.  In registers
-// the codes in flight cost no shared memory (48 KB at kDepth = 3) and the operand ring
-// has three slots.  The second pass of a tile runs two tiles behind the first where
-// tensor memory holds a third D1, so that the cluster exchange of W (about 3 us, as
-// long as the first pass of a whole tile) is off the chain.
+// unit crossed shared memory twice: 2,150 us a launch at n = 1M.  In registers the
+// codes in flight cost no shared memory (64 KB at kDepth = 2) and the operand ring has
+// three slots; a converter group for each pass overlaps the latencies of two units
+// (one group of eight warps spent 1,450 cycles on each); roles step through their own
+// units in closed form; the second pass runs two tiles behind the first where tensor
+// memory holds a third D1, which takes the cluster exchange of W off the chain; and the
+// exchange itself adds four columns at a time and waits for its copies only before it
+// rewrites their source (12,000 -> 9,000 cycles a tile).  1,190 us at n = 1M, 1.7 TB/s of
+// codes; n = 262,144: 456 -> 334 us over these steps, 123 -> 94 at d = 512 without a
+// cluster.  A group still takes about 2,500 cycles a unit (widening 640, issuing its
+// loads up to 600, the fence 90, the rest waiting for slots and data), three times what
+// the conversion pipe needs.
 //
-// Roles (448 threads): warps 0-3 and 8-11 convert; warps 4-7 run the epilogue; lane 0
+// Roles (448 threads): warps 0-3 and 8-11 convert (first and second pass); warps 4-7 run the epilogue; lane 0
 // of warps 12 and 13 issue the first and the second pass's MMAs (one thread issues a
 // small-N MMA only every ~55 cycles, ~100 when it polls barriers in between); warps
 // 4-7, 12 and 13 stage Z when the partition changes, while the converters go on.
@@ -48,10 +55,10 @@ namespace {
 using namespace tc;
 
 constexpr int kThreads8 = 448;
-constexpr int kConvThreads = 256;            // warps 0-3 and 8-11
-constexpr int kIssue1 = 12, kIssue2 = 13;    // warps whose lane 0 issues the first / second pass
+constexpr int kConvThreads = 256;            // warps 0-3 and 8-11, two groups
+constexpr int kIssue1 = 12;                  // lane 0 of this warp issues the first pass, of the next one the second
 constexpr int kOthers8 = kThreads8 - kConvThreads;
-constexpr int kDepth = 3;                    // units of codes in flight per converter thread
+constexpr int kDepth = 2;                    // units of codes in flight per converter group
 constexpr int kUnitBytes = 2 * kChunkBytes;  // 128 rows x 128 columns of FP16 (two 64-column chunks)
 constexpr int kMaxRing = 8;
 constexpr int kMaxD1 = 3;                    // D1 buffers
@@ -101,61 +108,34 @@ __device__ __forceinline__ Run8 run_at(const Segment* segs, int si, int se) {
   return r;
 }
 
-// The unit order of a cluster, walked by every role: within a run, the first pass of
-// tile t (units 0 .. U-1) interleaved with the second pass of tile t - behind, `lag`
-// units later.
-struct Walk8 {
-  const Segment* segs;
-  int se, U, lag, behind;
-  Run8 run;
-  uint32_t T = 0;       // tiles before the run
-  uint32_t pieces = 0;  // pieces before the run
-  int t = 0, u = -1, half = 1;
-  // the unit
-  bool second = false;
-  int tile = 0, blk = 0;
-  bool new_run = true;
-  __device__ Walk8(const Segment* s, int sb, int se_, int U_, int lag_, int behind_)
-      : segs(s), se(se_), U(U_), lag(lag_), behind(behind_) {
-    run = run_at(segs, sb, se);
+// The order of a run's units in the ring: the first pass of tile t (blocks 0 .. U-1)
+// interleaved with the second pass of tile t - behind, `lag` blocks later.  In closed
+// form, so that each role steps through its own units only (walking the whole order
+// cost an issuing thread some 300 cycles a unit).
+struct Order8 {
+  int U, lag, behind;
+  // units of the run before tile t's turn
+  __device__ __forceinline__ uint32_t before(int t, int ntiles) const {
+    return static_cast<uint32_t>(U * (min(t, ntiles) + max(0, t - behind)));
   }
-  __device__ static int pieces_of(int ntiles) {
-    constexpr int TP = static_cast<int>(kTcChainRows / kBM);
-    return (ntiles + TP - 1) / TP;
+  __device__ __forceinline__ uint32_t first(int t, int u, int ntiles) const {
+    return before(t, ntiles) + u + (t >= behind ? max(0, u - lag) : 0);
   }
-  // moves to the next unit; false after the last
-  __device__ bool next() {
-    new_run = false;
-    while (true) {
-      if (half == 0) {
-        half = 1;
-      } else {
-        half = 0;
-        if (++u == U + lag) {
-          u = 0;
-          if (++t == run.ntiles + behind) {
-            T += run.ntiles;
-            pieces += pieces_of(run.ntiles);
-            if (run.sj >= se) return false;
-            run = run_at(segs, run.sj, se);
-            t = 0;
-            new_run = true;
-          }
-        }
-      }
-      if (half == 0) {
-        if (t < run.ntiles && u < U) {
-          second = false;
-          tile = t;
-          blk = u;
-          return true;
-        }
-      } else if (t >= behind && u >= lag && u - lag < U) {
-        second = true;
-        tile = t - behind;
-        blk = u - lag;
-        return true;
-      }
+  __device__ __forceinline__ uint32_t second(int tile, int v, int ntiles) const {
+    const int t = tile + behind;
+    return before(t, ntiles) + (t < ntiles ? min(v + lag + 1, U) : 0) + v;
+  }
+};
+
+// A role's place in the ring: unit g sits in slot g mod R, its fill's number is g / R.
+struct Place8 {
+  uint32_t g = 0, slot = 0, fill = 0;
+  __device__ __forceinline__ void to(uint32_t next, uint32_t R) {
+    slot += next - g;
+    g = next;
+    while (slot >= R) {
+      slot -= R;
+      ++fill;
     }
   }
 };
@@ -166,10 +146,11 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, bool a_mn_major, 
          (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
 }
 
-__device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t two_codes) {
-  uint32_t r;
-  asm("{ .reg .b16 t; cvt.u16.u32 t, %1; cvt.rn.f16x2.e4m3x2 %0, t; }" : "=r"(r) : "r"(two_codes));
-  return r;
+// Four codes -> four FP16 in order.
+__device__ __forceinline__ void e4m3x4_to_f16x4(uint32_t codes, uint32_t& lo, uint32_t& hi) {
+  asm("{ .reg .b16 a, b; mov.b32 {a, b}, %2; cvt.rn.f16x2.e4m3x2 %0, a; cvt.rn.f16x2.e4m3x2 %1, b; }"
+      : "=r"(lo), "=r"(hi)
+      : "r"(codes));
 }
 
 __device__ __forceinline__ uint16_t f16_bits(float x) { return __half_as_ushort(__float2half_rn(x)); }
@@ -203,7 +184,7 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
   const int R = a.ring;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar + kNumBars8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  volatile uint32_t* filled = tmem_holder + 2;  // units the converters have begun to fill
+  volatile uint32_t* fills = tmem_holder + 4;  // per slot: fills begun
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t crank = cluster_rank();
@@ -231,11 +212,11 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
     mbar_init(&bar[S_DONE], 2);
     mbar_init(&bar[S_EPI], 128);
     for (int s = 0; s < kMaxRing; ++s) {
-      mbar_init(&bar[S_RING0 + s], kConvThreads / 32);  // one arrival per converter warp
+      mbar_init(&bar[S_RING0 + s], kConvThreads / 64);  // one arrival per warp of the group
       mbar_init(&bar[S_RING0 + kMaxRing + s], 1);        // MMA commit
     }
     *abort_flag = 0;
-    *filled = 0;
+    for (int s = 0; s < kMaxRing; ++s) fills[s] = 0;
     fence_mbar_init();
   }
   if (warp == 0) {
@@ -267,12 +248,13 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
       }
     }
   };
-  // Both issuers take units from one ring; before a parity wait on a slot an issuer sees
-  // that its unit's fill has begun, i.e. that the fill before was consumed (a wait a fill
-  // early would succeed at once).
-  auto wait_filled = [&](uint32_t g) -> bool {
+  // Both issuers and both converter groups share one ring in unit order; before a parity
+  // wait on a slot they see that enough of its fills have begun, i.e. that the phase
+  // before the one they wait for is over (a wait a phase early would succeed at once).
+  auto wait_fills = [&](uint32_t slot, uint32_t count) -> bool {
+    if (fills[slot] >= count) return true;
     const long long t0 = clock64();
-    while (*filled <= g) {
+    while (fills[slot] < count) {
       if (*abort_flag) return false;
       if (clock64() - t0 > kTimeoutCycles) {
         give_up();
@@ -281,6 +263,7 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
     }
     return true;
   };
+  const Order8 order{U, a.lag, a.behind};
 
   constexpr uint32_t idesc1 = idesc_f16(128, N, false, false);
   constexpr uint32_t idesc2 = idesc_f16(128, N, true, false);
@@ -291,80 +274,90 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
     // no rows: straight to the teardown
   } else if (converter) {
     // -------------------------------------------------------------- converters: codes -> FP16 operand
-    const int ct = warp < 4 ? tid : tid - 128;  // 0 .. 255
-    const int col16 = ct & 7, row8 = ct >> 3;   // 16 codes of row row8 + 32 i
-    uint64_t pol_keep = l2_policy_evict_last(), pol_drop = l2_policy_evict_first();
-    if (!a.hints) pol_drop = pol_keep;
-    uint4 buf[kDepth][4];
-    Walk8 ahead(a.segs, sb, se, U, a.lag, a.behind);
+    // thread: 16 codes at (lane & 3) of either 64-column chunk, rows 8 (warp mod 4) +
+    // (lane >> 2) + 32 i; eight lanes write two rows of four 16-byte pieces, all eight
+    // bank groups
+    const uint32_t grp = warp < 4 ? 0 : 1;
+    const int row0 = 8 * (warp & 3) + (lane >> 2);
+    const uint32_t at0 = row0 * 128 + (((2 * (lane & 3)) ^ (lane >> 2)) << 4);
+    const uint32_t at1 = row0 * 128 + (((2 * (lane & 3) + 1) ^ (lane >> 2)) << 4);
+    const uint64_t pol = grp == 0 || !a.hints ? l2_policy_evict_last() : l2_policy_evict_first();
+    uint4 buf[kDepth][8];
+    uint32_t unit[kDepth];  // the unit in buf[x]; ~0: none left
+    Run8 run = run_at(a.segs, sb, se);
+    uint32_t base_g = 0;  // units before the run
+    int t = 0, u = 0;
     bool more = true;
-    auto fetch = [&](uint4 (&v)[4]) {
-      if (more) more = ahead.next();
-      const int64_t r0 = ahead.run.row0 + static_cast<int64_t>(ahead.tile) * kBM + row8;
-      const int c = c0 + 128 * ahead.blk + 16 * col16;
+    // the next unit of this group's pass into v
+    auto fetch = [&](uint4 (&v)[8]) -> uint32_t {
+      if (!more) return ~0u;
+      const uint32_t g = base_g + (grp == 0 ? order.first(t, u, run.ntiles) : order.second(t, u, run.ntiles));
+      const int64_t r0 = run.row0 + static_cast<int64_t>(t) * kBM + row0;
+      const int c = c0 + 128 * u + 16 * (lane & 3);
       const unsigned char* p = a.codes + r0 * a.ld + c;
+      const int64_t step = 32 * a.ld;
+      if (r0 - row0 + kBM <= a.n && c0 + 128 * (u + 1) <= a.ld) {  // the whole unit lies in the matrix
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        v[i] = more && c < a.ld && r0 + 32 * i < a.n ? ld_codes(p + static_cast<int64_t>(32 * i) * a.ld,
-                                                                 ahead.second ? pol_drop : pol_keep)
-                                                     : make_uint4(0u, 0u, 0u, 0u);
+        for (int i = 0; i < 8; i += 2, p += step) {
+          v[i] = ld_codes(p, pol);
+          v[i + 1] = ld_codes(p + 64, pol);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          v[i] = c + 64 * (i & 1) < a.ld && r0 + 32 * (i >> 1) < a.n ? ld_codes(p + (i >> 1) * step + 64 * (i & 1), pol)
+                                                                   : make_uint4(0u, 0u, 0u, 0u);
+      }
+      if (++u == U) {
+        u = 0;
+        if (++t == run.ntiles) {
+          t = 0;
+          base_g += 2u * static_cast<uint32_t>(run.ntiles) * static_cast<uint32_t>(U);
+          more = run.sj < se;
+          if (more) run = run_at(a.segs, run.sj, se);
+        }
+      }
+      return g;
     };
-    // units in all: two passes over every tile's U units
-    uint32_t total = 0;
-    for (int si = sb; si < se;) {
-      const Run8 r = run_at(a.segs, si, se);
-      total += 2u * static_cast<uint32_t>(r.ntiles) * static_cast<uint32_t>(U);
-      si = r.sj;
-    }
 #pragma unroll
-    for (int x = 0; x < kDepth; ++x) fetch(buf[x]);
-    uint32_t slot = 0, phase = 0;
+    for (int x = 0; x < kDepth; ++x) unit[x] = fetch(buf[x]);
+    Place8 at;
     bool ok = true;
-    for (uint32_t g0 = 0; ok && g0 < total; g0 += kDepth) {
+    while (ok && unit[0] != ~0u) {
 #pragma unroll
       for (int x = 0; x < kDepth; ++x) {
-        if (!ok || g0 + x >= total) continue;
-        if (!(ok = wait(S_RING0 + kMaxRing + static_cast<int>(slot), phase ^ 1, false))) continue;
-        if (ct == 0) *filled = g0 + x + 1;
-        unsigned char* dst = sRing + slot * kUnitBytes + (col16 >> 2) * kChunkBytes;
+        if (!ok || unit[x] == ~0u) continue;
+        at.to(unit[x], R);
+        if (!(ok = wait_fills(at.slot, at.fill) &&
+                   wait(S_RING0 + kMaxRing + static_cast<int>(at.slot), (at.fill & 1) ^ 1, false)))
+          continue;
+        __syncwarp();
+        if ((warp & 3) == 0 && lane == 0) fills[at.slot] = at.fill + 1;
+        unsigned char* dst = sRing + at.slot * kUnitBytes;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int r = row8 + 32 * i;
+        for (int i = 0; i < 8; ++i) {
           const uint4 v = buf[x][i];
-          uint4 h[2];
-          h[0].x = e4m3x2_to_f16x2(v.x & 0xFFFFu);
-          h[0].y = e4m3x2_to_f16x2(v.x >> 16);
-          h[0].z = e4m3x2_to_f16x2(v.y & 0xFFFFu);
-          h[0].w = e4m3x2_to_f16x2(v.y >> 16);
-          h[1].x = e4m3x2_to_f16x2(v.z & 0xFFFFu);
-          h[1].y = e4m3x2_to_f16x2(v.z >> 16);
-          h[1].z = e4m3x2_to_f16x2(v.w & 0xFFFFu);
-          h[1].w = e4m3x2_to_f16x2(v.w >> 16);
-          // the two chunks' halves in opposite order: the eight lanes of a row hit eight bank groups
-          const int flip = col16 >> 2;
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const int hf = q ^ flip, c8 = 2 * (col16 & 3) + hf;
-            *reinterpret_cast<uint4*>(dst + r * 128 + ((c8 ^ (r & 7)) << 4)) = hf ? h[1] : h[0];
-          }
+          uint4 h0, h1;
+          e4m3x4_to_f16x4(v.x, h0.x, h0.y);
+          e4m3x4_to_f16x4(v.y, h0.z, h0.w);
+          e4m3x4_to_f16x4(v.z, h1.x, h1.y);
+          e4m3x4_to_f16x4(v.w, h1.z, h1.w);
+          unsigned char* q = dst + (i & 1) * kChunkBytes + (i >> 1) * 32 * 128;
+          *reinterpret_cast<uint4*>(q + at0) = h0;
+          *reinterpret_cast<uint4*>(q + at1) = h1;
         }
-        fetch(buf[x]);
         fence_async_smem();  // the MMAs read these tiles through the async proxy
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bar[S_RING0 + slot]);
-        if (++slot == static_cast<uint32_t>(R)) {
-          slot = 0;
-          phase ^= 1;
-        }
+        if (lane == 0) mbar_arrive(&bar[S_RING0 + at.slot]);
+        unit[x] = fetch(buf[x]);
       }
     }
   } else {
     // -------------------------------------------------------------- issuers and epilogue, run by run
     const int ot = warp < 8 ? tid - 128 : tid - 384 + 128;  // 0 .. kOthers8 - 1
     uint32_t T = 0, pieces = 0, epi_phase = 0;
-    uint32_t unit = 0, slot = 0, phase = 0;
-    Walk8 walk(a.segs, sb, se, U, a.lag, a.behind);
-    bool more = walk.next();
+    uint32_t base_g = 0;  // units before the run
+    Place8 at;
     for (int si = sb; si < se;) {
       const Run8 run = run_at(a.segs, si, se);
       __syncwarp();
@@ -379,59 +372,58 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
       if (warp >= kIssue1) {
         if (lane == 0) {
           // ---------------------------------------------------------- MMA issuers (one per pass)
-          const bool mine2 = warp == kIssue2;
           bool ok = true;
-          bool first_of_run = true;
-          while (more && (first_of_run || !walk.new_run)) {
-            first_of_run = false;
-            const uint32_t g = unit, s = slot, ph = phase;
-            const int t = walk.tile, u = walk.blk;
-            const bool second = walk.second;
-            ++unit;
-            if (++slot == static_cast<uint32_t>(R)) {
-              slot = 0;
-              phase ^= 1;
+          auto ready = [&](uint32_t g) -> bool {
+            at.to(base_g + g, R);
+            return wait_fills(at.slot, at.fill + 1) && wait(S_RING0 + static_cast<int>(at.slot), at.fill & 1, false);
+          };
+          if (warp == kIssue1) {
+            const uint32_t bS = su32(sB1);
+            uint32_t buf = T % ND1, use = T / ND1;
+            for (int t = 0; ok && t < run.ntiles; ++t) {
+              if (!(ok = wait(S_D1EMPTY0 + static_cast<int>(buf), (use + 1) & 1, false))) break;
+              for (int u = 0; u < U; ++u) {
+                if (!(ok = ready(order.first(t, u, run.ntiles)))) break;
+                tc_fence_after();
+                const uint32_t aS = su32(sRing + at.slot * kUnitBytes);
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+#pragma unroll
+                  for (int kk = 0; kk < 4; ++kk) {
+                    const uint64_t ad = sdesc(aS + j * kChunkBytes + kk * 32, 16, 1024);
+                    const uint64_t bd = sdesc(bS + (2 * u + j) * N * 128 + kk * 32, 16, 1024);
+                    mma_bf16(tmem + buf * N, ad, bd, idesc1, (u | j | kk) != 0);
+                  }
+                mma_commit(&bar[S_RING0 + kMaxRing + at.slot]);
+              }
+              if (ok) mma_commit(&bar[S_D1FULL0 + buf]);
+              if (++buf == static_cast<uint32_t>(ND1)) {
+                buf = 0;
+                ++use;
+              }
             }
-            more = walk.next();
-            if (second != mine2 || !ok) continue;
-            const uint32_t Tg = T + t;
-            if (!(ok = wait_filled(g) && wait(S_RING0 + static_cast<int>(s), ph, false))) continue;
-            const uint32_t aS = su32(sRing + s * kUnitBytes);
-            if (!second) {
-              const uint32_t buf = Tg % ND1;
-              if (u == 0 && !(ok = wait(S_D1EMPTY0 + static_cast<int>(buf), ((Tg / ND1) + 1) & 1, false))) continue;
-              tc_fence_after();
-              const uint32_t bS = su32(sB1);
-#pragma unroll
-              for (int j = 0; j < 2; ++j)
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                  const uint64_t ad = sdesc(aS + j * kChunkBytes + kk * 32, 16, 1024);
-                  const uint64_t bd = sdesc(bS + (2 * u + j) * N * 128 + kk * 32, 16, 1024);
-                  mma_bf16(tmem + buf * N, ad, bd, idesc1, (u | j | kk) != 0);
-                }
-              mma_commit(&bar[S_RING0 + kMaxRing + s]);
-              if (u == U - 1) mma_commit(&bar[S_D1FULL0 + buf]);
-            } else {
-              const uint32_t buf = Tg & 1;
-              if (u == 0) {
-                if (!(ok = wait(S_B2FULL0 + static_cast<int>(buf), (Tg >> 1) & 1, false))) continue;
-                // a new piece accumulates from zero: the previous one's sums have been read out
-                if (t % TP == 0 && !(ok = wait(S_D2EMPTY, (pieces + t / TP + 1) & 1, false))) continue;
-              }
-              tc_fence_after();
+          } else {
+            for (int t = 0; ok && t < run.ntiles; ++t) {
+              const uint32_t Tg = T + t, buf = Tg & 1;
+              if (!(ok = wait(S_B2FULL0 + static_cast<int>(buf), (Tg >> 1) & 1, false))) break;
+              // a new piece accumulates from zero: the previous one's sums have been read out
+              if (t % TP == 0 && !(ok = wait(S_D2EMPTY, (pieces + t / TP + 1) & 1, false))) break;
               const uint32_t bS = su32(sB2 + buf * B2BUF);
+              for (int u = 0; u < U; ++u) {
+                if (!(ok = ready(order.second(t, u, run.ntiles)))) break;
+                tc_fence_after();
+                const uint32_t aS = su32(sRing + at.slot * kUnitBytes);
 #pragma unroll
-              for (int kk = 0; kk < 8; ++kk) {
-                const uint64_t ad = sdesc(aS + kk * 2048, kChunkBytes, 1024);
-                const uint64_t bd = sdesc(bS + (kk >> 2) * N * 128 + (kk & 3) * 32, 16, 1024);
-                mma_bf16(tD2 + u * N, ad, bd, idesc2, (t % TP == 0 && kk == 0) ? 0u : 1u);
+                for (int kk = 0; kk < 8; ++kk) {
+                  const uint64_t ad = sdesc(aS + kk * 2048, kChunkBytes, 1024);
+                  const uint64_t bd = sdesc(bS + (kk >> 2) * N * 128 + (kk & 3) * 32, 16, 1024);
+                  mma_bf16(tD2 + u * N, ad, bd, idesc2, (t % TP == 0 && kk == 0) ? 0u : 1u);
+                }
+                mma_commit(&bar[S_RING0 + kMaxRing + at.slot]);
               }
-              mma_commit(&bar[S_RING0 + kMaxRing + s]);
-              if (u == U - 1) {
-                mma_commit(&bar[S_B2FREE0 + buf]);
-                if (t % TP == TP - 1 || t == run.ntiles - 1) mma_commit(&bar[S_D2FULL]);
-              }
+              if (!ok) break;
+              mma_commit(&bar[S_B2FREE0 + buf]);
+              if (t % TP == TP - 1 || t == run.ntiles - 1) mma_commit(&bar[S_D2FULL]);
             }
           }
           // the first pass's last D1 is full before the second pass ends, and the epilogue
@@ -505,6 +497,7 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
           }
           if (CL > 1) {
             const uint32_t rows_bytes = static_cast<uint32_t>(RPC * K * 4);
+            if (r == 0) bulk_wait_read0();  // the previous tile's copies have read sW
             if (!(ok = epi_sync())) break;
 #pragma unroll
             for (int j = 0; j < K; j += 4)
@@ -518,17 +511,38 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
                   bulk_s2s_cluster(mapa(su32(sWrecv + crank * RPC * K), o), su32(sW + o * RPC * K), rows_bytes,
                                    mapa(su32(&bar[S_REDFULL]), o));
               bulk_commit();
-              bulk_wait_read0();
             }
             if (!(ok = wait(S_REDFULL, Tg & 1, true))) break;
-            const int per = RPC * K / kBM;
-            for (int e = 0; e < per; ++e) {
-              const int idx = r * per + e, rl = idx / K, col = idx % K;
-              const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
-              const int rel = own - static_cast<int>(crank) * RPC * K;
-              float sum = 0.f;
-              for (uint32_t src = 0; src < CL; ++src) sum += src == crank ? sW[own] : sWrecv[src * RPC * K + rel];
-              sW[own] = sum;
+            const int per = RPC * K / kBM;  // values per epilogue thread (K / CL), neighbours in a row
+            // partials in source-rank order; four columns at a time where a thread has them
+            if (per % 4 == 0) {
+              for (int e = 0; e < per; e += 4) {
+                const int idx = r * per + e, rl = idx / K, col = idx % K;
+                const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
+                const int rel = own - static_cast<int>(crank) * RPC * K;  // offset inside one owner's row block
+                float4 v[8], sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (uint32_t src = 0; src < 8; ++src)
+                  if (src < CL) v[src] = *reinterpret_cast<const float4*>(src == crank ? sW + own : sWrecv + src * RPC * K + rel);
+#pragma unroll
+                for (uint32_t src = 0; src < 8; ++src)
+                  if (src < CL) {
+                    sum.x += v[src].x;
+                    sum.y += v[src].y;
+                    sum.z += v[src].z;
+                    sum.w += v[src].w;
+                  }
+                *reinterpret_cast<float4*>(sW + own) = sum;
+              }
+            } else {
+              for (int e = 0; e < per; ++e) {
+                const int idx = r * per + e, rl = idx / K, col = idx % K;
+                const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
+                const int rel = own - static_cast<int>(crank) * RPC * K;
+                float sum = 0.f;
+                for (uint32_t src = 0; src < CL; ++src) sum += src == crank ? sW[own] : sWrecv[src * RPC * K + rel];
+                sW[own] = sum;
+              }
             }
             fence_async_smem();
             if (!(ok = epi_sync())) break;
@@ -539,7 +553,6 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
                   bulk_s2s_cluster(mapa(su32(sW + crank * RPC * K), dst), su32(sW + crank * RPC * K), rows_bytes,
                                    mapa(su32(&bar[S_WFULL]), dst));
               bulk_commit();
-              bulk_wait_read0();
             }
             if (!(ok = wait(S_WFULL, Tg & 1, true))) break;
 #pragma unroll
@@ -570,11 +583,13 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
         }
       }
       T += run.ntiles;
-      pieces += Walk8::pieces_of(run.ntiles);
+      pieces += (run.ntiles + TP - 1) / TP;
+      base_g += 2u * static_cast<uint32_t>(run.ntiles) * static_cast<uint32_t>(U);
       si = run.sj;
     }
   }
 
+  if (tid == 4 * 32) bulk_wait_read0();  // the epilogue's last copies have read shared memory
   // ---- teardown: MMAs retired, no remote traffic, then free TMEM
   if (warp >= kIssue1 && lane == 0) mma_commit(&bar[S_DONE]);
   __syncthreads();
@@ -663,7 +678,7 @@ bool tcs8_plan_slice(int d, int k, int sms, const TcsTuning& tune, int ncd_max, 
   const uint32_t B1 = static_cast<uint32_t>(ncd) * N * 128;
   const uint32_t B2 = 2u * (2u * N * 128);
   const uint32_t W = cl > 1 ? 128u * K * 4 : 0u;
-  const uint32_t bars = kNumBars8 * 8 + 16;
+  const uint32_t bars = kNumBars8 * 8 + 16 + kMaxRing * 4;  // barriers, TMEM holder, abort flag, fills
   const int avail = kSmemLimit - 1024 - static_cast<int>(B1 + B2 + 2 * W + bars);
   // operand ring of 32 KB units: three at least (the narrower slices' plans start there), up
   // to four (the converters' registers hold the units in flight, the ring only what
@@ -677,7 +692,9 @@ bool tcs8_plan_slice(int d, int k, int sms, const TcsTuning& tune, int ncd_max, 
   p->ncd = ncd;
   p->cluster = cl;
   p->ring = ring;
-  int lag = tune.lag_units > 0 ? tune.lag_units : (cl > 1 ? 4 : 2);
+  // one block apart, the two converter groups and issuers alternate (lag 4, 2, 1 at d =
+  // 2,048, k = 32: 406, 395, 389 us with n = 262,144)
+  int lag = tune.lag_units > 0 ? tune.lag_units : 1;
   const int U = ncd / 2;
   p->lag = lag < U ? lag : U;
   p->prefetch = 0;
