@@ -363,7 +363,9 @@ const int* slot_begin_of(const lp_ctx* c) {
   return c->path == PATH_TCS ? c->dSlotBeginTcs : c->path == PATH_TC ? c->dSlotBeginTc : c->dSlotBegin;
 }
 
-lp_status launch_step(lp_ctx* c, int K, const float* Z, int64_t z_stride, bool timing) {
+// overlap: the launch may begin while the kernel before it ends (there is one, on this stream).
+lp_status launch_step(lp_ctx* c, int K, const float* Z, int64_t z_stride, bool timing, bool overlap = false) {
+  const lp::Lane at(c->stream, overlap && !timing);
   lp::StepArgs a;
   a.A = c->dA;
   a.ld = c->ld;
@@ -388,18 +390,18 @@ lp_status launch_step(lp_ctx* c, int K, const float* Z, int64_t z_stride, bool t
   cudaError_t e;
   if (c->path == PATH_TCS && c->tcs_cur->pair)
     e = lp::launch_step_pair(*c->tcs_cur, c->dSegsTcs, c->dSegPtrTcs, Z, z_stride, c->dP, static_cast<int>(c->d),
-                             c->dStatus, c->stream);
+                             c->dStatus, at);
   else if (c->path == PATH_TCS && c->tcs_cur->fp8)
     e = lp::launch_step_tcs8(*c->tcs_cur, c->dA, c->n, c->ld, c->dSegsTcs, c->dSegPtrTcs, Z, z_stride, c->dP,
-                             static_cast<int>(c->d), c->dScales, c->smax2, c->dStatus, c->stream);
+                             static_cast<int>(c->d), c->dScales, c->smax2, c->dStatus, at);
   else if (c->path == PATH_TCS)
     e = lp::launch_step_tcs(*c->tcs_cur, c->dSegsTcs, c->dSegPtrTcs, Z, z_stride, c->dP, static_cast<int>(c->d),
-                            c->dStatus, c->stream);
+                            c->dStatus, at);
   else if (c->path == PATH_TC)
     e = lp::launch_step_tc(c->tc, c->dSegsTc, c->dSegPtrTc, Z, z_stride, c->dP, static_cast<int>(c->d), c->dStatus,
-                           c->stream);
+                           at);
   else
-    e = lp::launch_step_simt(a, c->dtype, K, c->stream);
+    e = lp::launch_step_simt(a, c->dtype, K, at);
   if (e != cudaSuccess) return cuda_fail(c, e, "fused power-step launch");
   if (timing) {
     LP_CUDA(record_event(c->step_ev[c->step_ev_used + 1], c->stream));
@@ -960,27 +962,30 @@ static lp_status solve_body(lp_ctx* c, int k, const int* p_schedule, int T, lp_a
   const int NP = c->nprob;
   const bool multi = NP > 1;
   lp_status st;
-  LP_CUDA(cudaMemsetAsync(c->dStatus, 0, 4, c->stream));
-  if ((st = check_launch(c, lp::launch_pack(dy0, c->dY, NP, d, k, K, c->stream), "pack"))) return st;
-  if ((st = check_launch(c, lp::launch_cholqr2(c->dY, c->dZ, NP, d, k, K, c->dStatus, c->stream, kxk64), "orth")))
+  // Every kernel from here on follows a kernel, so its launch may overlap that one's end
+  // (timing events and trace copies between kernels exclude it).
+  const bool overlap = !timing && !trace;
+  const lp::Lane next(c->stream, overlap);
+  if ((st = check_launch(c, lp::launch_pack(dy0, c->dY, NP, d, k, K, c->stream, c->dStatus), "pack"))) return st;
+  if ((st = check_launch(c, lp::launch_cholqr2(c->dY, c->dZ, NP, d, k, K, c->dStatus, next, kxk64), "orth")))
     return st;
 
   const int rounds = T + refine_rounds;
   const int64_t zs = int64_t(d) * K;
   // the first step of a round: the shared basis, or each partition's copy of its problem's
   auto first_step = [&]() -> lp_status {
-    if (!multi) return launch_step(c, K, c->dZ, 0, timing);
-    lp_status s2 = check_launch(c, lp::launch_broadcast(c->dZ, c->dPartProb, m, d, K, c->dZl, c->stream), "broadcast");
-    return s2 ? s2 : launch_step(c, K, c->dZl, zs, timing);
+    if (!multi) return launch_step(c, K, c->dZ, 0, timing, overlap);
+    lp_status s2 = check_launch(c, lp::launch_broadcast(c->dZ, c->dPartProb, m, d, K, c->dZl, next), "broadcast");
+    return s2 ? s2 : launch_step(c, K, c->dZl, zs, timing, overlap);
   };
   for (int t = 0; t < rounds; ++t) {
     const int p = t < T ? p_schedule[t] : 1;
     for (int j = 0; j < p; ++j) {
-      if (j > 0 && (st = check_launch(c, lp::launch_cholqr2(c->dYl, c->dZl, m, d, k, K, c->dStatus, c->stream, kxk64),
+      if (j > 0 && (st = check_launch(c, lp::launch_cholqr2(c->dYl, c->dZl, m, d, k, K, c->dStatus, next, kxk64),
                                       "local orth")))
         return st;
-      if ((st = j == 0 ? first_step() : launch_step(c, K, c->dZl, zs, timing))) return st;
-      if ((st = check_launch(c, lp::launch_reduce(c->dP, slot_begin_of(c), c->dInvS, m, d, K, c->dYl, c->stream,
+      if ((st = j == 0 ? first_step() : launch_step(c, K, c->dZl, zs, timing, overlap))) return st;
+      if ((st = check_launch(c, lp::launch_reduce(c->dP, slot_begin_of(c), c->dInvS, m, d, K, c->dYl, next,
                                                   c->max_slots[c->path]),
                              "reduce")))
         return st;
@@ -990,15 +995,15 @@ static lp_status solve_body(lp_ctx* c, int k, const int* p_schedule, int T, lp_a
     if (align) {
       // The last basis each partition multiplied this round is Z_i (orth of its previous Y_i).
       if ((st = check_launch(c, lp::launch_align(c->dZl, zs, c->dZl + zs * c->base, m, d, k, K, c->base, agg, c->dG,
-                                                 c->dStatus, c->stream, kxk64, multi ? c->dPartBase : nullptr),
+                                                 c->dStatus, next, kxk64, multi ? c->dPartBase : nullptr),
                              "align")))
         return st;
     }
     if ((st = check_launch(c, lp::launch_aggregate(c->dYl, c->dW, align ? c->dG : nullptr, agg == LP_AGG_SIGN ? 1 : 0,
-                                                   m, d, K, c->dY, c->stream, multi ? c->dProbBegin : nullptr, NP),
+                                                   m, d, K, c->dY, next, multi ? c->dProbBegin : nullptr, NP),
                            "aggregate")))
       return st;
-    if ((st = check_launch(c, lp::launch_cholqr2(c->dY, c->dZ, NP, d, k, K, c->dStatus, c->stream, kxk64), "orth")))
+    if ((st = check_launch(c, lp::launch_cholqr2(c->dY, c->dZ, NP, d, k, K, c->dStatus, next, kxk64), "orth")))
       return st;
     if (trace) {
       LP_CUDA(cudaMemcpyAsync(c->dTraceZ + size_t(t) * d * K, c->dZ, size_t(d) * K * 4, cudaMemcpyDeviceToDevice,
@@ -1017,9 +1022,10 @@ static lp_status solve_body(lp_ctx* c, int k, const int* p_schedule, int T, lp_a
   }
   if (c->ritz) {
     if ((st = first_step())) return st;
-    if ((st = check_launch(c, lp::launch_reduce(c->dP, slot_begin_of(c), c->dInvS, m, d, K, c->dYl, c->stream, c->max_slots[c->path]), "reduce")))
+    if ((st = check_launch(c, lp::launch_reduce(c->dP, slot_begin_of(c), c->dInvS, m, d, K, c->dYl, next, c->max_slots[c->path]),
+                           "reduce")))
       return st;
-    if ((st = check_launch(c, lp::launch_aggregate(c->dYl, c->dW, nullptr, 0, m, d, K, c->dMZ, c->stream,
+    if ((st = check_launch(c, lp::launch_aggregate(c->dYl, c->dW, nullptr, 0, m, d, K, c->dMZ, next,
                                                    multi ? c->dProbBegin : nullptr, NP),
                            "aggregate")))
       return st;
@@ -1392,10 +1398,10 @@ lp_status lp_power_step(lp_ctx* c, int k, const double* z, int z_shared, double*
   if ((st = stage_in(c, z, size_t(nb) * d * k, space, &dz))) return st;
   float* Zt = z_shared ? c->dZ : c->dZl;
   if ((st = check_launch(c, lp::launch_pack(dz, Zt, nb, d, k, K, c->stream, c->dStatus), "pack"))) return st;
-  if ((st = launch_step(c, K, Zt, z_shared ? 0 : int64_t(d) * K, false))) return st;
+  if ((st = launch_step(c, K, Zt, z_shared ? 0 : int64_t(d) * K, false, true))) return st;
   double* dst = space == LP_DEVICE ? y_out : c->dStage;
   if ((st = check_launch(c, lp::launch_reduce_f64(c->dP, slot_begin_of(c), c->dInvS, c->m, d, k, K, dst, c->dStatus,
-                                                  c->hStatus, c->stream, c->max_slots[c->path]),
+                                                  c->hStatus, lp::Lane(c->stream, true), c->max_slots[c->path]),
                          "reduce")))
     return st;
   if (space == LP_HOST)

@@ -17,6 +17,51 @@ enum StatusBits : int {
   ST_TIMEOUT = 8,     // a bounded wait gave up
 };
 
+// Where a kernel is launched: the stream, and whether its launch may overlap the end of
+// the kernel before it on that stream (programmatic dependent launch; only where a
+// kernel comes before it).  Kernels launched this way wait for that kernel
+// (after_previous) before they read what a kernel wrote or write what one may read;
+// before that they set up and read only what no kernel writes (the partitions, the
+// segment tables).  Each lets the next one begin (before_next) shortly before it ends,
+// not earlier: a waiting CTA holds its SM against other streams' kernels.
+struct Lane {
+  cudaStream_t s;
+  bool overlap;
+  Lane(cudaStream_t stream, bool may_overlap = false) : s(stream), overlap(may_overlap) {}
+};
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void before_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+cudaError_t launch_on(const Lane& at, void (*kern)(Params...), dim3 grid, unsigned threads, size_t smem, unsigned cluster,
+                      Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = at.s;
+  cudaLaunchAttribute attr[2];
+  unsigned n = 0;
+  if (cluster > 0) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = cluster;
+    attr[n].val.clusterDim.y = 1;
+    attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (at.overlap) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
+#endif
+
 // One contiguous run of rows of one partition processed by one CTA of the
 // fused step kernel.  Global row indices into the packed A buffer.
 struct Segment {
@@ -60,11 +105,11 @@ struct StepArgs {
 };
 
 // Returns cudaErrorInvalidConfiguration when no SIMT instantiation fits.
-cudaError_t launch_step_simt(const StepArgs& a, lp_dtype dtype, int K, cudaStream_t s);
+cudaError_t launch_step_simt(const StepArgs& a, lp_dtype dtype, int K, Lane at);
 // FP32 SIMT step with Z_i resident in tensor memory (K = 16, d <= 1024); the FP32
 // dispatch of launch_step_simt prefers it where it is supported.
 bool step_simt_tmem_supported(int d, int64_t ld, int K);
-cudaError_t launch_step_simt_tmem(const StepArgs& a, cudaStream_t s);
+cudaError_t launch_step_simt_tmem(const StepArgs& a, Lane at);
 // Shared memory the SIMT step needs (0 if unsupported); used to validate up front.
 size_t step_simt_smem(int d, int64_t ld, lp_dtype dtype, int K, int* rows_per_tile);
 
@@ -82,7 +127,7 @@ bool tc_plan(int d, int k, int sms, TcPlan* p);
 // Encodes the 2-D tensor map of A (n rows, d columns, row pitch ld elements).
 cudaError_t tc_encode_map(void* A, int64_t n, int d, int64_t ld, TcPlan* p);
 cudaError_t launch_step_tc(const TcPlan& p, const Segment* segs, const int* seg_ptr, const float* Z, int64_t z_stride,
-                           float* P, int d, int* status, cudaStream_t s);
+                           float* P, int d, int* status, Lane at);
 
 // ---- fused local power step (tcgen05, streaming; BF16 plane or hi/lo planes) --
 struct TcsPlan {
@@ -125,7 +170,7 @@ bool tcs_plan(int d, int k, int planes, int sms, const TcsTuning& tune, TcsPlan*
 cudaError_t tcs_encode_maps(const void* plane0, const void* plane1, int64_t n, int d, int64_t ld, TcsPlan* p,
                             bool unit_boxes = false);
 cudaError_t launch_step_tcs(const TcsPlan& p, const Segment* segs, const int* seg_ptr, const float* Z,
-                            int64_t z_stride, float* P, int d, int* status, cudaStream_t s);
+                            int64_t z_stride, float* P, int d, int* status, Lane at);
 // Pass-split pair kernel: the same product with the HBM pass and the L2 pass on
 // the two CTAs of a cluster.  False when the shape has no plan (d > 1024 at
 // k > 16, d > 2048, or a ring under two units).
@@ -136,9 +181,9 @@ bool tcs8_plan(int d, int k, int sms, const TcsTuning& tune, TcsPlan* p);
 // codes: n rows of pitch ld (a multiple of 16, 16-byte aligned), columns d .. ld - 1 zero.
 cudaError_t launch_step_tcs8(const TcsPlan& p, const void* codes, int64_t n, int64_t ld, const Segment* segs,
                              const int* seg_ptr, const float* Z, int64_t z_stride, float* P, int d, const float* scales,
-                             float smax2, int* status, cudaStream_t s);
+                             float smax2, int* status, Lane at);
 cudaError_t launch_step_pair(const TcsPlan& p, const Segment* segs, const int* seg_ptr, const float* Z,
-                             int64_t z_stride, float* P, int d, int* status, cudaStream_t s);
+                             int64_t z_stride, float* P, int d, int* status, Lane at);
 // FP32 rows (pitch src_ld) -> hi = RNE_bf16(a), lo = RNE_bf16(a - hi) planes (pitch ld, a
 // multiple of 8, 16-byte aligned; columns d..ld-1 zero).  Partition i's rows become rows
 // row0[i] .. row0[i + 1] - 1 of the planes (row0[0] = 0).
@@ -189,29 +234,29 @@ inline void set_no_context_error(const std::string& msg) { set_no_context_error(
 // Y_i = scale_i * sum_{slot in [slot_begin[i], slot_begin[i+1])} P[slot]; max_slots (the most
 // slots any partition has) picks how many threads share one output.
 cudaError_t launch_reduce(const float* P, const int* slot_begin, const float* scale, int m, int d, int K,
-                          float* Y, cudaStream_t s, int max_slots);
+                          float* Y, Lane at, int max_slots);
 // The same sums as m blocks of d rows of k in FP64; *status_host (host memory the device can
 // write, may be nullptr) receives *status.
 cudaError_t launch_reduce_f64(const float* P, const int* slot_begin, const float* scale, int m, int d, int k, int K,
-                              double* Y, const int* status, int* status_host, cudaStream_t s, int max_slots);
+                              double* Y, const int* status, int* status_host, Lane at, int max_slots);
 // Z_b = orth(Y_b) (CholQR2 on FP32 data), batch blocks of d x K.  kxk_fp64: the k x k
 // Gram and Cholesky in FP64; else FP32 with an FP64 Cholesky when a pivot is too small.
-cudaError_t launch_cholqr2(const float* Y, float* Z, int batch, int d, int k, int K, int* status, cudaStream_t s,
+cudaError_t launch_cholqr2(const float* Y, float* Z, int batch, int d, int k, int K, int* status, Lane at,
                            bool kxk_fp64);
 // G_i = aligning matrices (K x K, FP32) for agg in {SIGN, OPT}; base gets I.  kxk_fp64:
 // the k x k Procrustes SVD in FP64, else FP32.
 // part_base (device, may be nullptr): per-partition base partition (several problems in
 // one context); then Zb and base are ignored and Z_b = Zl + z_stride * part_base[i].
 cudaError_t launch_align(const float* Zl, int64_t z_stride, const float* Zb, int m, int d, int k, int K, int base,
-                         lp_aggregator agg, float* G, int* status, cudaStream_t s, bool kxk_fp64,
+                         lp_aggregator agg, float* G, int* status, Lane at, bool kxk_fp64,
                          const int* part_base);
 // Y = sum_i w_i Y_i G_i  (G == nullptr: identity; diag_only: G_i diagonal).  With
 // prob_begin (device, nprob + 1 offsets): Y_q = the sum over problem q's partitions,
 // nprob consecutive d x K blocks.
 cudaError_t launch_aggregate(const float* Yl, const float* w, const float* G, int diag_only, int m, int d, int K,
-                             float* Y, cudaStream_t s, const int* prob_begin, int nprob);
+                             float* Y, Lane at, const int* prob_begin, int nprob);
 // Zl[i] = Z[part_prob[i]] for the m partitions' d x K blocks.
-cudaError_t launch_broadcast(const float* Z, const int* part_prob, int m, int d, int K, float* Zl, cudaStream_t s);
+cudaError_t launch_broadcast(const float* Z, const int* part_prob, int m, int d, int K, float* Zl, Lane at);
 // Ritz: H = Z^T MZ (FP64 sums), eig by Jacobi (FP64 when kxk_fp64, else FP32), Zout = Z W
 // (FP64), sigma = sqrt(n lambda).  Three launches; `scratch` holds ritz_scratch_bytes(d, K,
 // nprob) bytes.  nprob problems at once: Z, MZ consecutive d x K blocks, Zout consecutive

@@ -164,6 +164,8 @@ __global__ void reduce_kernel(const float* __restrict__ P, const int* __restrict
                               const float* __restrict__ scale, int d, int K, float* __restrict__ Y,
                               double* __restrict__ Yd, int k, const int* status, int* status_host) {
   const int i = blockIdx.y;
+  after_previous();
+  before_next();
   if (OUT64 && status_host && blockIdx.x == 0 && i == 0 && threadIdx.x == 0) *status_host = *status;
   const int64_t n4 = int64_t(d) * K / 4;
   const int g = threadIdx.x % G;
@@ -372,6 +374,7 @@ __global__ void __launch_bounds__(kT) align_kernel(const float* __restrict__ Zl,
   double* part = V + K * ks;                    // kT x 16 floats
   const int i = blockIdx.x;
   const int t = threadIdx.x;
+  after_previous();
   // the base of partition i's problem: one for the context, or per partition (batch groups)
   const int base = part_base ? part_base[i] : base_one;
   const float* Zb = part_base ? Zl + z_stride * base : Zb_one;
@@ -425,6 +428,7 @@ __global__ void __launch_bounds__(kT) align_kernel(const float* __restrict__ Zl,
       }
       __syncthreads();
     }
+    before_next();
     for (int e = t; e < K * K; e += kT) {
       const int a = e / K, b = e % K;
       float v = 0.f;
@@ -591,6 +595,8 @@ __global__ void __launch_bounds__(kT) aggregate_kernel(const float* __restrict__
   constexpr int JG = K / 4;
   __shared__ float4 red[kT];
   const int t = threadIdx.x;
+  after_previous();
+  before_next();
   const int RPB = kT / (JG * S);
   const int jg = t % JG, row = (t / JG) % RPB, sl = t / (JG * RPB);
   const int r = blockIdx.x * RPB + row;
@@ -656,6 +662,8 @@ __global__ void __launch_bounds__(kT) aggregate_kernel(const float* __restrict__
 // (batch groups, where the first step of a round multiplies per-problem bases).
 __global__ void broadcast_kernel(const float4* __restrict__ Z, const int* __restrict__ part_prob, int m,
                                  int64_t blk4, float4* __restrict__ Zl) {
+  after_previous();
+  before_next();
   const int64_t total = int64_t(m) * blk4;
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
     const int64_t i = e / blk4, off = e - i * blk4;
@@ -844,72 +852,70 @@ cudaError_t launch_unpack(const float* src, double* dst, int batch, int d, int k
 namespace {
 template <int G>
 cudaError_t launch_reduce_g(const float* P, const int* slot_begin, const float* scale, int m, int d, int K, float* Y,
-                            double* Yd, int k, const int* status, int* status_host, cudaStream_t s) {
+                            double* Yd, int k, const int* status, int* status_host, Lane at) {
   const int64_t n4 = int64_t(d) * K / 4;
   const dim3 grid(static_cast<unsigned>((n4 + kT / G - 1) / (kT / G)), static_cast<unsigned>(m));
-  if (Yd) reduce_kernel<G, true><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y, Yd, k, status, status_host);
-  else reduce_kernel<G, false><<<grid, kT, 0, s>>>(P, slot_begin, scale, d, K, Y, Yd, k, status, status_host);
-  return cudaGetLastError();
+  return launch_on(at, Yd ? reduce_kernel<G, true> : reduce_kernel<G, false>, grid, kT, 0, 0, P, slot_begin, scale, d, K, Y,
+                   Yd, k, status, status_host);
 }
 
 cudaError_t reduce_any(const float* P, const int* slot_begin, const float* scale, int m, int d, int K, float* Y,
-                       double* Yd, int k, const int* status, int* status_host, cudaStream_t s, int max_slots) {
+                       double* Yd, int k, const int* status, int* status_host, Lane at, int max_slots) {
   int G = 1;
   while (G < 32 && max_slots > 4 * G) G <<= 1;
   switch (G) {
-    case 1: return launch_reduce_g<1>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
-    case 2: return launch_reduce_g<2>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
-    case 4: return launch_reduce_g<4>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
-    case 8: return launch_reduce_g<8>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
-    case 16: return launch_reduce_g<16>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
-    default: return launch_reduce_g<32>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, s);
+    case 1: return launch_reduce_g<1>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, at);
+    case 2: return launch_reduce_g<2>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, at);
+    case 4: return launch_reduce_g<4>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, at);
+    case 8: return launch_reduce_g<8>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, at);
+    case 16: return launch_reduce_g<16>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, at);
+    default: return launch_reduce_g<32>(P, slot_begin, scale, m, d, K, Y, Yd, k, status, status_host, at);
   }
 }
 }  // namespace
 
 cudaError_t launch_reduce(const float* P, const int* slot_begin, const float* scale, int m, int d, int K, float* Y,
-                          cudaStream_t s, int max_slots) {
-  return reduce_any(P, slot_begin, scale, m, d, K, Y, nullptr, 0, nullptr, nullptr, s, max_slots);
+                          Lane at, int max_slots) {
+  return reduce_any(P, slot_begin, scale, m, d, K, Y, nullptr, 0, nullptr, nullptr, at, max_slots);
 }
 
 cudaError_t launch_reduce_f64(const float* P, const int* slot_begin, const float* scale, int m, int d, int k, int K,
-                              double* Y, const int* status, int* status_host, cudaStream_t s, int max_slots) {
-  return reduce_any(P, slot_begin, scale, m, d, K, nullptr, Y, k, status, status_host, s, max_slots);
+                              double* Y, const int* status, int* status_host, Lane at, int max_slots) {
+  return reduce_any(P, slot_begin, scale, m, d, K, nullptr, Y, k, status, status_host, at, max_slots);
 }
 
 cudaError_t launch_align(const float* Zl, int64_t z_stride, const float* Zb, int m, int d, int k, int K, int base,
-                         lp_aggregator agg, float* G, int* status, cudaStream_t s, bool kxk_fp64,
+                         lp_aggregator agg, float* G, int* status, Lane at, bool kxk_fp64,
                          const int* part_base) {
-  align_kernel<<<m, kT, align_smem(K), s>>>(Zl, z_stride, Zb, d, k, K, base, part_base, agg == LP_AGG_OPT ? 1 : 0,
-                                            kxk_fp64 ? 1 : 0, G, status);
-  return cudaGetLastError();
+  return launch_on(at, align_kernel, dim3(m), kT, align_smem(K), 0, Zl, z_stride, Zb, d, k, K, base, part_base,
+                   agg == LP_AGG_OPT ? 1 : 0, kxk_fp64 ? 1 : 0, G, status);
 }
 
 cudaError_t launch_aggregate(const float* Yl, const float* w, const float* G, int diag_only, int m, int d, int K,
-                             float* Y, cudaStream_t s, const int* prob_begin, int nprob) {
+                             float* Y, Lane at, const int* prob_begin, int nprob) {
   // slices: a power of two up to the partitions per problem, at most 16
   const int per = nprob > 0 ? m / nprob : m;
   int S = 1;
   while (S * 2 <= per && S * 2 <= 16) S *= 2;
   const int rpb = kT / (K / 4 * S);
   const dim3 grid((d + rpb - 1) / rpb, nprob);
+  auto go = [&](auto kern) {
+    return launch_on(at, kern, grid, kT, 0, 0, Yl, w, G, diag_only, m, d, S, prob_begin, Y);
+  };
   switch (K) {
-    case 4: aggregate_kernel<4><<<grid, kT, 0, s>>>(Yl, w, G, diag_only, m, d, S, prob_begin, Y); break;
-    case 8: aggregate_kernel<8><<<grid, kT, 0, s>>>(Yl, w, G, diag_only, m, d, S, prob_begin, Y); break;
-    case 16: aggregate_kernel<16><<<grid, kT, 0, s>>>(Yl, w, G, diag_only, m, d, S, prob_begin, Y); break;
-    case 32: aggregate_kernel<32><<<grid, kT, 0, s>>>(Yl, w, G, diag_only, m, d, S, prob_begin, Y); break;
+    case 8: return go(aggregate_kernel<8>);
+    case 16: return go(aggregate_kernel<16>);
+    case 32: return go(aggregate_kernel<32>);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
-cudaError_t launch_broadcast(const float* Z, const int* part_prob, int m, int d, int K, float* Zl, cudaStream_t s) {
+cudaError_t launch_broadcast(const float* Z, const int* part_prob, int m, int d, int K, float* Zl, Lane at) {
   const int64_t blk4 = int64_t(d) * K / 4;
   const int64_t total = int64_t(m) * blk4;
   const int blocks = static_cast<int>(std::min<int64_t>((total + kT - 1) / kT, 4096));
-  broadcast_kernel<<<blocks > 0 ? blocks : 1, kT, 0, s>>>(reinterpret_cast<const float4*>(Z), part_prob, m, blk4,
-                                                          reinterpret_cast<float4*>(Zl));
-  return cudaGetLastError();
+  return launch_on(at, broadcast_kernel, dim3(blocks > 0 ? blocks : 1), kT, 0, 0, reinterpret_cast<const float4*>(Z),
+                   part_prob, m, blk4, reinterpret_cast<float4*>(Zl));
 }
 
 cudaError_t launch_ritz(const float* Z, const float* MZ, int d, int k, int K, double n, double* Zout, double* sigma,

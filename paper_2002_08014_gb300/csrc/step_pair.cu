@@ -291,6 +291,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       bounded_drain(B_RING0 + g % R, (g / R) & 1);
   };
 
+  // the producers read only the partitions; every other role waits for the kernel before
+  if (warp != 0) after_previous();
   if (rank == 0) {
     // ===================================================================== rank 0: W = A_t Z
     constexpr uint32_t idesc1 = idesc_bf16(128, N, false, false);
@@ -513,6 +515,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     }
   }
 
+  before_next();
   // ---- teardown: MMAs retired, W copies addressed to rank 1 landed, then free TMEM
   if (issuer) mma_commit(&bar[B_DONE]);  // every issuer's MMAs (none for an idle issuer)
   __syncthreads();
@@ -574,14 +577,13 @@ int pair_active_for(int K, int planes, size_t smem) {
 }
 
 template <int K, int PL>
-cudaError_t launch_pair_t(const TcsPlan& p, const PairArgs& a, cudaStream_t s) {
+cudaError_t launch_pair_t(const TcsPlan& p, const PairArgs& a, Lane at) {
   cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void*>(step_pair_kernel<K, PL>));
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = pair_config<K, PL>(static_cast<unsigned>(2 * p.nclusters), p.smem, s, attr);
   const CUtensorMap* m0 = reinterpret_cast<const CUtensorMap*>(p.tmap[0]);
   const CUtensorMap* m1 = reinterpret_cast<const CUtensorMap*>(p.tmap[PL > 1 ? 1 : 0]);
-  return cudaLaunchKernelEx(&cfg, step_pair_kernel<K, PL>, *m0, *m1, a);
+  return launch_on(at, step_pair_kernel<K, PL>, dim3(static_cast<unsigned>(2 * p.nclusters)), kPairThreads, p.smem, 2, *m0,
+                   *m1, a);
 }
 
 }  // namespace
@@ -641,7 +643,7 @@ bool pair_plan(int d, int k, int planes, int sms, const TcsTuning& tune, TcsPlan
 }
 
 cudaError_t launch_step_pair(const TcsPlan& p, const Segment* segs, const int* seg_ptr, const float* Z,
-                             int64_t z_stride, float* P, int d, int* status, cudaStream_t s) {
+                             int64_t z_stride, float* P, int d, int* status, Lane at) {
   PairArgs a;
   a.segs = segs;
   a.seg_ptr = seg_ptr;
@@ -664,13 +666,13 @@ cudaError_t launch_step_pair(const TcsPlan& p, const Segment* segs, const int* s
   a.tmem0 = p.tmem_cols;
   a.tmem1 = p.tmem_cols1;
   if (p.planes == 1) {
-    if (p.K == 8) return launch_pair_t<8, 1>(p, a, s);
-    if (p.K == 16) return launch_pair_t<16, 1>(p, a, s);
-    return launch_pair_t<32, 1>(p, a, s);
+    if (p.K == 8) return launch_pair_t<8, 1>(p, a, at);
+    if (p.K == 16) return launch_pair_t<16, 1>(p, a, at);
+    return launch_pair_t<32, 1>(p, a, at);
   }
-  if (p.K == 8) return launch_pair_t<8, 2>(p, a, s);
-  if (p.K == 16) return launch_pair_t<16, 2>(p, a, s);
-  return launch_pair_t<32, 2>(p, a, s);
+  if (p.K == 8) return launch_pair_t<8, 2>(p, a, at);
+  if (p.K == 16) return launch_pair_t<16, 2>(p, a, at);
+  return launch_pair_t<32, 2>(p, a, at);
 }
 
 }  // namespace lp

@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(StepArgs a, Geo 
 
   int cur_part = -1;
   const int sb = a.seg_ptr[blockIdx.x], se = a.seg_ptr[blockIdx.x + 1];
+  after_previous();
   for (int si = sb; si < se; ++si) {
     const Segment sg = a.segs[si];
     const int64_t nrows = sg.row1 - sg.row0;
@@ -390,7 +391,8 @@ __global__ void __launch_bounds__(kThreads2, 1) step_simt2_kernel(StepArgs a, Ge
         }
       cp_async_commit();
     };
-    issue(0, buf0);  // the first tile loads while Z_i is staged
+    issue(0, buf0);  // the first tile loads while Z_i is staged (and while the kernel before ends)
+    if (si == sb) after_previous();
     if (sg.part != cur_part) {
       __syncthreads();
       cur_part = sg.part;
@@ -513,12 +515,11 @@ __global__ void __launch_bounds__(kThreads2, 1) step_simt2_kernel(StepArgs a, Ge
 constexpr size_t kSmemLimit2 = 227 * 1024;
 
 template <int K, int CPT, int R>
-cudaError_t launch_two(const StepArgs& a, const Geo2& g, size_t bytes, cudaStream_t s) {
+cudaError_t launch_two(const StepArgs& a, const Geo2& g, size_t bytes, Lane at) {
   auto kern = step_simt2_kernel<K, CPT, R>;
   cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void*>(kern));
   if (e != cudaSuccess) return e;
-  kern<<<a.grid, kThreads2, bytes, s>>>(a, g);
-  return cudaGetLastError();
+  return launch_on(at, kern, dim3(a.grid), kThreads2, bytes, 0, a, g);
 }
 
 // Chooses the row tile (16, else 8) whose shared memory fits; returns false if none.
@@ -539,14 +540,14 @@ bool simt2_pick(int d, int64_t ld, int* R, Geo2* g, size_t* bytes) {
 }
 
 template <int K>
-cudaError_t launch_v2(const StepArgs& a, cudaStream_t s) {
+cudaError_t launch_v2(const StepArgs& a, Lane at) {
   int R;
   Geo2 g;
   size_t bytes;
   if (!simt2_pick<K>(a.d, a.ld, &R, &g, &bytes)) return cudaErrorInvalidConfiguration;
   const bool two = a.d > kThreads2;
-  if (R == 16) return two ? launch_two<K, 2, 16>(a, g, bytes, s) : launch_two<K, 1, 16>(a, g, bytes, s);
-  return two ? launch_two<K, 2, 8>(a, g, bytes, s) : launch_two<K, 1, 8>(a, g, bytes, s);
+  if (R == 16) return two ? launch_two<K, 2, 16>(a, g, bytes, at) : launch_two<K, 1, 16>(a, g, bytes, at);
+  return two ? launch_two<K, 2, 8>(a, g, bytes, at) : launch_two<K, 1, 8>(a, g, bytes, at);
 }
 
 bool v2_supported(int d, int64_t ld, int K) {
@@ -561,54 +562,53 @@ bool v2_supported(int d, int64_t ld, int K) {
   return false;
 }
 
-cudaError_t launch_f32(const StepArgs& a, int K, cudaStream_t s) {
+cudaError_t launch_f32(const StepArgs& a, int K, Lane at) {
   if (v2_supported(a.d, a.ld, K)) {
     switch (K) {
-      case 8: return launch_v2<8>(a, s);
-      case 16: return launch_v2<16>(a, s);
-      case 32: return launch_v2<32>(a, s);
+      case 8: return launch_v2<8>(a, at);
+      case 16: return launch_v2<16>(a, at);
+      case 32: return launch_v2<32>(a, at);
     }
   }
   return cudaErrorInvalidConfiguration;
 }
 
 template <typename Tin, int K, int CPT, int R>
-cudaError_t launch_one(const StepArgs& a, cudaStream_t s) {
+cudaError_t launch_one(const StepArgs& a, Lane at) {
   const Geo g = make_geo(a.d, a.ld, R, K, sizeof(Tin));
   const size_t bytes = Smem<Tin, K, CPT, R>::bytes(g);
   auto kern = step_simt_kernel<Tin, K, CPT, R>;
   cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void*>(kern));
   if (e != cudaSuccess) return e;
-  kern<<<a.grid, kThreads, bytes, s>>>(a, g);
-  return cudaGetLastError();
+  return launch_on(at, kern, dim3(a.grid), kThreads, bytes, 0, a, g);
 }
 
 constexpr size_t kSmemLimit = 227 * 1024;
 
 template <typename Tin, int K, int CPT>
-cudaError_t launch_r(const StepArgs& a, cudaStream_t s) {
+cudaError_t launch_r(const StepArgs& a, Lane at) {
   const Geo g16 = make_geo(a.d, a.ld, 16, K, sizeof(Tin));
-  if (Smem<Tin, K, CPT, 16>::bytes(g16) <= kSmemLimit) return launch_one<Tin, K, CPT, 16>(a, s);
+  if (Smem<Tin, K, CPT, 16>::bytes(g16) <= kSmemLimit) return launch_one<Tin, K, CPT, 16>(a, at);
   const Geo g8 = make_geo(a.d, a.ld, 8, K, sizeof(Tin));
-  if (Smem<Tin, K, CPT, 8>::bytes(g8) <= kSmemLimit) return launch_one<Tin, K, CPT, 8>(a, s);
+  if (Smem<Tin, K, CPT, 8>::bytes(g8) <= kSmemLimit) return launch_one<Tin, K, CPT, 8>(a, at);
   return cudaErrorInvalidConfiguration;
 }
 
 template <typename Tin, int K>
-cudaError_t launch_cpt(const StepArgs& a, cudaStream_t s) {
+cudaError_t launch_cpt(const StepArgs& a, Lane at) {
   const int cpt = (a.d + kThreads - 1) / kThreads;
-  if (cpt <= 1) return launch_r<Tin, K, 1>(a, s);
-  if (cpt <= 2) return launch_r<Tin, K, 2>(a, s);
-  if (cpt <= 4) return launch_r<Tin, K, 4>(a, s);
+  if (cpt <= 1) return launch_r<Tin, K, 1>(a, at);
+  if (cpt <= 2) return launch_r<Tin, K, 2>(a, at);
+  if (cpt <= 4) return launch_r<Tin, K, 4>(a, at);
   return cudaErrorInvalidConfiguration;
 }
 
 template <typename Tin>
-cudaError_t launch_k(const StepArgs& a, int K, cudaStream_t s) {
+cudaError_t launch_k(const StepArgs& a, int K, Lane at) {
   switch (K) {
-    case 8: return launch_cpt<Tin, 8>(a, s);
-    case 16: return launch_cpt<Tin, 16>(a, s);
-    case 32: return launch_cpt<Tin, 32>(a, s);
+    case 8: return launch_cpt<Tin, 8>(a, at);
+    case 16: return launch_cpt<Tin, 16>(a, at);
+    case 32: return launch_cpt<Tin, 32>(a, at);
     default: return cudaErrorInvalidConfiguration;
   }
 }
@@ -634,13 +634,13 @@ size_t smem_for(int d, int64_t ld, int K, int* rows) {
 
 }  // namespace
 
-cudaError_t launch_step_simt(const StepArgs& a, lp_dtype dtype, int K, cudaStream_t s) {
+cudaError_t launch_step_simt(const StepArgs& a, lp_dtype dtype, int K, Lane at) {
   switch (dtype) {
     case LP_F32:
-      if (step_simt_tmem_supported(a.d, a.ld, K)) return launch_step_simt_tmem(a, s);
-      return v2_supported(a.d, a.ld, K) ? launch_f32(a, K, s) : launch_k<float>(a, K, s);
-    case LP_BF16: return launch_k<uint16_t>(a, K, s);
-    case LP_FP8_E4M3: return launch_k<uint8_t>(a, K, s);
+      if (step_simt_tmem_supported(a.d, a.ld, K)) return launch_step_simt_tmem(a, at);
+      return v2_supported(a.d, a.ld, K) ? launch_f32(a, K, at) : launch_k<float>(a, K, at);
+    case LP_BF16: return launch_k<uint16_t>(a, K, at);
+    case LP_FP8_E4M3: return launch_k<uint8_t>(a, K, at);
   }
   return cudaErrorInvalidConfiguration;
 }

@@ -173,7 +173,8 @@ __global__ void __launch_bounds__(kThr, 1) step_simt_tmem_kernel(StepArgs a, Geo
         }
       cp_async_commit();
     };
-    issue(0, buf0);  // the first tile loads while Z_i is staged
+    issue(0, buf0);  // the first tile loads while Z_i is staged (and while the kernel before ends)
+    if (si == sb) after_previous();
     if (sg.part != cur_part) {
       tc_sync();  // every warp's TMEM reads of the previous Z_i have completed
       cur_part = sg.part;
@@ -349,6 +350,7 @@ __global__ void __launch_bounds__(kThr, 1) step_simt_tmem_d1024_kernel(StepArgs 
   const uint32_t tmem = tmem_holder;
   const uint32_t tq = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
 
+  after_previous();
   float2 y[2][kK / 2];
 #pragma unroll
   for (int q = 0; q < 2; ++q)
@@ -512,7 +514,7 @@ bool step_simt_tmem_supported(int d, int64_t ld, int K) {
   return K == kK && geo_tmem(d, ld, &g, &b);
 }
 
-cudaError_t launch_step_simt_tmem(const StepArgs& a, cudaStream_t s) {
+cudaError_t launch_step_simt_tmem(const StepArgs& a, Lane at) {
   GeoT g;
   size_t bytes;
   if (!geo_tmem(a.d, a.ld, &g, &bytes)) return cudaErrorInvalidConfiguration;
@@ -520,14 +522,12 @@ cudaError_t launch_step_simt_tmem(const StepArgs& a, cudaStream_t s) {
     const size_t b3 = size_t(4) * (3 * kTile + 2 * kR * kK);
     cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void*>(step_simt_tmem_d1024_kernel));
     if (e != cudaSuccess) return e;
-    step_simt_tmem_d1024_kernel<<<a.grid, kThr, b3, s>>>(a);
-    return cudaGetLastError();
+    return launch_on(at, step_simt_tmem_d1024_kernel, dim3(a.grid), kThr, b3, 0, a);
   }
   auto kern = a.d > kThr ? step_simt_tmem_kernel<2> : step_simt_tmem_kernel<1>;
   cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void*>(kern));
   if (e != cudaSuccess) return e;
-  kern<<<a.grid, kThr, bytes, s>>>(a, g);
-  return cudaGetLastError();
+  return launch_on(at, kern, dim3(a.grid), kThr, bytes, 0, a, g);
 }
 
 }  // namespace lp

@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_tc_kernel(const __grid_const
   constexpr uint32_t idesc1 = idesc_bf16(128, N, false, false);
   constexpr uint32_t idesc2 = idesc_bf16(128, N, true, false);
 
+  after_previous();
   const int sb = a.seg_ptr[cluster_id], se = a.seg_ptr[cluster_id + 1];
   uint32_t T = 0;  // tiles processed so far (identical in every CTA of the cluster)
   uint32_t epi_phase = 0;  // uses of the epilogue barrier so far (epilogue threads)
@@ -157,15 +158,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_tc_kernel(const __grid_const
     // ---- stage Z slice as [Z_hi | Z_lo]^T (N rows x DC, K-major, SWIZZLE_128B)
     __syncthreads();
     if (si == sb || sg.part != a.segs[si - 1].part) {  // consecutive pieces of a partition share Z_i
-      const float* Zg = a.Z + a.z_stride * sg.part;
-      for (int e = tid; e < DC * K; e += kThreads) {
-        const int c = e / K, j = e % K;
-        const float z = (c0 + c < a.d) ? Zg[static_cast<int64_t>(c0 + c) * K + j] : 0.f;
-        const uint16_t hi = bf16_bits(z);
-        const uint16_t lo = bf16_bits(z - bf16_val(hi));
-        *reinterpret_cast<uint16_t*>(sB1 + sw128_off(j, c, N)) = hi;
-        *reinterpret_cast<uint16_t*>(sB1 + sw128_off(K + j, c, N)) = lo;
-      }
+      stage_z<K, Bf16Op>(sB1, a.Z + a.z_stride * sg.part, c0, DC, a.d, tid, kThreads);
     }
     fence_async_smem();
     __syncthreads();
@@ -422,6 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_tc_kernel(const __grid_const
   }
 
   // ---- teardown: all MMAs retired, no remote traffic in flight, then free TMEM
+  before_next();
   if (warp == 1 && lane == 0) mma_commit(&bar[B_DONE]);
   __syncthreads();
   if (warp == 0) {
@@ -439,25 +433,14 @@ __global__ void __launch_bounds__(kThreads, 1) step_tc_kernel(const __grid_const
 }
 
 template <int K, int NCH>
-cudaError_t launch_tc_t(const TcPlan& p, const TcArgs& a, cudaStream_t s) {
+cudaError_t launch_tc_t(const TcPlan& p, const TcArgs& a, Lane at) {
   using L = TcLayout<K, NCH>;
   auto kern = step_tc_kernel<K, NCH>;
   cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void*>(kern));
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(p.nclusters * p.cluster), 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = L::alloc_bytes;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(p.cluster);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   const CUtensorMap* map = reinterpret_cast<const CUtensorMap*>(p.tmap);
-  return cudaLaunchKernelEx(&cfg, kern, *map, a);
+  return launch_on(at, kern, dim3(static_cast<unsigned>(p.nclusters * p.cluster)), kThreads, L::alloc_bytes,
+                   static_cast<unsigned>(p.cluster), *map, a);
 }
 
 }  // namespace
@@ -540,7 +523,7 @@ cudaError_t tc_encode_map(void* A, int64_t n, int d, int64_t ld, TcPlan* p) {
 }
 
 cudaError_t launch_step_tc(const TcPlan& p, const Segment* segs, const int* seg_ptr, const float* Z, int64_t z_stride,
-                           float* P, int d, int* status, cudaStream_t s) {
+                           float* P, int d, int* status, Lane at) {
   TcArgs a;
   a.segs = segs;
   a.seg_ptr = seg_ptr;
@@ -550,13 +533,13 @@ cudaError_t launch_step_tc(const TcPlan& p, const Segment* segs, const int* seg_
   a.d = d;
   a.status = status;
   if (p.nch == 2) {
-    if (p.K == 8) return launch_tc_t<8, 2>(p, a, s);
-    if (p.K == 16) return launch_tc_t<16, 2>(p, a, s);
-    return launch_tc_t<32, 2>(p, a, s);
+    if (p.K == 8) return launch_tc_t<8, 2>(p, a, at);
+    if (p.K == 16) return launch_tc_t<16, 2>(p, a, at);
+    return launch_tc_t<32, 2>(p, a, at);
   }
-  if (p.K == 8) return launch_tc_t<8, 4>(p, a, s);
-  if (p.K == 16) return launch_tc_t<16, 4>(p, a, s);
-  return launch_tc_t<32, 4>(p, a, s);
+  if (p.K == 8) return launch_tc_t<8, 4>(p, a, at);
+  if (p.K == 16) return launch_tc_t<16, 4>(p, a, at);
+  return launch_tc_t<32, 4>(p, a, at);
 }
 
 }  // namespace lp

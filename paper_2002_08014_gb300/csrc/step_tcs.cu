@@ -179,6 +179,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr uint32_t idesc1 = idesc_bf16(128, N, false, false);
   constexpr uint32_t idesc2 = idesc_bf16(128, N, true, false);
 
+  // the producer reads only the partitions; every other role waits for the kernel before
+  if (warp != 0) after_previous();
   // A run: the consecutive pieces of one partition that this cluster owns.  They share
   // Z_i and their rows follow each other, every piece but the last a whole number of
   // tiles (TP), so a run is one stream of tiles; the accumulation of A^T W starts anew
@@ -481,6 +483,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   }
+  before_next();
   if (tid == 4 * 32) bulk_wait_read0();  // the epilogue's last copies have read shared memory
   // ---- teardown: all MMAs retired, no remote traffic in flight, then free TMEM
   if (issuer) mma_commit(&bar[S_DONE]);
@@ -537,15 +540,13 @@ int tcs_active_clusters(int cl, size_t smem) {
 }
 
 template <int K, int PL>
-cudaError_t launch_tcs_t(const TcsPlan& p, const TcsArgs& a, cudaStream_t s) {
+cudaError_t launch_tcs_t(const TcsPlan& p, const TcsArgs& a, Lane at) {
   cudaError_t e = set_smem_attr<K, PL>(p.smem);
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg =
-      tcs_config<K, PL>(static_cast<unsigned>(p.nclusters * p.cluster), p.cluster, p.smem, s, attr);
   const CUtensorMap* m0 = reinterpret_cast<const CUtensorMap*>(p.tmap[0]);
   const CUtensorMap* m1 = reinterpret_cast<const CUtensorMap*>(p.tmap[PL > 1 ? 1 : 0]);
-  return cudaLaunchKernelEx(&cfg, step_tcs_kernel<K, PL>, *m0, *m1, a);
+  return launch_on(at, step_tcs_kernel<K, PL>, dim3(static_cast<unsigned>(p.nclusters * p.cluster)), kThreads, p.smem,
+                   static_cast<unsigned>(p.cluster), *m0, *m1, a);
 }
 
 int active_for(int K, int planes, int cl, size_t smem) {
@@ -668,7 +669,7 @@ cudaError_t tcs_encode_maps(const void* plane0, const void* plane1, int64_t n, i
 }
 
 cudaError_t launch_step_tcs(const TcsPlan& p, const Segment* segs, const int* seg_ptr, const float* Z,
-                            int64_t z_stride, float* P, int d, int* status, cudaStream_t s) {
+                            int64_t z_stride, float* P, int d, int* status, Lane at) {
   TcsArgs a;
   a.segs = segs;
   a.seg_ptr = seg_ptr;
@@ -690,13 +691,13 @@ cudaError_t launch_step_tcs(const TcsPlan& p, const Segment* segs, const int* se
   a.off_bar = p.off_bar;
   a.tmem_cols = p.tmem_cols;
   if (p.planes == 1) {
-    if (p.K == 8) return launch_tcs_t<8, 1>(p, a, s);
-    if (p.K == 16) return launch_tcs_t<16, 1>(p, a, s);
-    return launch_tcs_t<32, 1>(p, a, s);
+    if (p.K == 8) return launch_tcs_t<8, 1>(p, a, at);
+    if (p.K == 16) return launch_tcs_t<16, 1>(p, a, at);
+    return launch_tcs_t<32, 1>(p, a, at);
   }
-  if (p.K == 8) return launch_tcs_t<8, 2>(p, a, s);
-  if (p.K == 16) return launch_tcs_t<16, 2>(p, a, s);
-  return launch_tcs_t<32, 2>(p, a, s);
+  if (p.K == 8) return launch_tcs_t<8, 2>(p, a, at);
+  if (p.K == 16) return launch_tcs_t<16, 2>(p, a, at);
+  return launch_tcs_t<32, 2>(p, a, at);
 }
 
 }  // namespace lp

@@ -270,6 +270,8 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
 
   const int sb = a.seg_ptr[cluster_id], se = a.seg_ptr[cluster_id + 1];
   const bool converter = warp < 4 || (warp >= 8 && warp < 12);
+  // the converters read only the codes; the other roles wait for the kernel before
+  if (!converter) after_previous();
   if (sb >= se) {
     // no rows: straight to the teardown
   } else if (converter) {
@@ -589,6 +591,7 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
     }
   }
 
+  before_next();
   if (tid == 4 * 32) bulk_wait_read0();  // the epilogue's last copies have read shared memory
   // ---- teardown: MMAs retired, no remote traffic, then free TMEM
   if (warp >= kIssue1 && lane == 0) mma_commit(&bar[S_DONE]);
@@ -640,12 +643,11 @@ int tcs8_active_clusters(int cl, size_t smem) {
 }
 
 template <int K>
-cudaError_t launch_tcs8_t(const TcsPlan& p, const Tcs8Args& a, cudaStream_t s) {
+cudaError_t launch_tcs8_t(const TcsPlan& p, const Tcs8Args& a, Lane at) {
   cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void*>(step_tcs8_kernel<K>));
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = tcs8_config<K>(static_cast<unsigned>(p.nclusters * p.cluster), p.cluster, p.smem, s, attr);
-  return cudaLaunchKernelEx(&cfg, step_tcs8_kernel<K>, a);
+  return launch_on(at, step_tcs8_kernel<K>, dim3(static_cast<unsigned>(p.nclusters * p.cluster)), kThreads8, p.smem,
+                   static_cast<unsigned>(p.cluster), a);
 }
 
 }  // namespace
@@ -725,7 +727,7 @@ bool tcs8_plan_slice(int d, int k, int sms, const TcsTuning& tune, int ncd_max, 
 
 cudaError_t launch_step_tcs8(const TcsPlan& p, const void* codes, int64_t n, int64_t ld, const Segment* segs,
                              const int* seg_ptr, const float* Z, int64_t z_stride, float* P, int d, const float* scales,
-                             float smax2, int* status, cudaStream_t s) {
+                             float smax2, int* status, Lane at) {
   Tcs8Args a;
   a.codes = static_cast<const unsigned char*>(codes);
   a.n = n;
@@ -750,9 +752,9 @@ cudaError_t launch_step_tcs8(const TcsPlan& p, const void* codes, int64_t n, int
   a.off_Wrecv = p.off_Wrecv;
   a.off_bar = p.off_bar;
   a.tmem_cols = p.tmem_cols;
-  if (p.K == 8) return launch_tcs8_t<8>(p, a, s);
-  if (p.K == 16) return launch_tcs8_t<16>(p, a, s);
-  return launch_tcs8_t<32>(p, a, s);
+  if (p.K == 8) return launch_tcs8_t<8>(p, a, at);
+  if (p.K == 16) return launch_tcs8_t<16>(p, a, at);
+  return launch_tcs8_t<32>(p, a, at);
 }
 
 }  // namespace lp
