@@ -146,6 +146,10 @@ struct TcsPlan {
   // off_B1 holds Z, off_B2 the W staging / W buffers
   int pair = 0;        // 1: this plan is for the pair kernel
   int ring1 = 0;       // rank 1 ring units
+  int parts0 = 1;      // rank 0: ring slots a unit fills (2: one for each 64-column chunk)
+  int slots0 = 0;      // rank 0: ring slots
+  int he0 = 1;         // rank 0: MMA issuers
+  int nstg = 2;        // rank 0: staging buffers of W
   int nd2 = 0;         // rank 1 Y-slice buffers in tensor memory
   uint32_t tmem_cols1 = 0;
   long long stall = 0;  // test hook (lp_tuning::test_stall_cycles)
@@ -165,7 +169,7 @@ struct TcsTuning {
 // Fills the geometry for (d, k, planes).  False when the shape has no streaming kernel.
 bool tcs_plan(int d, int k, int planes, int sms, const TcsTuning& tune, TcsPlan* p);
 // Encodes the tensor maps of the planes (plane1 may be NULL for one plane).
-// unit_boxes: where d is a multiple of 64 and rows are unpadded, encode three-dimensional
+// unit_boxes (whole units a slot): where d is a multiple of 64 and rows are unpadded, encode three-dimensional
 // maps whose one box covers a whole 128-column unit (p->map3d = 1; the pair kernel's loads).
 cudaError_t tcs_encode_maps(const void* plane0, const void* plane1, int64_t n, int d, int64_t ld, TcsPlan* p,
                             bool unit_boxes = false);

@@ -157,17 +157,34 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 // 32 lanes x 16 consecutive 32-bit TMEM columns; lane i of the warp gets lane (base + i).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
+// The registers may be read after tmem_wait and the tmem_value of each group of 16.
+__device__ __forceinline__ void tmem_ld16_begin(uint32_t taddr, uint32_t* r) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_value(uint32_t* r, float* v) {
+  // (nothing that reads the registers moves above this, nor it above the wait)
+  asm volatile(""
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                 "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+// 16 Q consecutive columns with one wait.
+template <int Q>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float* v) {
+  uint32_t r[16 * Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) tmem_ld16_begin(taddr + 16 * q, r + 16 * q);
+  tmem_wait();
+#pragma unroll
+  for (int q = 0; q < Q; ++q) tmem_value(r + 16 * q, v + 16 * q);
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) { tmem_ld<1>(taddr, v); }
 
 // Position (in floats) of the 4-float group holding column j of row r in a
 // row-major 128 x K FP32 buffer; groups are XOR-permuted so that a warp's
