@@ -157,7 +157,7 @@ struct TcsPlan {
   int fp8 = 0;         // 1: this plan is for step_tcs8_kernel
   int behind = 1;      // its second pass runs this many tiles behind the first
   int issuers = 1;     // streaming kernels: MMA-issuing threads (own partial D1 and ring slots each)
-  int map3d = 0;       // pair kernel: the maps are (64 columns, row, chunk), one box per unit
+  int map3d = 0;       // the maps are (64 columns, row, chunk), one box per unit
   alignas(64) unsigned char tmap[2][128];  // CUtensorMaps of the planes
 };
 // Tuning of the streaming kernel (lp_tuning without the C names); zeros are defaults.
@@ -169,8 +169,8 @@ struct TcsTuning {
 // Fills the geometry for (d, k, planes).  False when the shape has no streaming kernel.
 bool tcs_plan(int d, int k, int planes, int sms, const TcsTuning& tune, TcsPlan* p);
 // Encodes the tensor maps of the planes (plane1 may be NULL for one plane).
-// unit_boxes (whole units a slot): where d is a multiple of 64 and rows are unpadded, encode three-dimensional
-// maps whose one box covers a whole 128-column unit (p->map3d = 1; the pair kernel's loads).
+// unit_boxes (a ring slot holds a whole unit): where d is a multiple of 64 and rows are
+// unpadded, encode three-dimensional maps whose one box covers a 128-column unit (p->map3d = 1).
 cudaError_t tcs_encode_maps(const void* plane0, const void* plane1, int64_t n, int d, int64_t ld, TcsPlan* p,
                             bool unit_boxes = false);
 cudaError_t launch_step_tcs(const TcsPlan& p, const Segment* segs, const int* seg_ptr, const float* Z,

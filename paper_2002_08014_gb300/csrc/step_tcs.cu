@@ -59,6 +59,7 @@ struct TcsArgs {
   int lag;   // first-pass units of tile t+1 issued before the second pass of tile t starts
   int issuers;  // MMA-issuing threads (1 or 2), each with its own partial D1
   int prefetch;  // first-pass units brought into L2 ahead of their load (0: none)
+  int map3d;     // 1: the maps are (64 columns, row, chunk) and one box brings a whole unit
   int hints;     // 1: first-pass loads evict_last, second-pass loads evict_first
   uint32_t off_B1, off_B2, off_W, off_Wrecv, off_bar, tmem_cols;
 };
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   };
   auto wait = [&](int id, uint32_t parity, bool cluster_scope) -> bool {
     const uint32_t addr = su32(&bar[id]);
+    if (cluster_scope ? mbar_try_cluster(addr, parity) : mbar_try(addr, parity)) return true;
     const long long t0 = clock64();
     while (true) {
       if (cluster_scope ? mbar_try_cluster(addr, parity) : mbar_try(addr, parity)) return true;
@@ -165,6 +167,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   };
 
   auto wait_issued = [&](uint32_t g) -> bool {
+    if (*issued > g) return true;
     const long long t0 = clock64();
     while (*issued <= g) {
       if (*abort_flag) return false;
@@ -231,11 +234,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       const int PF = a.prefetch;
       // first-pass units [0, PF) of the segment go to L2 up front; later ones PF units ahead of their load
-      for (int q = 0; q < PF && q < ntiles * U; ++q) {
+      auto prefetch_unit = [&](int q) {
         const int t2 = q / U, u2 = q % U, b2 = u2 / PL, pl2 = u2 % PL;
-        for (int j = 0; j < 2; ++j)
-          tma_prefetch_2d(pl2 ? &map1 : &map0, c0 + 64 * (2 * b2 + j), static_cast<int>(sg.row0) + t2 * kBM);
-      }
+        const int row = static_cast<int>(sg.row0) + t2 * kBM;
+        if (a.map3d) {
+          tma_prefetch_3d(pl2 ? &map1 : &map0, 0, row, c0 / 64 + 2 * b2);
+          return;
+        }
+        for (int j = 0; j < 2; ++j) tma_prefetch_2d(pl2 ? &map1 : &map0, c0 + 64 * (2 * b2 + j), row);
+      };
+      for (int q = 0; q < PF && q < ntiles * U; ++q) prefetch_unit(q);
       prod_ok = for_each_unit(ntiles, U, LAG, [&](bool second, int t, int u) -> bool {
         const uint32_t s = slot;
         if (!wait(S_RING0 + R + s, phase ^ 1, false)) return false;
@@ -243,8 +251,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int b = u / PL, pl = u % PL;
         const int row = static_cast<int>(sg.row0) + t * kBM;
         const CUtensorMap* map = pl ? &map1 : &map0;
-        for (int j = 0; j < 2; ++j) {
-          const uint32_t dst = su32(sRing + s * kUnitBytes + j * kChunkBytes);
+        const uint32_t dst0 = su32(sRing + s * kUnitBytes);
+        if (a.map3d) {
+          // both 64-column chunks as one box (a chunk past d is out of range: zeros)
+          const int chunk = c0 / 64 + 2 * b;
+          if (a.hints) tma_load_3d_hint(dst0, map, 0, row, chunk, &bar[S_RING0 + s], second ? pol_drop : pol_keep);
+          else tma_load_3d(dst0, map, 0, row, chunk, &bar[S_RING0 + s]);
+        }
+        for (int j = a.map3d ? 2 : 0; j < 2; ++j) {
+          const uint32_t dst = dst0 + j * kChunkBytes;
           if (a.hints)
             tma_load_2d_hint(dst, map, c0 + 64 * (2 * b + j), row, &bar[S_RING0 + s], second ? pol_drop : pol_keep);
           else
@@ -254,11 +269,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         *issued = unit;
         if (!second && PF > 0) {
           const int q = t * U + u + PF;
-          if (q < ntiles * U) {
-            const int t2 = q / U, u2 = q % U, b2 = u2 / PL, pl2 = u2 % PL;
-            for (int j = 0; j < 2; ++j)
-              tma_prefetch_2d(pl2 ? &map1 : &map0, c0 + 64 * (2 * b2 + j), static_cast<int>(sg.row0) + t2 * kBM);
-          }
+          if (q < ntiles * U) prefetch_unit(q);
         }
         return true;
       });
@@ -332,15 +343,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int j = 0; j < K; ++j) w[j] = 0.f;
         for (int hh = 0; hh < HE; ++hh) {
+          float v[N];
+          tmem_ld<N / 16>(tmem + lane_base + (buf * HE + hh) * N, v);
 #pragma unroll
-          for (int q = 0; q < N / 16; ++q) {
-            float v[16];
-            tmem_ld16(tmem + lane_base + (buf * HE + hh) * N + q * 16, v);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const int col = q * 16 + i;
-              w[col < K ? col : col - K] += v[i];
-            }
+          for (int j = 0; j < K; ++j) {
+            w[j] += v[j];
+            w[j] += v[K + j];
           }
         }
         tc_fence_before();
@@ -445,18 +453,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_after();
         float* Pd = a.P + static_cast<int64_t>(a.segs[si + piece].slot) * a.d * K;
         for (int b = 0; b < NB; ++b) {
-          float y[K];
+          float y[K], v[N];
+          tmem_ld<N / 16>(tmem + lane_base + 2 * HE * N + b * N, v);
 #pragma unroll
-          for (int q = 0; q < N / 16; ++q) {
-            float v[16];
-            tmem_ld16(tmem + lane_base + 2 * HE * N + b * N + q * 16, v);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const int col = q * 16 + i;
-              if (col < K) y[col] = v[i];
-              else y[col - K] += v[i];
-            }
-          }
+          for (int j = 0; j < K; ++j) y[j] = v[j] + v[K + j];
           const int dcol = c0 + b * 128 + (warp & 3) * 32 + lane;
           if (dcol < a.d) {
             float4* dst = reinterpret_cast<float4*>(Pd + static_cast<int64_t>(dcol) * K);
@@ -592,7 +592,9 @@ bool tcs_plan(int d, int k, int planes, int sms, const TcsTuning& tune, TcsPlan*
   p->cluster = cl;
   p->ring = ring;
   const int U = (ncd / 2) * planes;
-  if (lag <= 0) lag = cl > 1 ? 4 : 2;
+  // (over a cluster W takes the exchange between CTAs: 1,000,000 x 2,048, k = 32, four units a
+  // tile: lag 2, 3, 4: 1,011, 993, 1,013 us)
+  if (lag <= 0) lag = cl > 1 ? 3 : 2;
   p->lag = lag < U ? lag : U;
   p->prefetch = tune.prefetch_units > 0 ? tune.prefetch_units : 0;
   p->hints = tune.cache_hints ? 1 : 0;
@@ -683,6 +685,7 @@ cudaError_t launch_step_tcs(const TcsPlan& p, const Segment* segs, const int* se
   a.lag = p.lag;
   a.issuers = p.issuers;
   a.prefetch = p.prefetch;
+  a.map3d = p.map3d;
   a.hints = p.hints;
   a.off_B1 = p.off_B1;
   a.off_B2 = p.off_B2;
