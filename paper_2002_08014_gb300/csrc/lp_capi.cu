@@ -71,6 +71,7 @@ struct lp_ctx {
   int* dSegPtrTcs = nullptr;
   int* dSlotBeginTcs = nullptr;
   const lp::TcsPlan* tcs_cur = nullptr;
+  int peers = 1;  // launch sequences that a batch's graph runs side by side with this one
 
   int path = 0;  // step kernel of the current solve / step (lp_stats::path)
   lp::TcsTuning tuning;
@@ -363,6 +364,19 @@ const int* slot_begin_of(const lp_ctx* c) {
   return c->path == PATH_TCS ? c->dSlotBeginTcs : c->path == PATH_TC ? c->dSlotBeginTc : c->dSlotBegin;
 }
 
+// Row ranges a cluster of the pass-split step takes.  A launch of few units a cluster spends
+// most of its time in its fixed parts (setup, Z, the first loads, the flush: 6-8 us, some 16
+// units' worth), on all SMs.  Where other sequences run beside it, it takes a quarter of the
+// SMs for kSpanUnits units instead, and up to four such launches share the chip.  24 instances
+// of mixed shapes in 16 groups: limit 8, 16, 32, 64 units: 10.93, 10.48, 9.91, 9.97 ms
+// against 11.24; a span of two or four for all: 10.29, 12.35; of up to eight: 9.98.
+int step_span(const lp_ctx* c) {
+  constexpr int kSpanUnits = 32, kMaxSpan = 4;
+  const int G = c->tcs_cur->nclusters;
+  const int64_t units = ((c->n + G - 1) / G + 127) / 128 * ((c->d + 127) / 128) * c->planes;
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({kMaxSpan, c->peers, kSpanUnits / units})));
+}
+
 // overlap: the launch may begin while the kernel before it ends (there is one, on this stream).
 lp_status launch_step(lp_ctx* c, int K, const float* Z, int64_t z_stride, bool timing, bool overlap = false) {
   const lp::Lane at(c->stream, overlap && !timing);
@@ -390,7 +404,7 @@ lp_status launch_step(lp_ctx* c, int K, const float* Z, int64_t z_stride, bool t
   cudaError_t e;
   if (c->path == PATH_TCS && c->tcs_cur->pair)
     e = lp::launch_step_pair(*c->tcs_cur, c->dSegsTcs, c->dSegPtrTcs, Z, z_stride, c->dP, static_cast<int>(c->d),
-                             c->dStatus, at);
+                             c->dStatus, at, step_span(c));
   else if (c->path == PATH_TCS && c->tcs_cur->fp8)
     e = lp::launch_step_tcs8(*c->tcs_cur, c->dA, c->n, c->ld, c->dSegsTcs, c->dSegPtrTcs, Z, z_stride, c->dP,
                              static_cast<int>(c->d), c->dScales, c->smax2, c->dStatus, at);
@@ -1637,12 +1651,14 @@ lp_status lp::batch_prepare(lp_ctx* c, int k, const int* p_schedule, int T, lp_a
 }
 
 lp_status lp::batch_enqueue(lp_ctx* c, int k, const int* p_schedule, int T, lp_aggregator agg, int refine_rounds,
-                            unsigned flags, lp_stats* captured) {
+                            unsigned flags, int peers, lp_stats* captured) {
   std::memset(&c->stats, 0, sizeof(c->stats));
   c->step_ev_used = 0;
   LP_CUDA(record_event(c->ev0, c->stream));
+  c->peers = peers;
   const lp_status st = solve_body(c, k, p_schedule, T, agg, refine_rounds, (flags & LP_FLAG_TIMING) != 0, c->dStage,
                                   (flags & LP_FLAG_TRACE) != 0, (flags & LP_FLAG_KXK_FP64) != 0);
+  c->peers = 1;
   if (st) return st;
   LP_CUDA(record_event(c->ev1, c->stream));
   *captured = c->stats;

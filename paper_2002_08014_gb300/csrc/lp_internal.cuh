@@ -186,8 +186,9 @@ bool tcs8_plan(int d, int k, int sms, const TcsTuning& tune, TcsPlan* p);
 cudaError_t launch_step_tcs8(const TcsPlan& p, const void* codes, int64_t n, int64_t ld, const Segment* segs,
                              const int* seg_ptr, const float* Z, int64_t z_stride, float* P, int d, const float* scales,
                              float smax2, int* status, Lane at);
+// span: row ranges a cluster takes (the grid is that many times smaller; same sums).
 cudaError_t launch_step_pair(const TcsPlan& p, const Segment* segs, const int* seg_ptr, const float* Z,
-                             int64_t z_stride, float* P, int d, int* status, Lane at);
+                             int64_t z_stride, float* P, int d, int* status, Lane at, int span = 1);
 // FP32 rows (pitch src_ld) -> hi = RNE_bf16(a), lo = RNE_bf16(a - hi) planes (pitch ld, a
 // multiple of 8, 16-byte aligned; columns d..ld-1 zero).  Partition i's rows become rows
 // row0[i] .. row0[i + 1] - 1 of the planes (row0[0] = 0).
@@ -216,7 +217,7 @@ int solve_state(lp_ctx* c);
 lp_status batch_prepare(lp_ctx* c, int k, const int* p_schedule, int T, lp_aggregator agg, const double* y0,
                         int refine_rounds, unsigned flags);
 lp_status batch_enqueue(lp_ctx* c, int k, const int* p_schedule, int T, lp_aggregator agg, int refine_rounds,
-                        unsigned flags, lp_stats* captured);
+                        unsigned flags, int peers, lp_stats* captured);
 void batch_mark(lp_ctx* c, int k, const lp_stats& captured, int rounds, unsigned flags);
 cudaStream_t ctx_stream(lp_ctx* c);
 // Several independent problems in one context (the batch runner's groups): load the

@@ -531,7 +531,7 @@ lp_status lp_batch_solve(lp_batch* b) {
       e = cudaStreamWaitEvent(s, b->fork, 0);
       if (e != cudaSuccess) break;
       st = lp::batch_enqueue(g.ctx, r.k, r.sched.empty() ? nullptr : r.sched.data(), r.T, r.agg, r.refine, r.flags,
-                             &g.captured);
+                             static_cast<int>(b->groups.size()), &g.captured);
       if (st) {
         b->err = lp_last_error(g.ctx);
         break;

@@ -86,7 +86,8 @@ constexpr int kNumBars = B_RING0 + 2 * kMaxRing;
 
 struct PairArgs {
   const Segment* segs;
-  const int* seg_ptr;  // per cluster
+  const int* seg_ptr;  // per row range
+  int ranges, span;    // a cluster takes `span` consecutive ones of the `ranges` row ranges
   const float* Z;
   int64_t z_stride;
   float* P;
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   const int cluster_id = blockIdx.x >> 1;
   unsigned char* sStage = base + (rank == 0 ? a.off_stage0 : a.off_stage1);  // rank 0: staging of W; rank 1: the W buffers
   // the segment range, loaded while the barriers and tensor memory are set up
-  const int sb = a.seg_ptr[cluster_id], se = a.seg_ptr[cluster_id + 1];
+  const int sb = a.seg_ptr[cluster_id * a.span], se = a.seg_ptr[min((cluster_id + 1) * a.span, a.ranges)];
   const int NB = a.ncd / 2;
   const int U = NB * PL;
   const int R = rank == 0 ? a.ring0 : a.ring1;
@@ -610,8 +611,8 @@ cudaError_t launch_pair_p(const TcsPlan& p, const PairArgs& a, Lane at) {
   if (e != cudaSuccess) return e;
   const CUtensorMap* m0 = reinterpret_cast<const CUtensorMap*>(p.tmap[0]);
   const CUtensorMap* m1 = reinterpret_cast<const CUtensorMap*>(p.tmap[PL > 1 ? 1 : 0]);
-  return launch_on(at, step_pair_kernel<K, PL, PARTS>, dim3(static_cast<unsigned>(2 * p.nclusters)), kPairThreads,
-                   p.smem, 2, *m0, *m1, a);
+  return launch_on(at, step_pair_kernel<K, PL, PARTS>, dim3(static_cast<unsigned>(2 * ((a.ranges + a.span - 1) / a.span))),
+                   kPairThreads, p.smem, 2, *m0, *m1, a);
 }
 
 template <int K, int PL>
@@ -693,8 +694,10 @@ bool pair_plan(int d, int k, int planes, int sms, const TcsTuning& tune, TcsPlan
 }
 
 cudaError_t launch_step_pair(const TcsPlan& p, const Segment* segs, const int* seg_ptr, const float* Z,
-                             int64_t z_stride, float* P, int d, int* status, Lane at) {
+                             int64_t z_stride, float* P, int d, int* status, Lane at, int span) {
   PairArgs a;
+  a.ranges = p.nclusters;
+  a.span = span;
   a.segs = segs;
   a.seg_ptr = seg_ptr;
   a.Z = Z;
