@@ -1670,6 +1670,8 @@ void lp::batch_mark(lp_ctx* c, int k, const lp_stats& captured, int rounds, unsi
   solve_mark(c, k, rounds, flags);
 }
 
+void lp::set_peers(lp_ctx* c, int peers) { c->peers = peers; }
+
 cudaStream_t lp::ctx_stream(lp_ctx* c) { return c->stream; }
 
 lp_status lp::problem_result(lp_ctx* c, int q, double* z_out, double* sigma_out, lp_stats* stats) {

@@ -214,6 +214,7 @@ int solve_state(lp_ctx* c);
 // choice and y0 upload (outside the capture); the launch sequence on the
 // context's stream (inside it; *captured receives its counters); and marking
 // the context solved after the graph ran.
+void set_peers(lp_ctx* c, int peers);
 lp_status batch_prepare(lp_ctx* c, int k, const int* p_schedule, int T, lp_aggregator agg, const double* y0,
                         int refine_rounds, unsigned flags);
 lp_status batch_enqueue(lp_ctx* c, int k, const int* p_schedule, int T, lp_aggregator agg, int refine_rounds,

@@ -112,6 +112,7 @@ void admit(lp_server* s, Request* r) {
   s->peak = std::max(s->peak, s->in_use);
   st = lp::load_pitched(c, r->m, r->rows.data(), r->d, r->pitch, r->dtype, r->parts.data(),
                         r->dtype == LP_FP8_E4M3 ? r->scales.data() : nullptr, r->space);
+  if (!st) lp::set_peers(c, static_cast<int>(s->active.size() + s->queue.size()) + 1);
   if (!st)
     st = lp_solve(c, r->k, r->sched.empty() ? nullptr : r->sched.data(), r->T, r->agg, r->y0.data(), r->refine,
                   r->flags | (enqueue_directly(r) ? LP_FLAG_NO_GRAPH : 0u));
