@@ -310,7 +310,13 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(StepArgs a, Geo 
 // warp are combined with shuffles, the warps through shared memory.  A's
 // shared row stride is 8 floats past a multiple of 32 and Z's 4-row blocks
 // swap row pairs on odd quads, which keeps both read patterns conflict free.
-// Phase 2 is the design above with two columns per thread.
+// Phase 2: four threads share four columns of A, each a quarter of the columns of Y.
+// Shared memory returns 128 bytes a clock, one FP32 for each FMA lane, and a thread that
+// holds whole columns of Y reads all of a row of W for one element of A (k = 32: 9 loads
+// for 32 FMAs against 3 now).  Tiles of 32 rows (8 x 4 micro-tiles) were no better and
+// lost where d is small, 8 x 8 micro-tiles with half the threads were slower throughout.
+// us, whole columns a thread -> now: 20,000 x 400, k = 17: 49.8 -> 42.4; 10,003 x 300,
+// k = 20: 26.8 -> 23.0; 60,000 x 724, k = 8: 75.2 -> 66.4; 4,000 x 100, k = 32: 10.9 -> 9.9.
 constexpr int kThreads2 = 512;
 
 struct Geo2 {
@@ -338,10 +344,11 @@ struct Simt2 {
   }
 };
 
-template <int K, int CPT, int R>
+template <int K, int CQ, int R>
 __global__ void __launch_bounds__(kThreads2, 1) step_simt2_kernel(StepArgs a, Geo2 g) {
   using G2 = Simt2<K, R>;
   constexpr int MT = G2::MT, SPW = G2::SPW, RG = R / 4;
+  constexpr int JJ = K / 4;  // columns of Y a thread of phase 2 holds, for each of 4 CQ columns of A
   extern __shared__ __align__(16) float sm2[];
   float* buf0 = sm2;
   float* buf1 = buf0 + R * g.lds;
@@ -360,6 +367,7 @@ __global__ void __launch_bounds__(kThreads2, 1) step_simt2_kernel(StepArgs a, Ge
   const int rg = mt / (K / 4), jg = mt % (K / 4);
   const int s_id = warp * SPW + sp;
   const int nq = g.Qp / g.S;
+  const int cq = tid >> 2, j2 = (tid & 3) * JJ;  // phase 2
 
   for (int r = 0; r < R; ++r)
     for (int c = static_cast<int>(a.ld) + tid; c < g.lds; c += kThreads2) {
@@ -367,11 +375,13 @@ __global__ void __launch_bounds__(kThreads2, 1) step_simt2_kernel(StepArgs a, Ge
       buf1[r * g.lds + c] = 0.f;
     }
 
-  float2 y[CPT][K / 2];
+  float2 y[CQ][4][JJ / 2];
 #pragma unroll
-  for (int q = 0; q < CPT; ++q)
+  for (int q = 0; q < CQ; ++q)
 #pragma unroll
-    for (int j = 0; j < K / 2; ++j) y[q][j] = make_float2(0.f, 0.f);
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < JJ / 2; ++j) y[q][i][j] = make_float2(0.f, 0.f);
 
   int cur_part = -1;
   const int sb = a.seg_ptr[blockIdx.x], se = a.seg_ptr[blockIdx.x + 1];
@@ -391,10 +401,10 @@ __global__ void __launch_bounds__(kThreads2, 1) step_simt2_kernel(StepArgs a, Ge
         }
       cp_async_commit();
     };
-    issue(0, buf0);  // the first tile loads while Z_i is staged (and while the kernel before ends)
+    __syncthreads();  // phase 2 of the segment before has read its tile and Z_i
+    issue(0, buf0);   // the first tile loads while Z_i is staged (and while the kernel before ends)
     if (si == sb) after_previous();
     if (sg.part != cur_part) {
-      __syncthreads();
       cur_part = sg.part;
       const float* Zg = a.Z + a.z_stride * sg.part;
       for (int e = tid; e < g.Qp * 4 * (K / 4); e += kThreads2) {
@@ -407,13 +417,9 @@ __global__ void __launch_bounds__(kThreads2, 1) step_simt2_kernel(StepArgs a, Ge
     }
     for (int t = 0; t < ntiles; ++t) {
       const float* T = (t & 1) ? buf1 : buf0;
-      if (t + 1 < ntiles) {
-        issue(t + 1, (t & 1) ? buf0 : buf1);
-        cp_async_wait<1>();
-      } else {
-        cp_async_wait<0>();
-      }
-      __syncthreads();
+      cp_async_wait<0>();
+      __syncthreads();  // the tile is here; phase 2 of the tile before is done with the other buffer
+      if (t + 1 < ntiles) issue(t + 1, (t & 1) ? buf0 : buf1);
 
       // ---- phase 1: rows {rg + RG*aa}, columns {4jg .. 4jg+3}, quads q = s_id + S*u
       // (packed FP32 FMAs: two output columns per instruction)
@@ -466,57 +472,72 @@ __global__ void __launch_bounds__(kThreads2, 1) step_simt2_kernel(StepArgs a, Ge
       }
       __syncthreads();
       for (int e = tid; e < R * K; e += kThreads2) {
-        float sum = 0.f;
-#pragma unroll 4
-        for (int w = 0; w < 16; ++w) sum += red[size_t(w) * R * K + e];
+        float v[16], sum = 0.f;
+#pragma unroll
+        for (int w = 0; w < 16; ++w) v[w] = red[size_t(w) * R * K + e];
+#pragma unroll
+        for (int w = 0; w < 16; ++w) sum += v[w];
         Ws[e] = sum;
       }
       __syncthreads();
 
-      // ---- phase 2: Y += T^T W (packed FP32 FMAs)
+      // ---- phase 2: Y += T^T W (packed FP32 FMAs): four threads share four columns of A
 #pragma unroll 2
       for (int r = 0; r < R; ++r) {
-        float2 w[K / 2];
+        float2 w[JJ / 2];
+        if constexpr (JJ == 2) {
+          w[0] = *reinterpret_cast<const float2*>(Ws + r * K + j2);
+        } else {
 #pragma unroll
-        for (int j = 0; j < K; j += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(Ws + r * K + j);
-          w[j / 2] = make_float2(v.x, v.y);
-          w[j / 2 + 1] = make_float2(v.z, v.w);
+          for (int j = 0; j < JJ; j += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(Ws + r * K + j2 + j);
+            w[j / 2] = make_float2(v.x, v.y);
+            w[j / 2 + 1] = make_float2(v.z, v.w);
+          }
         }
 #pragma unroll
-        for (int q = 0; q < CPT; ++q) {
-          const int c = tid + kThreads2 * q;
+        for (int q = 0; q < CQ; ++q) {
+          const int c = 4 * (cq + kThreads2 / 4 * q);
           if (c < d) {
-            const float av = T[size_t(r) * g.lds + c];
-            const float2 a2 = make_float2(av, av);
+            const float4 v = *reinterpret_cast<const float4*>(T + size_t(r) * g.lds + c);
 #pragma unroll
-            for (int j = 0; j < K / 2; ++j) y[q][j] = __ffma2_rn(a2, w[j], y[q][j]);
+            for (int i = 0; i < 4; ++i) {
+              const float ai = i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
+              const float2 a2 = make_float2(ai, ai);
+#pragma unroll
+              for (int j = 0; j < JJ / 2; ++j) y[q][i][j] = __ffma2_rn(a2, w[j], y[q][i][j]);
+            }
           }
         }
       }
-      __syncthreads();
     }
-    float* Pd = a.P + size_t(sg.slot) * d * pld;
+    float* Pd = a.P + size_t(sg.slot) * d * pld + j2;
 #pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-      const int c = tid + kThreads2 * q;
-      if (c < d) {
+    for (int q = 0; q < CQ; ++q)
 #pragma unroll
-        for (int j = 0; j < K / 2; j += 2)
-          *reinterpret_cast<float4*>(Pd + size_t(c) * pld + 2 * j) = make_float4(y[q][j].x, y[q][j].y, y[q][j + 1].x,
-                                                                              y[q][j + 1].y);
+      for (int i = 0; i < 4; ++i) {
+        const int c = 4 * (cq + kThreads2 / 4 * q) + i;
+        if (c < d) {
+          if constexpr (JJ == 2) {
+            *reinterpret_cast<float2*>(Pd + size_t(c) * pld) = y[q][i][0];
+          } else {
+#pragma unroll
+            for (int j = 0; j < JJ / 2; j += 2)
+              *reinterpret_cast<float4*>(Pd + size_t(c) * pld + 2 * j) =
+                  make_float4(y[q][i][j].x, y[q][i][j].y, y[q][i][j + 1].x, y[q][i][j + 1].y);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < JJ / 2; ++j) y[q][i][j] = make_float2(0.f, 0.f);
       }
-#pragma unroll
-      for (int j = 0; j < K / 2; ++j) y[q][j] = make_float2(0.f, 0.f);
-    }
   }
 }
 
 constexpr size_t kSmemLimit2 = 227 * 1024;
 
-template <int K, int CPT, int R>
+template <int K, int CQ, int R>
 cudaError_t launch_two(const StepArgs& a, const Geo2& g, size_t bytes, Lane at) {
-  auto kern = step_simt2_kernel<K, CPT, R>;
+  auto kern = step_simt2_kernel<K, CQ, R>;
   cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void*>(kern));
   if (e != cudaSuccess) return e;
   return launch_on(at, kern, dim3(a.grid), kThreads2, bytes, 0, a, g);
@@ -539,15 +560,13 @@ bool simt2_pick(int d, int64_t ld, int* R, Geo2* g, size_t* bytes) {
   return false;
 }
 
-template <int K>
+template <int K, int CQ>
 cudaError_t launch_v2(const StepArgs& a, Lane at) {
   int R;
   Geo2 g;
   size_t bytes;
   if (!simt2_pick<K>(a.d, a.ld, &R, &g, &bytes)) return cudaErrorInvalidConfiguration;
-  const bool two = a.d > kThreads2;
-  if (R == 16) return two ? launch_two<K, 2, 16>(a, g, bytes, at) : launch_two<K, 1, 16>(a, g, bytes, at);
-  return two ? launch_two<K, 2, 8>(a, g, bytes, at) : launch_two<K, 1, 8>(a, g, bytes, at);
+  return R == 16 ? launch_two<K, CQ, 16>(a, g, bytes, at) : launch_two<K, CQ, 8>(a, g, bytes, at);
 }
 
 bool v2_supported(int d, int64_t ld, int K) {
@@ -565,9 +584,9 @@ bool v2_supported(int d, int64_t ld, int K) {
 cudaError_t launch_f32(const StepArgs& a, int K, Lane at) {
   if (v2_supported(a.d, a.ld, K)) {
     switch (K) {
-      case 8: return launch_v2<8>(a, at);
-      case 16: return launch_v2<16>(a, at);
-      case 32: return launch_v2<32>(a, at);
+      case 8: return a.d > kThreads2 ? launch_v2<8, 2>(a, at) : launch_v2<8, 1>(a, at);
+      case 16: return a.d > kThreads2 ? launch_v2<16, 2>(a, at) : launch_v2<16, 1>(a, at);
+      case 32: return a.d > kThreads2 ? launch_v2<32, 2>(a, at) : launch_v2<32, 1>(a, at);
     }
   }
   return cudaErrorInvalidConfiguration;
