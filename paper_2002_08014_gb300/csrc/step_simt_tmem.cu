@@ -17,13 +17,15 @@
 //            c = l + 32 t (one shared-memory word per step, consecutive across
 //            the warp) times row c of Z_i from TMEM; a shuffle reduce-scatter
 //            sums the 32 lanes, so no cross-warp reduction is needed;
-//   phase 2  Y += A_tile^T W with each thread's columns c = tid + 512 q of the
-//            d x 16 partial Y in registers for the CTA's whole segment.
+//   phase 2  Y += A_tile^T W with 4 x 4 (d <= 512) or 4 x 8 blocks of the d x 16
+//            partial Y in a thread's registers for the CTA's whole segment.  (Whole
+//            columns of Y a thread, us -> now: 112,151 x 762 211 -> 177; 60,001 x 256
+//            58.8 -> 48.0; 20,000 x 64 15.7 -> 13.3; 250,000 x 1,024 372 -> 357.)
 // For d = 1024 (the row length of the FP32 benchmark) a second kernel with
 // compile-time geometry software-pipelines the tiles: phase 2 of tile t runs
 // interleaved with phase 1 of tile t + 1 in every warp.
-// Only one CTA fits an SM (512 threads x 128 registers), so the TMEM
-// allocation never waits on another CTA.
+// The registers of one CTA (512 threads x 112 or more) leave no room for another CTA that
+// takes tensor memory, so the TMEM allocation never waits on one.
 #include "lp_internal.cuh"
 #include "tc_ptx.cuh"
 
@@ -115,8 +117,37 @@ __device__ __forceinline__ void store_row_sum(const float2 (&acc)[kK / 2], int l
   if ((lane & 1) == 0) Wrow[lane >> 1] = v[0];
 }
 
-template <int CPT>
+// Phase 2 for one row: y[i] += v_i w over four columns of A and JJ columns of W (packed FMAs).
+// Shared memory returns one FP32 a clock for each FMA lane, so a row costs a thread JJ + 4
+// words for 4 JJ FMAs (whole columns of Y: 16 words of W and one of A for 16 FMAs).
+template <int JJ>
+__device__ __forceinline__ void phase2_row(const float4& v, const float* W, float2 (&y)[4][JJ / 2]) {
+  float2 w[JJ / 2];
+#pragma unroll
+  for (int j = 0; j < JJ; j += 4) {
+    const float4 q4 = *reinterpret_cast<const float4*>(W + j);
+    w[j / 2] = make_float2(q4.x, q4.y);
+    w[j / 2 + 1] = make_float2(q4.z, q4.w);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float ai = i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
+    const float2 a2 = make_float2(ai, ai);
+#pragma unroll
+    for (int j = 0; j < JJ / 2; ++j) y[i][j] = __ffma2_rn(a2, w[j], y[i][j]);
+  }
+}
+template <int JJ>
+__device__ __forceinline__ void store_columns(float* P, const float2 (&y)[JJ / 2]) {
+#pragma unroll
+  for (int j = 0; j < JJ / 2; j += 2)
+    *reinterpret_cast<float4*>(P + 2 * j) = make_float4(y[j].x, y[j].y, y[j + 1].x, y[j + 1].y);
+}
+
+// JG = 4 (d <= 512) or 2 threads share four columns of A in phase 2, each holding JJ columns of Y.
+template <int JG>
 __global__ void __launch_bounds__(kThr, 1) step_simt_tmem_kernel(StepArgs a, GeoT g) {
+  constexpr int JJ = kK / JG;
   extern __shared__ __align__(16) float smt[];
   __shared__ uint32_t tmem_holder;
   const int T = g.T;
@@ -149,11 +180,12 @@ __global__ void __launch_bounds__(kThr, 1) step_simt_tmem_kernel(StepArgs a, Geo
   const uint32_t tmem = tmem_holder;
   const uint32_t tq = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);  // this warp's lane quarter
 
-  float2 y[CPT][kK / 2];
+  const int c4 = 4 * (tid / JG), j2 = (tid % JG) * JJ;  // phase 2
+  float2 y[4][JJ / 2];
 #pragma unroll
-  for (int q = 0; q < CPT; ++q)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < kK / 2; ++j) y[q][j] = make_float2(0.f, 0.f);
+    for (int j = 0; j < JJ / 2; ++j) y[i][j] = make_float2(0.f, 0.f);
 
   int cur_part = -1;
   const int sb = a.seg_ptr[blockIdx.x], se = a.seg_ptr[blockIdx.x + 1];
@@ -230,38 +262,16 @@ __global__ void __launch_bounds__(kThr, 1) step_simt_tmem_kernel(StepArgs a, Geo
       // ---- phase 2: Y += T^T W (packed FP32 FMAs)
 #pragma unroll 2
       for (int r = 0; r < kR; ++r) {
-        float2 w[kK / 2];
-#pragma unroll
-        for (int j = 0; j < kK; j += 4) {
-          const float4 q4 = *reinterpret_cast<const float4*>(Ws + r * kK + j);
-          w[j / 2] = make_float2(q4.x, q4.y);
-          w[j / 2 + 1] = make_float2(q4.z, q4.w);
-        }
-#pragma unroll
-        for (int q = 0; q < CPT; ++q) {
-          const int c = tid + kThr * q;
-          if (c < d) {
-            const float av = Tt[size_t(r) * lds + c];
-            const float2 a2 = make_float2(av, av);
-#pragma unroll
-            for (int j = 0; j < kK / 2; ++j) y[q][j] = __ffma2_rn(a2, w[j], y[q][j]);
-          }
-        }
+        if (c4 < d) phase2_row<JJ>(*reinterpret_cast<const float4*>(Tt + size_t(r) * lds + c4), Ws + r * kK + j2, y);
       }
       __syncthreads();
     }
-    float* Pd = a.P + size_t(sg.slot) * d * pld;
+    float* Pd = a.P + size_t(sg.slot) * d * pld + j2;
 #pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-      const int c = tid + kThr * q;
-      if (c < d) {
+    for (int i = 0; i < 4; ++i) {
+      if (c4 + i < d) store_columns<JJ>(Pd + size_t(c4 + i) * pld, y[i]);
 #pragma unroll
-        for (int j = 0; j < kK / 2; j += 2)
-          *reinterpret_cast<float4*>(Pd + size_t(c) * pld + 2 * j) =
-              make_float4(y[q][j].x, y[q][j].y, y[q][j + 1].x, y[q][j + 1].y);
-      }
-#pragma unroll
-      for (int j = 0; j < kK / 2; ++j) y[q][j] = make_float2(0.f, 0.f);
+      for (int j = 0; j < JJ / 2; ++j) y[i][j] = make_float2(0.f, 0.f);
     }
   }
   tc_sync();
@@ -291,7 +301,7 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
 
 template <bool NEXT>
 __device__ __forceinline__ void fused_rows(const float* __restrict__ Acur, const float* __restrict__ Wcur,
-                                           const float* Anext_row, uint32_t tq, int tid, float2 (&y)[2][kK / 2],
+                                           const float* Anext_row, uint32_t tq, int c4, int j2, float2 (&y)[4][4],
                                            float2 (&acc)[kK / 2]) {
 #pragma unroll 2
   for (int r = 0; r < kR; ++r) {
@@ -302,20 +312,7 @@ __device__ __forceinline__ void fused_rows(const float* __restrict__ Acur, const
       a0 = Anext_row[64 * r];
       a1 = Anext_row[64 * r + 32];
     }
-    float2 w[kK / 2];
-#pragma unroll
-    for (int j = 0; j < kK; j += 4) {
-      const float4 q4 = *reinterpret_cast<const float4*>(Wcur + r * kK + j);
-      w[j / 2] = make_float2(q4.x, q4.y);
-      w[j / 2 + 1] = make_float2(q4.z, q4.w);
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const float av = Acur[r * kD + tid + kThr * q];
-      const float2 a2 = make_float2(av, av);
-#pragma unroll
-      for (int j = 0; j < kK / 2; ++j) y[q][j] = __ffma2_rn(a2, w[j], y[q][j]);
-    }
+    phase2_row<8>(*reinterpret_cast<const float4*>(Acur + r * kD + c4), Wcur + r * kK + j2, y);
     if (NEXT) {
       tmem_wait_ld();
       fma_row(acc, a0, z0);
@@ -351,11 +348,12 @@ __global__ void __launch_bounds__(kThr, 1) step_simt_tmem_d1024_kernel(StepArgs 
   const uint32_t tq = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
 
   after_previous();
-  float2 y[2][kK / 2];
+  const int c4 = 4 * (tid >> 1), j2 = 8 * (tid & 1);  // phase 2: four columns of A, eight of Y
+  float2 y[4][4];
 #pragma unroll
-  for (int q = 0; q < 2; ++q)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < kK / 2; ++j) y[q][j] = make_float2(0.f, 0.f);
+    for (int j = 0; j < 4; ++j) y[i][j] = make_float2(0.f, 0.f);
 
   uint32_t g0 = 0;  // tiles of earlier segments: tile t of this one is the CTA's tile g0 + t
   // CTA tiles whose copy was issued / whose wait succeeded (both in tile order);
@@ -456,26 +454,22 @@ __global__ void __launch_bounds__(kThr, 1) step_simt_tmem_d1024_kernel(StepArgs 
 #pragma unroll
       for (int j = 0; j < kK / 2; ++j) acc[j] = make_float2(0.f, 0.f);
       if (next) {
-        fused_rows<true>(Acur, Wcur, bufs + ((g0 + t + 1) % 3) * kTile + warp * kD + lane, tq, tid, y, acc);
+        fused_rows<true>(Acur, Wcur, bufs + ((g0 + t + 1) % 3) * kTile + warp * kD + lane, tq, c4, j2, y, acc);
         store_row_sum(acc, lane, Wb + ((t + 1) & 1) * kR * kK + warp * kK);
       } else {
-        fused_rows<false>(Acur, Wcur, nullptr, tq, tid, y, acc);
+        fused_rows<false>(Acur, Wcur, nullptr, tq, c4, j2, y, acc);
       }
       __syncthreads();  // W(t + 1) complete; tile t's buffer and W(t) free
     }
     if (!aborted && s_abort) aborted = true;  // a wait in the segment's last tile gave up
     if (aborted) break;
     g0 += ntiles;
-    float* Pd = a.P + size_t(sg.slot) * kD * pld;
+    float* Pd = a.P + (size_t(sg.slot) * kD + c4) * pld + j2;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int c = tid + kThr * q;
+    for (int i = 0; i < 4; ++i) {
+      store_columns<8>(Pd + size_t(i) * pld, y[i]);
 #pragma unroll
-      for (int j = 0; j < kK / 2; j += 2)
-        *reinterpret_cast<float4*>(Pd + size_t(c) * pld + 2 * j) =
-            make_float4(y[q][j].x, y[q][j].y, y[q][j + 1].x, y[q][j + 1].y);
-#pragma unroll
-      for (int j = 0; j < kK / 2; ++j) y[q][j] = make_float2(0.f, 0.f);
+      for (int j = 0; j < 4; ++j) y[i][j] = make_float2(0.f, 0.f);
     }
   }
   // After a wait gave up: the copies issued but not seen to land must land
@@ -524,7 +518,7 @@ cudaError_t launch_step_simt_tmem(const StepArgs& a, Lane at) {
     if (e != cudaSuccess) return e;
     return launch_on(at, step_simt_tmem_d1024_kernel, dim3(a.grid), kThr, b3, 0, a);
   }
-  auto kern = a.d > kThr ? step_simt_tmem_kernel<2> : step_simt_tmem_kernel<1>;
+  auto kern = a.d > kThr ? step_simt_tmem_kernel<2> : step_simt_tmem_kernel<4>;
   cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void*>(kern));
   if (e != cudaSuccess) return e;
   return launch_on(at, kern, dim3(a.grid), kThr, bytes, 0, a, g);

@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d", [32, 33, 130, 511, 513, 766, 1021, 1024])
-@pytest.mark.parametrize("k", [1, 8, 17, 32])
+@pytest.mark.parametrize("k", [1, 8, 11, 16, 17, 32])
 @pytest.mark.parametrize("sizes", [[32], [47, 33], [5_003, 100, 64]])
 def test_step_against_fp64(gpu_lib, d, k, sizes):
     import torch
