@@ -201,11 +201,11 @@ def run_reference(args):
 # DRAM bytes per launch / algorithmic bytes at d = 1024, k = 16, from ncu
 # captures of the current kernels, keyed by (path, planes, cache hints, slice
 # columns, lag); other configurations report traffic as unknown.
-DRAM_RATIO = {(0, 0, 0, 0, 0): 1081.1 / 1073.7,    # SIMT FP32, Z_i in TMEM (n = 262,144)
-              (3, 2, 0, 0, 0): 2118.4 / 2048.0}    # pass-split pair tcgen05, hi/lo planes (n = 500,000)
+DRAM_RATIO = {(0, 0, 0, 0, 0): 1081.7 / 1073.7,    # SIMT FP32, Z_i in TMEM (n = 262,144)
+              (3, 2, 0, 0, 0): 2154.4 / 2048.0}    # pass-split pair tcgen05, hi/lo planes (n = 500,000)
 # the precision workload's shape (d = 2,048, k = 32), from captures at n = 131,072 scaled by rows
-DRAM_RATIO_PRECISION = {"bf16": 552.866 / 536.871,   # streaming tcgen05 (profiles/step_tcs_bf16_d2048_k32.md)
-                        "e4m3": 275.163 / 268.960}   # FP8 tcgen05, codes + scales (profiles/step_tcs8_e4m3_d2048_k32.md)
+DRAM_RATIO_PRECISION = {"bf16": 575.510 / 536.871,   # streaming tcgen05 (profiles/step_kernels_dram.md)
+                        "e4m3": 281.026 / 268.960}   # FP8 tcgen05, codes + scales (profiles/step_kernels_dram.md)
 
 
 def _traffic(path, planes, tuning, launch_bytes, d=1024, k=16):
@@ -225,7 +225,7 @@ KERNELS = {0: "step_simt2_kernel (SIMT FP32 fused A_i^T (A_i Z_i))",
 def _kernel(path, dtype="f32", d=1024, k=16):
     """Name of the step kernel a solve ran (lp_stats.path plus the shape for the SIMT path)."""
     if path == 2 and dtype == "e4m3":
-        return "step_tcs8_kernel (tcgen05 streaming, E4M3 codes widened to FP16 in shared memory, row scales factored out)"
+        return "step_tcs8_kernel (tcgen05 streaming, E4M3 codes widened to FP16 on their way to shared memory, row scales factored out)"
     if path != 0:
         return KERNELS[path]
     if dtype != "f32":
