@@ -7,10 +7,11 @@
 //   rho        residual error of Def. 3 per partition (traced solves)
 // (the orthonormalisation is in cholqr2.cu).
 // Precision, by default: the d-sized work (averaging) and the k x k Jacobi SVD /
-// eigen-solves are FP32; the Ritz matrix H and the sign-fix inner products that
-// decide D_i are accumulated in FP64.  GB300's FP64 pipe is a small fraction of
-// its FP32 pipe, and these k x k steps are serial latency on every round.  With
-// LP_FLAG_KXK_FP64 the Procrustes SVD and the Ritz eigen-solve are FP64 too.
+// eigen-solves are FP32; the Ritz matrix H is accumulated in FP64, and the sign-fix
+// inner products that decide D_i are wherever an FP32 sum's error bound leaves the
+// sign open.  GB300's FP64 pipe is a small fraction of its FP32 pipe, and these k x k
+// steps are serial latency on every round.  With LP_FLAG_KXK_FP64 the Procrustes SVD
+// and the Ritz eigen-solve are FP64 too.
 #include <algorithm>
 #include <cfloat>
 #include <mutex>
@@ -390,8 +391,10 @@ __global__ void __launch_bounds__(kT) align_kernel(const float* __restrict__ Zl,
     // entry at 2 per clock), so an FP32 sum decides where it can: with D the sum of
     // the products' magnitudes, any order of n FP32 multiply-adds is within n u D / (1 -
     // n u) of the exact sum, u = 2^-24 (Higham, Accuracy and Stability of Numerical
-    // Algorithms, Sec. 3.1), and the FP64 sum within far less.  A column whose FP32
-    // sum is not above twice that bound (or is NaN) sends the block to the FP64 sums.
+    // Algorithms, Sec. 3.1), plus 2^-150 for each that falls below the normal range
+    // (Sec. 2.1), and the FP64 sum within far less.  The computed D lacks up to as much
+    // of that again (n u <= 1).  A column whose FP32 sum is not above twice the first
+    // term plus 2^-149 for each row (or is NaN) sends the block to the FP64 sums.
     // Measured, 64 blocks of 1,024 x 16: 16.3 -> 5.6 us; 4 of 100 x 5: 3.6 -> 2.2.
     const int j = t % K, sl = t / K, RS = kT / K;
     float* dots = reinterpret_cast<float*>(part);
@@ -413,7 +416,8 @@ __global__ void __launch_bounds__(kT) align_kernel(const float* __restrict__ Zl,
         mag += dots[kT + q * K + t];
       }
       // columns beyond k hold zeros: nothing to decide
-      sure = t >= k || fabsf(tot) > 2.f * (static_cast<float>(d) + RS + 2) * 0x1.0p-24f * mag;
+      const float terms = static_cast<float>(d) + RS + 2;
+      sure = t >= k || fabsf(tot) > 2.f * terms * 0x1.0p-24f * mag + terms * 0x1.0p-149f;
       part[kT + t] = tot;  // beyond the sums of either precision
     }
     if (__syncthreads_or(!sure)) {
