@@ -71,7 +71,7 @@ struct lp_ctx {
   int* dSegPtrTcs = nullptr;
   int* dSlotBeginTcs = nullptr;
   const lp::TcsPlan* tcs_cur = nullptr;
-  int peers = 1;  // launch sequences that a batch's graph runs side by side with this one
+  int peers = 1;  // launch sequences on the device at once (a batch's groups, a server's requests), this one included
 
   int path = 0;  // step kernel of the current solve / step (lp_stats::path)
   lp::TcsTuning tuning;

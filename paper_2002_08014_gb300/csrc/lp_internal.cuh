@@ -210,11 +210,13 @@ size_t estimate_bytes(int sms, int m, const int64_t* rows, int64_t d, int64_t pi
                       lp_ptr_space space);
 // 1: the last lp_solve finished on the device; 0: still running; -1: no solve or a CUDA error.
 int solve_state(lp_ctx* c);
+// Launch sequences that run side by side on the device in the solves that follow, this
+// context's included (1: its steps take the whole chip).
+void set_peers(lp_ctx* c, int peers);
 // A solve split for capture into one graph over many contexts: checks, kernel
 // choice and y0 upload (outside the capture); the launch sequence on the
 // context's stream (inside it; *captured receives its counters); and marking
 // the context solved after the graph ran.
-void set_peers(lp_ctx* c, int peers);
 lp_status batch_prepare(lp_ctx* c, int k, const int* p_schedule, int T, lp_aggregator agg, const double* y0,
                         int refine_rounds, unsigned flags);
 lp_status batch_enqueue(lp_ctx* c, int k, const int* p_schedule, int T, lp_aggregator agg, int refine_rounds,

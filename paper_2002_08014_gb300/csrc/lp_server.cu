@@ -99,6 +99,21 @@ bool enqueue_directly(const Request* r) {
   return 4 * steps <= 1000;
 }
 
+// Solves that will run side by side once the queue's head is admitted as far as the active
+// limit and the budget let it, the one being admitted (its bytes are in in_use) included.
+// Requests that have to wait leave the chip to the running ones: with max_active = 1 and
+// four waiting, 9,728 x 1,024 steps that made room for them took 32 us against 21 alone.
+int side_by_side(const lp_server* s) {
+  int n = static_cast<int>(s->active.size()) + 1;
+  size_t used = s->in_use;
+  for (const Request* q : s->queue) {
+    if (n >= s->max_active || (s->budget && used + q->est > s->budget)) break;
+    used += q->est;
+    ++n;
+  }
+  return n;
+}
+
 // Copies the partitions in and enqueues the solve; failures complete the request.
 void admit(lp_server* s, Request* r) {
   lp_ctx* c = nullptr;
@@ -112,7 +127,7 @@ void admit(lp_server* s, Request* r) {
   s->peak = std::max(s->peak, s->in_use);
   st = lp::load_pitched(c, r->m, r->rows.data(), r->d, r->pitch, r->dtype, r->parts.data(),
                         r->dtype == LP_FP8_E4M3 ? r->scales.data() : nullptr, r->space);
-  if (!st) lp::set_peers(c, static_cast<int>(s->active.size() + s->queue.size()) + 1);
+  if (!st) lp::set_peers(c, side_by_side(s));
   if (!st)
     st = lp_solve(c, r->k, r->sched.empty() ? nullptr : r->sched.data(), r->T, r->agg, r->y0.data(), r->refine,
                   r->flags | (enqueue_directly(r) ? LP_FLAG_NO_GRAPH : 0u));
