@@ -185,7 +185,9 @@ lp_status lp_result(lp_ctx* ctx, double* z_out, double* sigma_out, lp_stats* sta
 typedef struct lp_tuning {
     int32_t ring_units;      /* 32 KB shared-memory ring units (default: as many as fit, <= 8) */
     int32_t lag_units;       /* first-pass units of tile t+1 issued before the second pass of
-                              * tile t starts (default 2 without a cluster, 4 with one)         */
+                              * tile t starts (default 2 without a cluster, 3 with one; for FP8
+                              * data, whose second pass runs one tile behind the first or, over
+                              * a cluster, two: 1)                                               */
     int32_t prefetch_units;  /* first-pass units brought into L2 ahead of their load (default 0) */
     int32_t cache_hints;     /* 1: first-pass loads mark lines evict_last, second-pass loads
                               * evict_first (default 0: no hint)                                  */
@@ -225,11 +227,13 @@ lp_status lp_set_tuning(lp_ctx* ctx, const lp_tuning* tuning);
  * lp_autotune: time the step-kernel candidates for rank k on the loaded
  * partitions and keep the fastest for later solves on this context (it sets
  * the context's tuning, and for LP_BF16 data whether the resident or the
- * streaming tensor-core kernel runs).  Candidates: the streaming kernel with
- * lag in {1, 2, 4}, cache hints off/on and the default or 512-column slices,
- * and the resident kernel where it has a plan.  Each is timed over 3 launches after a warm-up launch, on the
- * context's stream; the call synchronises.  Other dtypes have one candidate
- * (the SIMT kernel) and return at once.
+ * streaming tensor-core kernel runs).  Candidates for BF16 and split-plane data:
+ * the pair kernel, the streaming kernel with lag in {1, 2, 3}, cache hints off/on
+ * and the default or 512-column slices, and the resident kernel, each where it
+ * has a plan; for FP8 data lag in {1, 2} and the default or 256-column slices.
+ * Each is timed over 3 launches after a warm-up launch, on the context's stream;
+ * the call synchronises.  FP32 data have one candidate (the SIMT kernel) and
+ * return at once.
  *   chosen      receives the winning tuning (may be NULL).
  *   path        receives the winning lp_stats::path code (may be NULL).
  *   best_ms     receives the winner's mean launch time in ms (may be NULL).

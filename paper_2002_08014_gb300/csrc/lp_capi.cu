@@ -1112,7 +1112,7 @@ lp_status lp_autotune(lp_ctx* c, int k, lp_tuning* chosen, int* path_out, double
   std::vector<Cand> cands;
   if (c->dtype == LP_FP8_E4M3) {
     for (int slice : {0, 256})
-      for (int lag : {2, 4}) {
+      for (int lag : lp::kTcs8Lags) {
         Cand cd;
         cd.t.kernel = LP_KERNEL_STREAM;
         cd.t.lag_units = lag;
@@ -1129,7 +1129,7 @@ lp_status lp_autotune(lp_ctx* c, int k, lp_tuning* chosen, int* path_out, double
       cands.push_back(cd);
     }
     for (int slice : {0, 512})
-      for (int lag : {1, 2, 4})
+      for (int lag : lp::kTcsLags)
         for (int hint : {0, 1}) {
           Cand cd;
           cd.t.kernel = LP_KERNEL_STREAM;

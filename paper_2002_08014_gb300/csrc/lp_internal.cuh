@@ -166,6 +166,24 @@ struct TcsTuning {
   int kernel = 0;  // LP_KERNEL_* of lp_tuning
   long long test_stall_cycles = 0;  // lp_tuning::test_stall_cycles
 };
+// Lag (lp_tuning::lag_units) of a plan that sets none, and the lags that lp_autotune tries
+// (the default among them, or tuning could only lose against leaving it alone).
+// Streaming kernel: over a cluster W takes the exchange between CTAs (1,000,000 x 2,048,
+// k = 32, lag 1, 2, 3, 4: 1,130, 1,010, 993, 1,014 us); lag 4 was nowhere better than 3.
+constexpr int tcs_default_lag(int cluster) { return cluster > 1 ? 3 : 2; }
+constexpr int kTcsLags[] = {1, 2, 3};
+// FP8: one block apart, the two converter groups and issuers alternate.
+constexpr int tcs8_default_lag(int) { return 1; }
+constexpr int kTcs8Lags[] = {1, 2};
+template <size_t N>
+constexpr bool lag_tried(const int (&lags)[N], int lag) {
+  for (int x : lags)
+    if (x == lag) return true;
+  return false;
+}
+static_assert(lag_tried(kTcsLags, tcs_default_lag(1)) && lag_tried(kTcsLags, tcs_default_lag(2)) &&
+                  lag_tried(kTcs8Lags, tcs8_default_lag(1)) && lag_tried(kTcs8Lags, tcs8_default_lag(2)),
+              "the default lags are among the autotuner's");
 // Fills the geometry for (d, k, planes).  False when the shape has no streaming kernel.
 bool tcs_plan(int d, int k, int planes, int sms, const TcsTuning& tune, TcsPlan* p);
 // Encodes the tensor maps of the planes (plane1 may be NULL for one plane).

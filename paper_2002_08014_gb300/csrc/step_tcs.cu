@@ -592,9 +592,7 @@ bool tcs_plan(int d, int k, int planes, int sms, const TcsTuning& tune, TcsPlan*
   p->cluster = cl;
   p->ring = ring;
   const int U = (ncd / 2) * planes;
-  // (over a cluster W takes the exchange between CTAs: 1,000,000 x 2,048, k = 32, four units a
-  // tile: lag 2, 3, 4: 1,011, 993, 1,013 us)
-  if (lag <= 0) lag = cl > 1 ? 3 : 2;
+  if (lag <= 0) lag = tcs_default_lag(cl);
   p->lag = lag < U ? lag : U;
   p->prefetch = tune.prefetch_units > 0 ? tune.prefetch_units : 0;
   p->hints = tune.cache_hints ? 1 : 0;

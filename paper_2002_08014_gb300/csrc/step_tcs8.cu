@@ -694,9 +694,7 @@ bool tcs8_plan_slice(int d, int k, int sms, const TcsTuning& tune, int ncd_max, 
   p->ncd = ncd;
   p->cluster = cl;
   p->ring = ring;
-  // one block apart, the two converter groups and issuers alternate (lag 4, 2, 1 at d =
-  // 2,048, k = 32: 406, 395, 389 us with n = 262,144)
-  int lag = tune.lag_units > 0 ? tune.lag_units : 1;
+  const int lag = tune.lag_units > 0 ? tune.lag_units : tcs8_default_lag(cl);
   const int U = ncd / 2;
   p->lag = lag < U ? lag : U;
   p->prefetch = 0;
