@@ -186,8 +186,8 @@ typedef struct lp_tuning {
     int32_t ring_units;      /* 32 KB shared-memory ring units (default: as many as fit, <= 8) */
     int32_t lag_units;       /* first-pass units of tile t+1 issued before the second pass of
                               * tile t starts (default 2 without a cluster, 3 with one; for FP8
-                              * data, whose second pass runs one tile behind the first or, over
-                              * a cluster, two: 1)                                               */
+                              * data, whose second pass runs a tile behind the first or, over a
+                              * cluster, two: 1 without a cluster, 2 with one)                   */
     int32_t prefetch_units;  /* first-pass units brought into L2 ahead of their load (default 0) */
     int32_t cache_hints;     /* 1: first-pass loads mark lines evict_last, second-pass loads
                               * evict_first (default 0: no hint)                                  */

@@ -172,8 +172,12 @@ struct TcsTuning {
 // k = 32, lag 1, 2, 3, 4: 1,130, 1,010, 993, 1,014 us); lag 4 was nowhere better than 3.
 constexpr int tcs_default_lag(int cluster) { return cluster > 1 ? 3 : 2; }
 constexpr int kTcsLags[] = {1, 2, 3};
-// FP8: one block apart, the two converter groups and issuers alternate.
-constexpr int tcs8_default_lag(int) { return 1; }
+// FP8: one block apart, the two converter groups and issuers alternate; over a cluster a
+// block more takes up the exchange.  us at lag 1, 2, 3, 4: 1,000,000 x 2,048, k = 32 1,238,
+// 1,211, 1,237, 1,238; 262,144 x 1,024, k = 32 173.6, 170.6, 174.4, 174.4; without a cluster,
+// at lag 1, 2: 400,000 x 362, k = 8 77.6, 81.4; 500,000 x 512, k = 8 122.4, 122.9; but
+// 262,144 x 1,024, k = 16 165.9, 164.1.
+constexpr int tcs8_default_lag(int cluster) { return cluster > 1 ? 2 : 1; }
 constexpr int kTcs8Lags[] = {1, 2};
 template <size_t N>
 constexpr bool lag_tried(const int (&lags)[N], int lag) {

@@ -32,8 +32,8 @@
 // units in closed form; the second pass runs two tiles behind the first where tensor
 // memory holds a third D1, which takes the cluster exchange of W off the chain; and the
 // exchange itself adds four columns at a time and waits for its copies only before it
-// rewrites their source (12,000 -> 9,000 cycles a tile).  1,190 us at n = 1M, 1.7 TB/s of
-// codes; n = 262,144: 456 -> 334 us over these steps, 123 -> 94 at d = 512 without a
+// rewrites their source (12,000 -> 9,000 cycles a tile).  1,211 us at n = 1M, 1.7 TB/s of
+// codes; n = 262,144: 456 -> 332 us over these steps, 123 -> 94 at d = 512 without a
 // cluster.  A group still takes about 2,500 cycles a unit (widening 640, issuing its
 // loads up to 600, the fence 90, the rest waiting for slots and data), three times what
 // the conversion pipe needs.
