@@ -1,7 +1,8 @@
-"""lp_orth under LP_FLAG_KXK_FP64 where many blocks take one CTA each: the sums keep
-their order, so every block has the bits that it has in a small batch, where a cluster
-takes it (rows around whole rounds of the 85 or 25 slices and the rows widened at a
-time, limits of the choice in blocks and rows, rows that fill shared memory).
+"""lp_orth where many blocks take one CTA each (FP64 k x k work, and FP32 at k <= 8) or
+larger clusters than few blocks would: the sums keep their order, so every block has the
+bits that it has in a small batch (rows around whole rounds of the 85 or 25 FP64 slices
+and the rows widened at a time, limits of the choice in blocks and rows, rows that fill
+shared memory).
 
 Tolerances against the FP64 factorisation as for the clusters, k 2^-20, on blocks with
 four times as many rows as columns (square Gaussian blocks are not well-conditioned)."""
@@ -22,6 +23,17 @@ TOL = 32 * 2.0 ** -20
     (16, 16, 183), (9, 24, 200), (16, 25, 190), (12, 26, 183), (13, 126, 183), (16, 384, 183), (10, 448, 251),
     (16, 768, 151), (11, 1_000, 152), (16, 2_250, 129), (16, 2_400, 151)])
 def test_many_fp64_blocks_have_the_bits_of_few(gpu_lib, k, d, batch):
+    _many_and_few(k, d, batch, True)
+
+
+@pytest.mark.parametrize("k,d,batch", [
+    (8, 8, 600), (5, 1_024, 153), (5, 1_025, 77), (3, 3_072, 153), (8, 3_073, 153), (8, 5_120, 77), (5, 5_121, 100),
+    (16, 2_500, 153), (12, 4_200, 100), (32, 1_500, 153), (20, 2_300, 80)])
+def test_many_fp32_blocks_have_the_bits_of_few(gpu_lib, k, d, batch):
+    _many_and_few(k, d, batch, False)
+
+
+def _many_and_few(k, d, batch, fp64):
     import torch
     g = torch.Generator(device="cuda").manual_seed(d + k)
     mix = torch.eye(k, dtype=torch.float64, device="cuda") + 0.1 / k
@@ -29,8 +41,8 @@ def test_many_fp64_blocks_have_the_bits_of_few(gpu_lib, k, d, batch):
     torch.cuda.synchronize()
     ctx = B.lp_create(0)
     try:
-        Z = B.lp_orth(ctx, Y, kxk_fp64=True)
-        few = torch.cat([B.lp_orth(ctx, y.contiguous(), kxk_fp64=True) for y in Y.split(50)])
+        Z = B.lp_orth(ctx, Y, kxk_fp64=fp64)
+        few = torch.cat([B.lp_orth(ctx, y.contiguous(), kxk_fp64=fp64) for y in Y.split(20)])
     finally:
         B.lp_destroy(ctx)
     assert torch.equal(Z, few)
