@@ -210,7 +210,7 @@ typedef struct lp_tuning {
  * PAIR:   the two passes run on the two CTAs of a cluster: rank 0 reads the
  *         tile from HBM and forms W = A_t Z, copies W into rank 1's shared
  *         memory, and rank 1 re-reads the tile from L2 and accumulates A_t^T W
- *         (d <= 1024 for k <= 16, d <= 512 for k > 16).  Same products, same
+ *         (d <= 4096 for k <= 8, 2048 for k <= 16, 1024 for k > 16).  Same products, same
  *         summation order within a tile.
  * DEFAULT picks the pass-split pair kernel where it has a plan, else STREAM. */
 enum { LP_KERNEL_DEFAULT = 0, LP_KERNEL_STREAM = 1, LP_KERNEL_PAIR = 2 };

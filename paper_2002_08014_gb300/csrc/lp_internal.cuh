@@ -161,7 +161,7 @@ struct TcsPlan {
   // FP8-E4M3 streaming kernel (step_tcs8.cu): codes read to registers, widened to FP16
   int fp8 = 0;         // 1: this plan is for step_tcs8_kernel
   int behind = 1;      // its second pass runs this many tiles behind the first
-  int issuers = 1;     // streaming kernels: MMA-issuing threads (own partial D1 and ring slots each)
+  int issuers = 1;     // streaming kernel: MMA-issuing threads (own partial D1 each)
   int map3d = 0;       // the maps are (64 columns, row, chunk), one box per unit
   alignas(64) unsigned char tmap[2][128];  // CUtensorMaps of the planes
 };
@@ -203,8 +203,8 @@ cudaError_t tcs_encode_maps(const void* plane0, const void* plane1, int64_t n, i
 cudaError_t launch_step_tcs(const TcsPlan& p, const Segment* segs, const int* seg_ptr, const float* Z,
                             int64_t z_stride, float* P, int d, int* status, Lane at);
 // Pass-split pair kernel: the same product with the HBM pass and the L2 pass on
-// the two CTAs of a cluster.  False when the shape has no plan (d > 1024 at
-// k > 16, d > 2048, or a ring under two units).
+// the two CTAs of a cluster.  False when the shape has no plan (d > 4096 at k <= 8,
+// d > 2048 at k <= 16, d > 1024 beyond, or a ring under two units).
 bool pair_plan(int d, int k, int planes, int sms, const TcsTuning& tune, TcsPlan* p);
 // FP8-E4M3 codes with FP32 row scales on the tensor cores (streaming form; the
 // codes are widened to FP16 in shared memory).  False when the shape has no plan.

@@ -91,8 +91,9 @@ void release(lp_server* s, Request* r) {
 // A request is solved once, so a graph of it is captured and instantiated for one launch:
 // 1.2 ms of host time for some 500 kernels against 0.8 ms launched one by one, which the GPU
 // also begins at once.  (8 requests: admitted in 11.8 -> 9.3 ms, done in 28.4 -> 25.4.)  A
-// stream takes about a thousand launches before the host has to wait; longer solves, at up
-// to four launches a local step, stay one graph launch.
+// stream takes about a thousand launches before the host has to wait; longer solves, counted
+// as four launches a local step (three and a round's two or so more, five where every round
+// is one step), stay one graph launch.
 bool enqueue_directly(const Request* r) {
   int64_t steps = r->refine;
   for (int p : r->sched) steps += p;

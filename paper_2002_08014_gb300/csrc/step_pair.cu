@@ -59,7 +59,10 @@ using namespace tc;
 constexpr int kUnitBytes = 2 * kChunkBytes;  // 128 rows x 128 columns of one BF16 plane
 constexpr int kPairThreads = 384;
 constexpr int kIssuers = 4;    // MMA-issuing threads: lane 0 of warps 1 .. kIssuers
-constexpr int kIssuers1 = 3;   // rank 1 uses at most three (its ring of six units splits 3 x 2)
+// rank 1 uses at most three: a second and a third issuer pay (150,001 x 362, k = 8 on 2, 3, 4:
+// 31.3, 28.2, 28.2 us; 131,072 x 362 planes 50.1, 47.8, 47.8), a fourth does not (60,000 x 512
+// planes, k = 32 43.9, 44.1, 44.4)
+constexpr int kIssuers1 = 3;
 constexpr int kRecycler = 5;   // rank 1: warp of the W-buffer recycler
 constexpr int kCopier = 5;     // rank 0: warp of the thread that copies W to rank 1
 constexpr int kProducer1 = 6;  // TMA-issuing threads beside warp 0's: lane 0 of this warp and on

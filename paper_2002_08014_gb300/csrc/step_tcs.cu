@@ -604,8 +604,7 @@ bool tcs_plan(int d, int k, int planes, int sms, const TcsTuning& tune, TcsPlan*
   p->smem = p->off_bar + (S_RING0 + 2 * ring) * 8 + 16 + 1024;
   // two issuers (two partial D1 per buffer) when tensor memory holds them
   const int NBp = ncd / 2;
-  // (independent of the ring depth, which must only reorder loads: any ring of two
-  // or more units deals each issuer at least one slot)
+  // (independent of the ring depth, which must only reorder loads)
   p->issuers = (4 * N + NBp * N <= 512 && NBp >= 2) ? 2 : 1;
   const uint32_t used = static_cast<uint32_t>(2 * p->issuers * N + NBp * N);
   uint32_t cols = 32;
