@@ -497,75 +497,11 @@ __global__ void __launch_bounds__(kThreads8, 1) step_tcs8_kernel(Tcs8Args a) {
 #pragma unroll
             for (int j = 0; j < K; ++j) w[j] = 0.f;
           }
-          if (CL > 1) {
-            const uint32_t rows_bytes = static_cast<uint32_t>(RPC * K * 4);
-            if (r == 0) bulk_wait_read0();  // the previous tile's copies have read sW
-            if (!(ok = epi_sync())) break;
-#pragma unroll
-            for (int j = 0; j < K; j += 4)
-              *reinterpret_cast<float4*>(sW + wpos<K>(r, j)) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
-            fence_async_smem();
-            if (!(ok = epi_sync())) break;
-            if (r == 0) {
-              mbar_expect_tx(&bar[S_REDFULL], (CL - 1) * rows_bytes);
-              for (uint32_t o = 0; o < CL; ++o)
-                if (o != crank)
-                  bulk_s2s_cluster(mapa(su32(sWrecv + crank * RPC * K), o), su32(sW + o * RPC * K), rows_bytes,
-                                   mapa(su32(&bar[S_REDFULL]), o));
-              bulk_commit();
-            }
-            if (!(ok = wait(S_REDFULL, Tg & 1, true))) break;
-            const int per = RPC * K / kBM;  // values per epilogue thread (K / CL), neighbours in a row
-            // partials in source-rank order; four columns at a time where a thread has them
-            if (per % 4 == 0) {
-              for (int e = 0; e < per; e += 4) {
-                const int idx = r * per + e, rl = idx / K, col = idx % K;
-                const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
-                const int rel = own - static_cast<int>(crank) * RPC * K;  // offset inside one owner's row block
-                float4 v[8], sum = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (uint32_t src = 0; src < 8; ++src)
-                  if (src < CL) v[src] = *reinterpret_cast<const float4*>(src == crank ? sW + own : sWrecv + src * RPC * K + rel);
-#pragma unroll
-                for (uint32_t src = 0; src < 8; ++src)
-                  if (src < CL) {
-                    sum.x += v[src].x;
-                    sum.y += v[src].y;
-                    sum.z += v[src].z;
-                    sum.w += v[src].w;
-                  }
-                *reinterpret_cast<float4*>(sW + own) = sum;
-              }
-            } else {
-              for (int e = 0; e < per; ++e) {
-                const int idx = r * per + e, rl = idx / K, col = idx % K;
-                const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
-                const int rel = own - static_cast<int>(crank) * RPC * K;
-                float sum = 0.f;
-                for (uint32_t src = 0; src < CL; ++src) sum += src == crank ? sW[own] : sWrecv[src * RPC * K + rel];
-                sW[own] = sum;
-              }
-            }
-            fence_async_smem();
-            if (!(ok = epi_sync())) break;
-            if (r == 0) {
-              mbar_expect_tx(&bar[S_WFULL], (CL - 1) * rows_bytes);
-              for (uint32_t dst = 0; dst < CL; ++dst)
-                if (dst != crank)
-                  bulk_s2s_cluster(mapa(su32(sW + crank * RPC * K), dst), su32(sW + crank * RPC * K), rows_bytes,
-                                   mapa(su32(&bar[S_WFULL]), dst));
-              bulk_commit();
-            }
-            if (!(ok = wait(S_WFULL, Tg & 1, true))) break;
-#pragma unroll
-            for (int j = 0; j < K; j += 4) {
-              const float4 v = *reinterpret_cast<const float4*>(sW + wpos<K>(r, j));
-              w[j] = v.x;
-              w[j + 1] = v.y;
-              w[j + 2] = v.z;
-              w[j + 3] = v.w;
-            }
-          }
+          if (CL > 1 &&
+              !(ok = sum_over_cluster<K>(
+                    w, r, crank, CL, RPC, sW, sWrecv, &bar[S_REDFULL], &bar[S_WFULL], [&] { return wait(S_REDFULL, Tg & 1, true); },
+                    [&] { return wait(S_WFULL, Tg & 1, true); }, epi_sync)))
+            break;
           // row scale: W_r <- W_r s_r^2 / S (so the FP16 operand cannot overflow)
           const float f = sc * sc / a.smax2;
 #pragma unroll

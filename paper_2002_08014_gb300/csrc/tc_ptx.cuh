@@ -285,5 +285,85 @@ __device__ __forceinline__ bool bar_or(int id, int n, bool flag) {
   return r != 0;
 }
 
+// Cluster sum of W (128 x K FP32, row r of this CTA's partial in w of epilogue thread r).
+// Owner o holds rows [o RPC, (o + 1) RPC), RPC = 128 / CL.  Every CTA writes its partial rows to sW and one
+// thread ships each owner its rows (bulk copies counted in bytes on the owner's parts_full);
+// owners add the partials in source-rank order, in place, and ship the sums back the same
+// way (sums_full).  A buffer is rewritten only after the waits show its previous contents
+// were consumed.  The waits return false when they gave up, and so does this.
+template <int K, typename WaitParts, typename WaitSums, typename Sync>
+__device__ __forceinline__ bool sum_over_cluster(float (&w)[K], int r, uint32_t crank, uint32_t CL, int RPC, float* sW,
+                                                 float* sWrecv, uint64_t* parts_full, uint64_t* sums_full,
+                                                 WaitParts&& wait_parts, WaitSums&& wait_sums, Sync&& epi_sync) {
+  const uint32_t rows_bytes = static_cast<uint32_t>(RPC * K * 4);
+  if (r == 0) bulk_wait_read0();  // the previous tile's copies have read sW
+  if (!epi_sync()) return false;
+#pragma unroll
+  for (int j = 0; j < K; j += 4)
+    *reinterpret_cast<float4*>(sW + wpos<K>(r, j)) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
+  fence_async_smem();
+  if (!epi_sync()) return false;
+  if (r == 0) {
+    mbar_expect_tx(parts_full, (CL - 1) * rows_bytes);
+    for (uint32_t o = 0; o < CL; ++o)
+      if (o != crank)
+        bulk_s2s_cluster(mapa(su32(sWrecv + crank * RPC * K), o), su32(sW + o * RPC * K), rows_bytes,
+                         mapa(su32(parts_full), o));
+    bulk_commit();
+  }
+  if (!wait_parts()) return false;
+  const int per = RPC * K / kBM;  // values per epilogue thread (K / CL), neighbours in a row
+  // partials in source-rank order; four columns at a time where a thread has them
+  if (per % 4 == 0) {
+    for (int e = 0; e < per; e += 4) {
+      const int idx = r * per + e, rl = idx / K, col = idx % K;
+      const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
+      const int rel = own - static_cast<int>(crank) * RPC * K;  // offset inside one owner's row block
+      float4 v[8], sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (uint32_t src = 0; src < 8; ++src)
+        if (src < CL) v[src] = *reinterpret_cast<const float4*>(src == crank ? sW + own : sWrecv + src * RPC * K + rel);
+#pragma unroll
+      for (uint32_t src = 0; src < 8; ++src)
+        if (src < CL) {
+          sum.x += v[src].x;
+          sum.y += v[src].y;
+          sum.z += v[src].z;
+          sum.w += v[src].w;
+        }
+      *reinterpret_cast<float4*>(sW + own) = sum;
+    }
+  } else {
+    for (int e = 0; e < per; ++e) {
+      const int idx = r * per + e, rl = idx / K, col = idx % K;
+      const int own = wpos<K>(static_cast<int>(crank) * RPC + rl, col);
+      const int rel = own - static_cast<int>(crank) * RPC * K;
+      float sum = 0.f;
+      for (uint32_t src = 0; src < CL; ++src) sum += src == crank ? sW[own] : sWrecv[src * RPC * K + rel];
+      sW[own] = sum;
+    }
+  }
+  fence_async_smem();
+  if (!epi_sync()) return false;
+  if (r == 0) {
+    mbar_expect_tx(sums_full, (CL - 1) * rows_bytes);
+    for (uint32_t dst = 0; dst < CL; ++dst)
+      if (dst != crank)
+        bulk_s2s_cluster(mapa(su32(sW + crank * RPC * K), dst), su32(sW + crank * RPC * K), rows_bytes,
+                         mapa(su32(sums_full), dst));
+    bulk_commit();
+  }
+  if (!wait_sums()) return false;
+#pragma unroll
+  for (int j = 0; j < K; j += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(sW + wpos<K>(r, j));
+    w[j] = v.x;
+    w[j + 1] = v.y;
+    w[j + 2] = v.z;
+    w[j + 3] = v.w;
+  }
+  return true;
+}
+
 }  // namespace tc
 }  // namespace lp
