@@ -21,14 +21,15 @@ TOL = 32 * 2.0 ** -20
     (8, 8, 81), (1, 33, 183), (5, 84, 300), (8, 85, 153), (7, 86, 101), (5, 255, 92), (8, 257, 200), (3, 384, 92),
     (5, 385, 122), (8, 512, 152), (5, 1_408, 201), (5, 1_025, 149), (8, 2_600, 122), (6, 3_800, 152), (6, 4_200, 152),
     (16, 16, 183), (9, 24, 200), (16, 25, 190), (12, 26, 183), (13, 126, 183), (16, 384, 183), (10, 448, 251),
-    (16, 768, 151), (11, 1_000, 152), (16, 2_250, 129), (16, 2_400, 151)])
+    (16, 768, 151), (11, 1_000, 152), (16, 2_250, 129), (16, 2_400, 151),
+    (32, 4_300, 24), (20, 4_000, 24), (16, 6_000, 40), (7, 12_000, 40)])
 def test_many_fp64_blocks_have_the_bits_of_few(gpu_lib, k, d, batch):
     _many_and_few(k, d, batch, True)
 
 
 @pytest.mark.parametrize("k,d,batch", [
     (8, 8, 600), (5, 1_024, 153), (5, 1_025, 77), (3, 3_072, 153), (8, 3_073, 153), (8, 5_120, 77), (5, 5_121, 100),
-    (16, 2_500, 153), (12, 4_200, 100), (32, 1_500, 153), (20, 2_300, 80)])
+    (5, 4_272, 250), (5, 4_000, 170), (16, 2_500, 153), (12, 4_200, 100), (32, 1_500, 153), (20, 2_300, 80)])
 def test_many_fp32_blocks_have_the_bits_of_few(gpu_lib, k, d, batch):
     _many_and_few(k, d, batch, False)
 
