@@ -25,8 +25,8 @@ enum StatusBits : int {
 // segment tables).  The long ones (tensor-core steps, CholQR2, sign align) let the next one
 // begin (before_next) shortly before they end, not earlier: a waiting CTA holds its SM
 // against other streams' kernels.  Reduce, aggregate and broadcast, a few microseconds of
-// many small CTAs, let it begin at once; the SIMT steps and the Procrustes align when their
-// CTAs are gone.  All of them shortly before their end instead: the 4,000 x 100 solve 1,423
+// many small CTAs, let it begin at once; the SIMT steps and the Procrustes align, which also
+// waits for the kernel before it to end, when their CTAs are gone.  All of them shortly before their end instead: the 4,000 x 100 solve 1,423
 // -> 1,440 us, a batch of 24 9,720 -> 9,774, serving 23.3 -> 23.4 ms, but 60,007 x 362 with
 // Procrustes 3,539 -> 3,479 and a reload with 14 plane steps 2,220 -> 2,189.
 struct Lane {
